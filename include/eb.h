@@ -280,7 +280,7 @@ typedef struct {
  * |a_ij| >= theta sqrt(a_ii a_jj); distance-2 maximal independent set with
  * priorities (lowbias32 hash of the index, index); aggregates grown from its
  * nodes; P = (I - 4/(3 rho) D^-1 A) P_hat; Galerkin A_c = P^T A P; on the
- * coarsest level an explicit dense inverse formed by Gauss-Jordan elimination
+ * coarsest level an explicit dense inverse formed by symmetric block sweeps
  * without pivoting (the coarsest matrix is SPD), applied as a dense
  * matrix-vector product.  opts may be NULL for the defaults.
  * Synchronous. */
