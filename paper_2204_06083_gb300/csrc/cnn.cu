@@ -13,16 +13,14 @@
 // (130 pixels x 32 channels) and the 9 x 32 x 32 weights sit in shared memory;
 // K = 9 taps x 32 channels.  Data gradients run through
 // the same kernel with flipped, transposed weights and the ReLU mask of the
-// layer input applied in its epilogue; weight gradients are GEMMs over pixels
-// (mma.sync fragments) with per-CTA partials summed in a fixed order.  The
+// layer input applied in its epilogue; weight gradients are tcgen05 GEMMs over
+// pixels (k_conv32_wgrad) with per-CTA partials summed in a fixed order.  The
 // 2 -> 32 and 32 -> 1 layers run on the CUDA cores.  Inference (nn_forward,
 // the stage in the PCG) runs all six layers in one launch instead
 // (k_net_fwd), with the hidden activations kept in shared memory and tensor
 // memory and results identical to the layer-by-layer launches.
 #include "eb_solver.cuh"
 #include "tma.cuh"
-
-#include <mma.h>
 
 #include <algorithm>
 #include <cmath>
@@ -32,12 +30,10 @@
 namespace ebk {
 
 using bf16 = __nv_bfloat16;
-namespace wm = nvcuda::wmma;
 
 constexpr int NC = 32;    // hidden channels
 constexpr int NMID = 4;   // 32 -> 32 layers
 constexpr int TPX = 128;  // pixels per CTA job (one row segment)
-constexpr int LDA = 48;   // weight-gradient staging: pixel stride in bf16 (96 bytes: 32-byte aligned rows)
 
 // flat parameter vector
 constexpr int W1_N = NC * 9 * 2, B1_N = NC;
@@ -125,20 +121,6 @@ __global__ void __launch_bounds__(128) k_l1_fwd(Image im, const float2* __restri
   if (x + 1 < im.W) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) dst[4 + q] = make_int4(o1[4 * q], o1[4 * q + 1], o1[4 * q + 2], o1[4 * q + 3]);
-  }
-}
-
-// Stages the rows r-1, r, r+1 (pixels x0-1 .. x0+TPX) of x into sIn [3][TPX+2][LDA],
-// zero outside the image.
-__device__ __forceinline__ void stage_rows(const Image& im, const bf16* __restrict__ x, int r, int x0, bf16* sIn) {
-  const int lo = (r / im.R) * im.R, hi = lo + im.R;
-  for (int i = threadIdx.x; i < 3 * (TPX + 2) * 4; i += blockDim.x) {
-    const int q = i & 3, px = (i >> 2) % (TPX + 2), rr = (i >> 2) / (TPX + 2);
-    const int gx = x0 - 1 + px, gr = r - 1 + rr;
-    int4 v = make_int4(0, 0, 0, 0);
-    if (gx >= 0 && gx < im.W && gr >= lo && gr < hi)
-      v = *reinterpret_cast<const int4*>(x + ((int64_t)gr * im.W + gx) * NC + q * 8);
-    *reinterpret_cast<int4*>(sIn + (rr * (TPX + 2) + px) * LDA + q * 8) = v;
   }
 }
 
@@ -962,228 +944,492 @@ __global__ void __launch_bounds__(FZ_THREADS, 1) k_net_fwd(const __grid_constant
 }
 
 // ----------------------------------------------------------- backward
-// g6 = dout * m; dy5[p][ci] = (sum_d W6[d][ci] g6[p - off(d)]) * (y5[p][ci] > 0)
-__global__ void k_l6_bwd(Image im, const float* __restrict__ dout, const float2* __restrict__ in,
-                         const bf16* __restrict__ y5, const float* __restrict__ P, bf16* __restrict__ dy5) {
-  __shared__ float w[W6_N];
-  for (int i = threadIdx.x; i < W6_N; i += blockDim.x) w[i] = P[OFF_W6 + i];
-  __syncthreads();
+// g6 = dout * m
+__global__ void __launch_bounds__(256) k_l6_gate(int64_t npx, const float* __restrict__ dout,
+                                                 const float2* __restrict__ in, float* __restrict__ g6) {
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= im.npx()) return;
-  const int x = (int)(p % im.W), r = (int)(p / im.W);
-  const int lo = (r / im.R) * im.R, hi = lo + im.R;
-  float g[9];
+  if (p < npx) g6[p] = dout[p] * in[p].y;
+}
+
+// The gradients of layers 1 and 6 on the CUDA cores walk the image the same
+// way: a warp takes a run of BW_RUN pixels of one row in four segments; lane
+// (seg, cg) walks its segment left to right for channels 4 cg .. 4 cg + 3 (8
+// lanes read a pixel's 64 bytes), keeping the 3 x 3 window of the other
+// operand in registers (three new values a pixel) and BW_PF pixels' loads in
+// flight, and its share of the weight gradient in registers to the end.  The
+// lanes' and warps' shares are added in a fixed order.  Bounded by the
+// packed FMAs (fma.rn.f32x2) and the one pass over the 32-channel operand.
+// At 16 x 512^2: k_l6_back 161 us and k_l1_wgrad 147 us; one pixel per warp
+// (lane = channel, every tap gathered anew) took 1668 + 197 us (weight and data
+// gradient apart) and 1481 us.
+constexpr int BW_THREADS = 128;
+constexpr int BW_SEG = 32;           // pixels per lane and run
+constexpr int BW_RUN = 4 * BW_SEG;
+constexpr int BW_CTAS = 3;           // per SM
+
+// sum over the four segments (lanes that share cg)
+__device__ __forceinline__ float seg_sum(float v) {
+  v += __shfl_xor_sync(0xffffffffu, v, 8);
+  return v + __shfl_xor_sync(0xffffffffu, v, 16);
+}
+
+__device__ __forceinline__ float2 fz_unpk(uint64_t v) {
+  return make_float2(__uint_as_float((uint32_t)v), __uint_as_float((uint32_t)(v >> 32)));
+}
+
+// the four BF16 of v as two packed FP32 pairs
+__device__ __forceinline__ void bf4_pairs(uint2 v, uint64_t& a, uint64_t& b) {
+  a = fz_pk(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u));
+  b = fz_pk(__uint_as_float(v.y << 16), __uint_as_float(v.y & 0xFFFF0000u));
+}
+
+// Layer 6 backward in one pass over y5: the data gradient
+//   dy5[p][ci] = (sum_d W6[d][ci] g6[p - off(d)]) (y5[p][ci] > 0)
+// and the weight-gradient partials, slot d * 32 + ci: sum_p g6[p - off(d)]
+// y5[p][ci]; slot 288: sum g6.  Both need the same 3 x 3 window of g6.
+__global__ void __launch_bounds__(BW_THREADS, BW_CTAS) k_l6_back(Image im, const float* __restrict__ g6,
+                                                                 const bf16* __restrict__ y5,
+                                                                 const float* __restrict__ P, bf16* __restrict__ dy5,
+                                                                 float* __restrict__ part) {
+  constexpr int PF = 8;
+  __shared__ float sm[BW_THREADS / 32][W6_N + B6_N];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, cg = lane & 7, seg = lane >> 3;
+  uint64_t wt[9][2], acc[9][2];
 #pragma unroll
   for (int d = 0; d < 9; ++d) {
-    const int xx = x - (d % 3 - 1), rr = r - (d / 3 - 1);
-    const int64_t q = (int64_t)rr * im.W + xx;
-    g[d] = (xx >= 0 && xx < im.W && rr >= lo && rr < hi) ? dout[q] * in[q].y : 0.0f;
+    const float* q = P + OFF_W6 + d * NC + 4 * cg;
+    wt[d][0] = fz_pk(q[0], q[1]);
+    wt[d][1] = fz_pk(q[2], q[3]);
+    acc[d][0] = acc[d][1] = 0;
   }
-  __align__(16) bf16 yv[NC];
-  __align__(16) bf16 ov[NC];
+  float bacc = 0.0f;
+  const int runs = (im.W + BW_RUN - 1) / BW_RUN;
+  const int64_t tasks = (int64_t)runs * im.H;
+  for (int64_t t = (int64_t)blockIdx.x * (BW_THREADS / 32) + w; t < tasks; t += (int64_t)gridDim.x * (BW_THREADS / 32)) {
+    const int r = (int)(t / runs), xs = (int)(t - (int64_t)r * runs) * BW_RUN + seg * BW_SEG;
+    const int lo = (r / im.R) * im.R, hi = lo + im.R;
+    const bool rv[3] = {r - 1 >= lo, true, r + 1 < hi};
+    const float* gr = g6 + (int64_t)r * im.W;
+    auto g_at = [&](int k, int x) {  // g6 at row r + k - 1, column x
+      return (rv[k] && x >= 0 && x < im.W) ? __ldg(gr + (int64_t)(k - 1) * im.W + x) : 0.0f;
+    };
+    float g0[3], g1[3];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) reinterpret_cast<int4*>(yv)[q] = reinterpret_cast<const int4*>(y5 + p * NC)[q];
-#pragma unroll 4
-  for (int ci = 0; ci < NC; ++ci) {
-    float a = 0.0f;
+    for (int k = 0; k < 3; ++k) {
+      g0[k] = g_at(k, xs - 1);
+      g1[k] = g_at(k, xs);
+    }
+    const int64_t px0 = (int64_t)r * im.W;
+    for (int x0 = xs; x0 < xs + BW_SEG && x0 < im.W; x0 += PF) {
+      uint2 yv[PF];
+      float gn[3][PF];
 #pragma unroll
-    for (int d = 0; d < 9; ++d) a += w[d * NC + ci] * g[d];
-    ov[ci] = __float2bfloat16_rn(__bfloat162float(yv[ci]) > 0.0f ? a : 0.0f);
-  }
+      for (int j = 0; j < PF; ++j)
+        yv[j] = x0 + j < im.W ? __ldg(reinterpret_cast<const uint2*>(y5 + (px0 + x0 + j) * NC + 4 * cg))
+                              : make_uint2(0u, 0u);
 #pragma unroll
-  for (int q = 0; q < 4; ++q) reinterpret_cast<int4*>(dy5 + p * NC)[q] = reinterpret_cast<const int4*>(ov)[q];
-}
-
-// pixels [p0, p1) of CTA b out of nb over n pixels
-__device__ __forceinline__ void chunk_of(int64_t n, int b, int nb, int64_t& p0, int64_t& p1) {
-  const int64_t c = (n + nb - 1) / nb;
-  p0 = (int64_t)b * c < n ? (int64_t)b * c : n;
-  p1 = p0 + c < n ? p0 + c : n;
-}
-
-// layer 6 gradient partials: slot d * 32 + ci: sum g6[p] y5[p + off(d)][ci]; slot 288: sum g6[p].
-// A warp walks pixels of the CTA's chunk (lane = input channel, 9 tap sums in
-// registers); the 8 warps' sums are added in a fixed order.
-__global__ void __launch_bounds__(256) k_l6_wgrad(Image im, const float* __restrict__ dout,
-                                                  const float2* __restrict__ in, const bf16* __restrict__ y5,
-                                                  float* __restrict__ part) {
-  __shared__ float sm[8][W6_N + B6_N];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int64_t p0, p1;
-  chunk_of(im.npx(), blockIdx.x, gridDim.x, p0, p1);
-  float acc[9], bacc = 0.0f;
+      for (int k = 0; k < 3; ++k)
 #pragma unroll
-  for (int d = 0; d < 9; ++d) acc[d] = 0.0f;
-  // 4 pixels per step, their loads issued before the sums (latency hiding)
-  for (int64_t pb = p0 + w; pb < p1; pb += 32) {
-    float g[4], v[4][9];
+        for (int j = 0; j < PF; ++j) gn[k][j] = g_at(k, x0 + j + 1);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int64_t p = pb + 8 * u;
-      g[u] = p < p1 ? dout[p] * in[p].y : 0.0f;
-      const int x = (int)(p % im.W), r = (int)(p / im.W);
-      const int lo = (r / im.R) * im.R, hi = lo + im.R;
+      for (int j = 0; j < PF; ++j) {
+        uint64_t ya, yb, da = 0, db = 0;
+        bf4_pairs(yv[j], ya, yb);
 #pragma unroll
-      for (int d = 0; d < 9; ++d) {
-        const int xx = x + d % 3 - 1, rr = r + d / 3 - 1;
-        v[u][d] = (p < p1 && xx >= 0 && xx < im.W && rr >= lo && rr < hi)
-                      ? __bfloat162float(y5[((int64_t)rr * im.W + xx) * NC + lane])
-                      : 0.0f;
+        for (int d = 0; d < 9; ++d) {  // g6 at p - off(d): row 2 - d / 3, column 2 - d % 3 of the window
+          const int k = 2 - d / 3, c = 2 - d % 3;
+          const float g = c == 0 ? g0[k] : (c == 1 ? g1[k] : gn[k][j]);
+          const uint64_t gg = fz_pk(g, g);
+          fz_fma2(acc[d][0], ya, gg);
+          fz_fma2(acc[d][1], yb, gg);
+          fz_fma2(da, wt[d][0], gg);
+          fz_fma2(db, wt[d][1], gg);
+        }
+        if (x0 + j < im.W) {
+          bacc += g1[1];
+          const float2 a = fz_unpk(da), b = fz_unpk(db), p = fz_unpk(ya), q = fz_unpk(yb);
+          const __nv_bfloat162 h0 = __floats2bfloat162_rn(p.x > 0.0f ? a.x : 0.0f, p.y > 0.0f ? a.y : 0.0f);
+          const __nv_bfloat162 h1 = __floats2bfloat162_rn(q.x > 0.0f ? b.x : 0.0f, q.y > 0.0f ? b.y : 0.0f);
+          *reinterpret_cast<uint2*>(dy5 + (px0 + x0 + j) * NC + 4 * cg) =
+              make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          g0[k] = g1[k];
+          g1[k] = gn[k][j];
+        }
       }
     }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      bacc += g[u];
-#pragma unroll
-      for (int d = 0; d < 9; ++d) acc[d] += g[u] * v[u][d];
-    }
   }
 #pragma unroll
-  for (int d = 0; d < 9; ++d) sm[w][d * NC + lane] = acc[d];
+  for (int d = 0; d < 9; ++d)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float2 v = fz_unpk(acc[d][h]);
+      const float a = seg_sum(v.x), b = seg_sum(v.y);
+      if (seg == 0) {
+        sm[w][d * NC + 4 * cg + 2 * h] = a;
+        sm[w][d * NC + 4 * cg + 2 * h + 1] = b;
+      }
+    }
+  bacc = seg_sum(bacc);
   if (lane == 0) sm[w][W6_N] = bacc;
   __syncthreads();
-  for (int i = threadIdx.x; i < W6_N + B6_N; i += blockDim.x) {
+  for (int i = threadIdx.x; i < W6_N + B6_N; i += BW_THREADS) {
     float t = 0.0f;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) t += sm[k][i];
+    for (int k = 0; k < BW_THREADS / 32; ++k) t += sm[k][i];
     part[(int64_t)blockIdx.x * (W6_N + B6_N) + i] = t;
   }
 }
 
-// layer 1 gradient partials: slot (co * 9 + d) * 2 + ci: sum dy1[p][co] in[p + off(d)][ci];
-// slot 576 + co: sum dy1[p][co].  A warp walks pixels (lane = output channel).
-__global__ void __launch_bounds__(256) k_l1_wgrad(Image im, const bf16* __restrict__ dy1,
-                                                  const float2* __restrict__ in, float* __restrict__ part) {
-  __shared__ float sm[8][W1_N + B1_N];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int64_t p0, p1;
-  chunk_of(im.npx(), blockIdx.x, gridDim.x, p0, p1);
-  float acc[9][2], bacc = 0.0f;
+// Layer 1 gradient partials: slot (co * 9 + d) * 2 + ci: sum dy1[p][co] in[p + off(d)][ci];
+// slot 576 + co: sum dy1[p][co].  The packed pairs are the two input channels.
+__global__ void __launch_bounds__(BW_THREADS, BW_CTAS) k_l1_wgrad(Image im, const bf16* __restrict__ dy1,
+                                                                  const float2* __restrict__ in,
+                                                                  float* __restrict__ part) {
+  constexpr int PF = 4;
+  __shared__ float sm[BW_THREADS / 32][W1_N + B1_N];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, cg = lane & 7, seg = lane >> 3;
+  uint64_t acc[9][4];
+  float bacc[4];
 #pragma unroll
-  for (int d = 0; d < 9; ++d) acc[d][0] = acc[d][1] = 0.0f;
-  // 4 pixels per step, their loads issued before the sums (latency hiding)
-  for (int64_t pb = p0 + w; pb < p1; pb += 32) {
-    float g[4];
-    float2 v[4][9];
+  for (int d = 0; d < 9; ++d)
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int64_t p = pb + 8 * u;
-      g[u] = p < p1 ? __bfloat162float(dy1[p * NC + lane]) : 0.0f;
-      const int x = (int)(p % im.W), r = (int)(p / im.W);
-      const int lo = (r / im.R) * im.R, hi = lo + im.R;
+    for (int c = 0; c < 4; ++c) acc[d][c] = 0;
 #pragma unroll
-      for (int d = 0; d < 9; ++d) {
-        const int xx = x + d % 3 - 1, rr = r + d / 3 - 1;
-        v[u][d] = (p < p1 && xx >= 0 && xx < im.W && rr >= lo && rr < hi) ? in[(int64_t)rr * im.W + xx]
-                                                                            : make_float2(0.0f, 0.0f);
-      }
+  for (int c = 0; c < 4; ++c) bacc[c] = 0.0f;
+  const int runs = (im.W + BW_RUN - 1) / BW_RUN;
+  const int64_t tasks = (int64_t)runs * im.H;
+  for (int64_t t = (int64_t)blockIdx.x * (BW_THREADS / 32) + w; t < tasks; t += (int64_t)gridDim.x * (BW_THREADS / 32)) {
+    const int r = (int)(t / runs), xs = (int)(t - (int64_t)r * runs) * BW_RUN + seg * BW_SEG;
+    const int lo = (r / im.R) * im.R, hi = lo + im.R;
+    const bool rv[3] = {r - 1 >= lo, true, r + 1 < hi};
+    const unsigned long long* ir = reinterpret_cast<const unsigned long long*>(in) + (int64_t)r * im.W;
+    auto v_at = [&](int k, int x) -> uint64_t {  // in at row r + k - 1, column x
+      return (rv[k] && x >= 0 && x < im.W) ? __ldg(ir + (int64_t)(k - 1) * im.W + x) : 0ull;
+    };
+    uint64_t v0[3], v1[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      v0[k] = v_at(k, xs - 1);
+      v1[k] = v_at(k, xs);
     }
+    const int64_t px0 = (int64_t)r * im.W;
+    for (int x0 = xs; x0 < xs + BW_SEG && x0 < im.W; x0 += PF) {
+      uint2 dv[PF];
+      uint64_t vn[3][PF];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      bacc += g[u];
+      for (int j = 0; j < PF; ++j)
+        dv[j] = x0 + j < im.W ? __ldg(reinterpret_cast<const uint2*>(dy1 + (px0 + x0 + j) * NC + 4 * cg))
+                              : make_uint2(0u, 0u);
 #pragma unroll
-      for (int d = 0; d < 9; ++d) {
-        acc[d][0] += g[u] * v[u][d].x;
-        acc[d][1] += g[u] * v[u][d].y;
+      for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int j = 0; j < PF; ++j) vn[k][j] = v_at(k, x0 + j + 1);
+#pragma unroll
+      for (int j = 0; j < PF; ++j) {
+        const float g[4] = {__uint_as_float(dv[j].x << 16), __uint_as_float(dv[j].x & 0xFFFF0000u),
+                            __uint_as_float(dv[j].y << 16), __uint_as_float(dv[j].y & 0xFFFF0000u)};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          bacc[c] += g[c];
+          const uint64_t gg = fz_pk(g[c], g[c]);
+#pragma unroll
+          for (int d = 0; d < 9; ++d) {
+            const int k = d / 3;
+            fz_fma2(acc[d][c], d % 3 == 0 ? v0[k] : (d % 3 == 1 ? v1[k] : vn[k][j]), gg);
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          v0[k] = v1[k];
+          v1[k] = vn[k][j];
+        }
       }
     }
   }
 #pragma unroll
-  for (int d = 0; d < 9; ++d) {
-    sm[w][(lane * 9 + d) * 2] = acc[d][0];
-    sm[w][(lane * 9 + d) * 2 + 1] = acc[d][1];
+  for (int c = 0; c < 4; ++c) {
+    const int co = 4 * cg + c;
+#pragma unroll
+    for (int d = 0; d < 9; ++d) {
+      const float2 v = fz_unpk(acc[d][c]);
+      const float a = seg_sum(v.x), b = seg_sum(v.y);
+      if (seg == 0) {
+        sm[w][(co * 9 + d) * 2] = a;
+        sm[w][(co * 9 + d) * 2 + 1] = b;
+      }
+    }
+    const float bs = seg_sum(bacc[c]);
+    if (seg == 0) sm[w][W1_N + co] = bs;
   }
-  sm[w][W1_N + lane] = bacc;
   __syncthreads();
-  for (int i = threadIdx.x; i < W1_N + B1_N; i += blockDim.x) {
+  for (int i = threadIdx.x; i < W1_N + B1_N; i += BW_THREADS) {
     float t = 0.0f;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) t += sm[k][i];
+    for (int k = 0; k < BW_THREADS / 32; ++k) t += sm[k][i];
     part[(int64_t)blockIdx.x * (W1_N + B1_N) + i] = t;
   }
 }
 
-// 32 -> 32 weight-gradient partials on the tensor cores (mma.sync fragments):
-// part[cta][d][k = ci][n = co] = sum_p x[p + off(d)][ci] dy[p][co].
-// Warp w owns the 16 x 16 quadrant (ci block w >> 1, co block w & 1) of all 9
-// taps: per 16-pixel step it loads one dy fragment and 9 shifted x fragments.
-__global__ void __launch_bounds__(128) k_conv32_wgrad(Image im, const bf16* __restrict__ x,
-                                                      const bf16* __restrict__ dy, float* __restrict__ part) {
+// Weight and bias gradients of a 32 -> 32 layer on the tensor cores:
+//   dW[d][ci][co] = sum_p x[p + off(d)][ci] dy[p][co],  db[co] = sum_p dy[p][co].
+// With q = p + off(d), a tap's row offset is a row of dy and its column offset
+// a shift of x, so one MMA over 16 pixels of a row forms all nine taps at once:
+// M = four column shifts of x times 32 channels (three used), N = three rows of
+// dy times 32 channels, K = 16 pixels, 128 x 96 x 16.  Both operands are
+// "MN-major": a pixel's 32 channels are one 64-byte row of the tensor copy's
+// 64-byte swizzled layout, eight pixels along K make a 512-byte atom (SBO), and
+// the stride between atoms along M is one pixel (LBO 64 bytes: the shifts) and
+// along N one row of dy.  A job is WG_ROWS rows x 128 pixels: two tensor copies
+// (x with its halo columns, dy with its halo rows), zero outside the image.
+// Warps 5-8 issue the MMAs of one row of the job each (one thread's issue takes
+// some 190 cycles whatever N, see k_net_fwd; four overlap) into accumulators of
+// their own (128 x 96, TMEM columns 128 apart); every WG_FLUSH jobs warps 0-3
+// add the accumulators to FP32 sums in registers, so no chain in the tensor
+// core is longer than 8 WG_FLUSH MMAs.  Warps 0-3 also sum dy for the bias from
+// the staged rows.  One CTA per SM; part[cta]: 9 x 32 x 32 sums ([d][ci][co]),
+// then 32 bias sums.  Bounded by the two passes over HBM: 99 us per layer at 16
+// x 512^2 (537 MB, 5.4 TB/s); the mma.sync form, staged by the threads, took
+// 607 us and its separate bias pass 66 us.
+// Barriers: full[s] (copies), empty[s] (4 commits + 4 sum warps), tfull (4
+// commits), tempty (4 sum warps), drain[w] (warp 5 + w's last commit).  Waits
+// are bounded as in k_conv32_tma.
+constexpr int WG_ROWS = 4;
+constexpr int WG_STAGES = 2;
+constexpr int WG_FLUSH = 16;
+constexpr int WG_X_BYTES = WG_ROWS * TC_PIX * NC * 2;        // 33,280
+constexpr int WG_DY_BYTES = (WG_ROWS + 2) * TPX * NC * 2;    // 49,152
+constexpr int WG_DY = (WG_X_BYTES + 64 + 1023) / 1024 * 1024;  // dy after x (whose fourth shift reads one row past it)
+constexpr int WG_STAGE = WG_DY + WG_DY_BYTES;
+constexpr int WG_BAR = WG_STAGES * WG_STAGE;
+constexpr int WG_NBAR = 2 * WG_STAGES + 2 + 4;
+constexpr int WG_SB = WG_BAR + 8 * WG_NBAR + 16;             // after the TMEM slot and the abort flag: bias sums
+constexpr int WG_SMEM = WG_SB + 4 * NC * 4;
+constexpr int WG_THREADS = 288;  // warps 0-3 sums, 4 copies, 5-8 MMAs
+constexpr int WG_PART = WM_N + BM_N;
+static_assert(WG_DY % 1024 == 0 && WG_STAGE % 1024 == 0 && WG_SMEM <= 227 * 1024, "wgrad shared memory");
+
+// descriptor of an MN-major operand in the 64-byte swizzled layout: atoms of 32
+// channels x 8 pixels, lbo bytes between atoms along M / N, 512 along K
+__device__ __forceinline__ uint64_t tc_desc_mn64(uint32_t saddr, uint32_t lbo) {
+  return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
+         ((uint64_t)(512 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
+}
+
+__global__ void __launch_bounds__(WG_THREADS, 1) k_conv32_wgrad(const __grid_constant__ CUtensorMap xmap,
+                                                                const __grid_constant__ CUtensorMap dmap, Image im,
+                                                                float* __restrict__ part, int* __restrict__ err) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  bf16* sIn = reinterpret_cast<bf16*>(smem_raw);  // [3][TPX + 2][LDA]
-  bf16* sDy = sIn + 3 * (TPX + 2) * LDA;          // [TPX][LDA]
-  const int segs = (im.W + TPX - 1) / TPX;
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int kb = warp >> 1, nb = warp & 1;
-  wm::fragment<wm::accumulator, 16, 16, 16, float> acc[9];
-#pragma unroll
-  for (int d = 0; d < 9; ++d) wm::fill_fragment(acc[d], 0.0f);
-  const int64_t jobs = (int64_t)segs * im.H;
-  for (int64_t job = blockIdx.x; job < jobs; job += gridDim.x) {
-    const int r = (int)(job / segs), x0 = (int)(job % segs) * TPX;
-    __syncthreads();
-    stage_rows(im, x, r, x0, sIn);
-    for (int i = tid; i < TPX * 4; i += blockDim.x) {
-      const int q = i & 3, px = i >> 2, gx = x0 + px;
-      int4 v = make_int4(0, 0, 0, 0);
-      if (gx < im.W) v = *reinterpret_cast<const int4*>(dy + ((int64_t)r * im.W + gx) * NC + q * 8);
-      *reinterpret_cast<int4*>(sDy + px * LDA + q * 8) = v;
+  const uint32_t base = smem_addr(smem_raw), bars = base + WG_BAR;
+  auto full = [&](int st) { return bars + 8 * st; };
+  auto empty = [&](int st) { return bars + 8 * (WG_STAGES + st); };
+  const uint32_t tfull = bars + 8 * (2 * WG_STAGES), tempty = tfull + 8;
+  auto drain = [&](int w) { return tempty + 8 + 8 * w; };
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(smem_raw + WG_BAR + 8 * WG_NBAR);
+  volatile int* abort = reinterpret_cast<volatile int*>(smem_raw + WG_BAR + 8 * WG_NBAR + 8);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid == 0) {
+    for (int b = 0; b < WG_NBAR; ++b) {
+      const uint32_t cnt = b < WG_STAGES ? 1u : (b < 2 * WG_STAGES ? 8u : (b < 2 * WG_STAGES + 2 ? 4u : 1u));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bars + 8 * b), "r"(cnt));
     }
-    __syncthreads();
-#pragma unroll 1
-    for (int ks = 0; ks < TPX / 16; ++ks) {
-      wm::fragment<wm::matrix_b, 16, 16, 16, bf16, wm::row_major> fb;
-      wm::load_matrix_sync(fb, sDy + (16 * ks) * LDA + nb * 16, LDA);
-#pragma unroll
-      for (int d = 0; d < 9; ++d) {
-        wm::fragment<wm::matrix_a, 16, 16, 16, bf16, wm::col_major> fa;
-        wm::load_matrix_sync(fa, sIn + ((d / 3) * (TPX + 2) + 16 * ks + d % 3) * LDA + kb * 16, LDA);
-        wm::mma_sync(acc[d], fa, fb, acc[d]);
+    *abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;");
+  }
+  if (warp == 5) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_addr(tslot)));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  const uint32_t tmem = *tslot;
+  const int segs = (im.W + TPX - 1) / TPX, chunks = (im.R + WG_ROWS - 1) / WG_ROWS;
+  const int64_t jobs = (int64_t)segs * chunks * (im.H / im.R);
+  const int64_t njob = jobs > (int64_t)blockIdx.x ? (jobs - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+  if (warp == 4) {
+    if (lane == 0) {
+      int64_t k = 0;
+      for (; k < njob; ++k) {
+        const int st = (int)(k % WG_STAGES);
+        const uint32_t u = (uint32_t)(k / WG_STAGES);
+        if (u > 0 && !cp_wait(empty(st), (u - 1) & 1u, abort)) break;
+        const int64_t job = blockIdx.x + k * gridDim.x;
+        const int x0 = (int)(job % segs) * TPX, c = (int)((job / segs) % chunks);
+        const int img = (int)(job / ((int64_t)segs * chunks)), r0 = c * WG_ROWS;
+        const uint32_t sa = base + st * WG_STAGE;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full(st)),
+                     "r"((uint32_t)(WG_X_BYTES + WG_DY_BYTES))
+                     : "memory");
+        asm volatile(
+            "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
+            "%5}], [%6];" ::"r"(sa),
+            "l"(reinterpret_cast<uint64_t>(&xmap)), "r"(0), "r"(x0 - 1), "r"(r0), "r"(img), "r"(full(st))
+            : "memory");
+        asm volatile(
+            "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
+            "%5}], [%6];" ::"r"(sa + WG_DY),
+            "l"(reinterpret_cast<uint64_t>(&dmap)), "r"(0), "r"(x0), "r"(r0 - 1), "r"(img), "r"(full(st))
+            : "memory");
+      }
+      // copies still in flight (an aborted run) land before the CTA ends
+      for (int64_t q = k > WG_STAGES ? k - WG_STAGES : 0; q < k; ++q) {
+        volatile int never = 0;
+        cp_wait(full((int)(q % WG_STAGES)), (uint32_t)(q / WG_STAGES) & 1u, &never);
       }
     }
-  }
-  float* out = part + (int64_t)blockIdx.x * WM_N;
+  } else if (warp >= 5) {
+    if (lane == 0) {
+      const int row = warp - 5;  // of every job
+      // bf16 operands, f32 accumulators, both MN-major (bits 15, 16)
+      constexpr uint32_t idesc = tc_idesc(128, 96) | (1u << 15) | (1u << 16);
+      const uint32_t dst = tmem + (uint32_t)(128 * row);
+      uint32_t nf = 0;  // flushes so far
+      bool fresh = true;
+      for (int64_t k = 0; k < njob; ++k) {
+        const int st = (int)(k % WG_STAGES);
+        if (!cp_wait(full(st), (uint32_t)(k / WG_STAGES) & 1u, abort)) break;
+        if (fresh && nf > 0 && !cp_wait(tempty, (nf - 1) & 1u, abort)) break;
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        const uint32_t sx = base + st * WG_STAGE + row * TC_PIX * 64;
+        const uint32_t sd = base + st * WG_STAGE + WG_DY + row * TPX * 64;
+#pragma unroll 1
+        for (int q = 0; q < TPX / 16; ++q) {
+          const uint64_t da = tc_desc_mn64(sx + q * 1024, 64);
+          const uint64_t db = tc_desc_mn64(sd + q * 1024, TPX * 64);
+          asm volatile(
+              "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+              "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(dst),
+              "l"(da), "l"(db), "r"(idesc), "r"((uint32_t)(!fresh || q > 0)));
+        }
+        fresh = false;
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(empty(st))
+                     : "memory");
+        if ((k + 1) % WG_FLUSH == 0 || k + 1 == njob) {
+          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(tfull)
+                       : "memory");
+          ++nf;
+          fresh = true;
+        }
+      }
+      // the last MMAs complete before TMEM is freed
+      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(drain(row))
+                   : "memory");
+      volatile int never = 0;
+      cp_wait(drain(row), 0u, &never);
+    }
+  } else {
+    // sums: thread t = TMEM lane t = x's shift t / 32, channel ci = t % 32, 96 columns (dy's row, co)
+    float sum[96], bsum[8];
 #pragma unroll
-  for (int d = 0; d < 9; ++d)
-    wm::store_matrix_sync(out + (d * NC + 16 * kb) * NC + 16 * nb, acc[d], NC, wm::mem_row_major);
-}
-
-// bias-gradient partials of a 32-channel gradient: part[cta][c] = sum over the CTA's pixels
-__global__ void __launch_bounds__(256) k_bias_grad(int64_t npx, const bf16* __restrict__ dy,
-                                                   float* __restrict__ part) {
-  __shared__ float sm[8][NC];
-  const int c = threadIdx.x & 31, row = threadIdx.x >> 5;
-  int64_t p0, p1;
-  chunk_of(npx, blockIdx.x, gridDim.x, p0, p1);
-  float a = 0.0f;
-  for (int64_t p = p0 + row; p < p1; p += 8) a += __bfloat162float(dy[p * NC + c]);
-  sm[row][c] = a;
+    for (int c = 0; c < 96; ++c) sum[c] = 0.0f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) bsum[c] = 0.0f;
+    const int ch = tid & 3;  // the 8-channel chunk this thread sums for the bias
+    uint32_t nf = 0;
+    for (int64_t k = 0; k < njob; ++k) {
+      const int st = (int)(k % WG_STAGES);
+      bool ok = cp_wait(full(st), (uint32_t)(k / WG_STAGES) & 1u, abort);
+      if (!__all_sync(0xffffffffu, ok)) {
+        *abort = 1;
+        break;
+      }
+      const unsigned char* sd = smem_raw + st * WG_STAGE + WG_DY + TPX * 64;  // without the halo row above
+#pragma unroll 4
+      for (int q = 0; q < WG_ROWS * TPX / 32; ++q) {
+        const uint32_t off = (uint32_t)(32 * q + (tid >> 2)) * 64;
+        const uint32_t sw = (off >> 7) & 3u;  // 64-byte swizzle: chunk index xor address bits 7-8
+        const uint4 v = *reinterpret_cast<const uint4*>(sd + off + (((uint32_t)ch ^ sw) << 4));
+        const uint32_t e[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          bsum[2 * c] += __uint_as_float(e[c] << 16);
+          bsum[2 * c + 1] += __uint_as_float(e[c] & 0xFFFF0000u);
+        }
+      }
+      __syncwarp();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(empty(st)) : "memory");
+      if ((k + 1) % WG_FLUSH != 0 && k + 1 != njob) continue;
+      ok = cp_wait(tfull, nf & 1u, abort);
+      if (!__all_sync(0xffffffffu, ok)) {
+        *abort = 1;
+        break;
+      }
+      ++nf;
+      asm volatile("tcgen05.fence::after_thread_sync;");
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int h = 0; h < 3; ++h) {
+          uint32_t v[NC];
+          asm volatile(
+              "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,"
+              "%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+              : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
+                "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]),
+                "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]),
+                "=r"(v[30]), "=r"(v[31])
+              : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(128 * a + NC * h)));
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+          for (int c = 0; c < NC; ++c) sum[NC * h + c] += __uint_as_float(v[c]);
+        }
+      asm volatile("tcgen05.fence::before_thread_sync;");
+      __syncwarp();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty) : "memory");
+    }
+    float* out = part + (int64_t)blockIdx.x * WG_PART;
+    if (warp < 3) {  // shift = tap column; dy's row n belongs to tap row 2 - n
+#pragma unroll
+      for (int h = 0; h < 3; ++h)
+#pragma unroll
+        for (int c = 0; c < NC; c += 4)
+          *reinterpret_cast<float4*>(out + (((2 - h) * 3 + warp) * NC + lane) * NC + c) =
+              make_float4(sum[NC * h + c], sum[NC * h + c + 1], sum[NC * h + c + 2], sum[NC * h + c + 3]);
+    }
+    // bias: lanes of equal chunk within the warp, then the four warps through shared memory
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      for (int o = 4; o < 32; o <<= 1) bsum[c] += __shfl_xor_sync(0xffffffffu, bsum[c], o);
+    float* sb = reinterpret_cast<float*>(smem_raw + WG_SB);
+    if (lane < 4)
+#pragma unroll
+      for (int c = 0; c < 8; ++c) sb[warp * NC + lane * 8 + c] = bsum[c];
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    if (tid < NC) out[WM_N + tid] = ((sb[tid] + sb[NC + tid]) + sb[2 * NC + tid]) + sb[3 * NC + tid];
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
-  if (row == 0) {
-    float s = 0.0f;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) s += sm[i][c];
-    part[(int64_t)blockIdx.x * NC + c] = s;
+  if (tid == 0 && *abort) atomicExch(err, 1);
+  if (warp == 5) {
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
   }
 }
 
-// out[i] = sum over parts of part[c][i] (fixed order)
-__global__ void k_sum_parts(const float* __restrict__ part, int nparts, int n, float* __restrict__ out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+// out[place(i)] = sum over parts of part[c][i], i < n: 32 outputs per CTA, 32
+// threads per output take every 32nd part, their sums added in a fixed order.
+// wm >= 0: the first wm outputs are a middle layer's weights, (d 32 + ci) 32 +
+// co -> (co 9 + d) 32 + ci.
+constexpr int SP_THREADS = 1024;
+__global__ void __launch_bounds__(SP_THREADS) k_sum_parts(const float* __restrict__ part, int nparts, int n, int wm,
+                                                          float* __restrict__ out) {
+  __shared__ float sm[32][33];
+  const int o = threadIdx.x & 31, g = threadIdx.x >> 5, i = blockIdx.x * 32 + o;
   float s = 0.0f;
-  for (int c = 0; c < nparts; ++c) s += part[(int64_t)c * n + i];
-  out[i] = s;
-}
-
-// middle-layer weight gradient: G[(co 9 + d) 32 + ci] = sum over parts of part[c][(d 32 + ci) 32 + co]
-__global__ void k_sum_wgrad(const float* __restrict__ part, int nparts, float* __restrict__ G) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= WM_N) return;
-  float s = 0.0f;
-  for (int c = 0; c < nparts; ++c) s += part[(int64_t)c * WM_N + j];
-  const int co = j % NC, ci = (j / NC) % NC, d = j / (NC * NC);
-  G[(co * 9 + d) * NC + ci] = s;
+  if (i < n)
+    for (int c = g; c < nparts; c += 32) s += part[(int64_t)c * n + i];
+  sm[g][o] = s;
+  __syncthreads();
+  if (g != 0 || i >= n) return;
+  s = 0.0f;
+#pragma unroll
+  for (int k = 0; k < 32; ++k) s += sm[k][o];
+  const int co = i % NC, ci = (i / NC) % NC, d = i / (NC * NC);
+  out[i < wm ? (co * 9 + d) * NC + ci : i] = s;
 }
 
 // ------------------------------------------------------------- weights
@@ -1513,28 +1759,26 @@ struct NN {
   int snblk = 0;
 };
 
-static size_t wgrad_smem() { return (size_t)(3 * (TPX + 2) * LDA + TPX * LDA) * sizeof(bf16); }
-
 static void set_attrs() {
   static bool done = false;
   if (done) return;
   EB_CUDA(cudaFuncSetAttribute(k_conv32_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CP_SMEM));
-  EB_CUDA(cudaFuncSetAttribute(k_conv32_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wgrad_smem()));
+  EB_CUDA(cudaFuncSetAttribute(k_conv32_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WG_SMEM));
   EB_CUDA(cudaFuncSetAttribute(k_net_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FZ_SMEM));
   done = true;
 }
 
-// Tensor map of a BF16 NHWC activation stack for k_conv32_tma: dimensions
-// (32 channels, pixel, row in image, image), strides 64 B, W * 64 B,
-// R * W * 64 B; box (32, 130, 3, 1) written in the 64-byte swizzled layout;
+// Tensor map of a BF16 NHWC activation stack: dimensions (32 channels, pixel,
+// row in image, image), strides 64 B, W * 64 B, R * W * 64 B; box (32, px,
+// rows, 1), k_conv32_tma's by default, written in the 64-byte swizzled layout;
 // out-of-range elements read as zero.
-static CUtensorMap conv_map(const bf16* x, const Image& im) {
+static CUtensorMap conv_map(const bf16* x, const Image& im, int px = TC_PIX, int rows = 3) {
   EB_REQUIRE(((uintptr_t)x & 15) == 0, EB_ERR_INVALID, "conv: activations not 16-byte aligned");
   EB_REQUIRE(im.R > 0 && im.H % im.R == 0, EB_ERR_INVALID, "conv: rows are not whole images");
   CUtensorMap m;
   const cuuint64_t dims[4] = {(cuuint64_t)NC, (cuuint64_t)im.W, (cuuint64_t)im.R, (cuuint64_t)(im.H / im.R)};
   const cuuint64_t strides[3] = {(cuuint64_t)NC * 2, (cuuint64_t)im.W * NC * 2, (cuuint64_t)im.R * im.W * NC * 2};
-  const cuuint32_t box[4] = {(cuuint32_t)NC, (cuuint32_t)TC_PIX, 3, 1};
+  const cuuint32_t box[4] = {(cuuint32_t)NC, (cuuint32_t)px, (cuuint32_t)rows, 1};
   const cuuint32_t estr[4] = {1, 1, 1, 1};
   const CUresult r = tensor_map_encoder()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16*>(x), dims,
                                           strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -1580,11 +1824,6 @@ static float* ensure_part(NN& N, int64_t n, cudaStream_t s) {
   return N.part;
 }
 
-static unsigned conv_grid(const Image& im, int per_sm) {
-  const int64_t jobs = (int64_t)((im.W + TPX - 1) / TPX) * im.H;
-  return (unsigned)std::max<int64_t>(1, std::min<int64_t>(jobs, (int64_t)num_sms() * per_sm));
-}
-
 static int64_t npx_of(const Image& im) { return (int64_t)im.W * im.H; }
 
 static void pack(NN& N, cudaStream_t s, int64_t& nl) {
@@ -1592,8 +1831,9 @@ static void pack(NN& N, cudaStream_t s, int64_t& nl) {
   ++nl;
 }
 
-// out = N(in) over the stack; the activations stay for backward.  prof (may be
-// NULL): a solver timing the 32 -> 32 convolution launches.
+// out = N(in) over the stack (out NULL: only the activations that backward
+// reads, layer 6 is not needed).  prof (may be NULL): a solver timing the
+// 32 -> 32 convolution launches.
 static void forward(NN& N, const Image& im, const float2* in, float* out, cudaStream_t s, int64_t& nl,
                     Solver* prof = nullptr) {
   const int64_t npx = npx_of(im);
@@ -1615,8 +1855,11 @@ static void forward(NN& N, const Image& im, const float2* in, float* out, cudaSt
     if (prof) prof->prof_mark(s, false, PROF_CONV);
     if (own) EB_CUDA(cudaEventRecord(N.prof_ev[N.prof_n++].second, s));
   }
-  k_l6_fwd<<<blocks_for(npx, 128), 128, 0, s>>>(im, N.act[5], N.P, in, out);
-  nl += 6;
+  nl += 1 + NMID;
+  if (out) {
+    k_l6_fwd<<<blocks_for(npx, 128), 128, 0, s>>>(im, N.act[5], N.P, in, out);
+    nl += 1;
+  }
   EB_CUDA(cudaGetLastError());
 }
 
@@ -1682,39 +1925,34 @@ static void forward_infer(NN& N, const Image& im, const float2* in, float* out, 
   else forward(N, im, in, out, s, nl, prof);
 }
 
-// gradient of sum(dout * out) into N.G (forward ran on the same input)
+static void sum_parts(const float* part, int nparts, int n, int wm, float* out, cudaStream_t s) {
+  k_sum_parts<<<blocks_for(n, 32), SP_THREADS, 0, s>>>(part, nparts, n, wm, out);
+}
+
+// gradient of sum(dout * out) into N.G (the activations of a forward on the
+// same input are in N.act); N.out is overwritten
 static void backward(NN& N, const Image& im, const float2* in, const float* dout, cudaStream_t s, int64_t& nl) {
   const int64_t npx = npx_of(im);
-  const int nsm = num_sms();
-  {
-    const int nb = nsm * 4;
-    float* part = ensure_part(N, (int64_t)nb * (W6_N + B6_N), s);
-    k_l6_wgrad<<<nb, 256, 0, s>>>(im, dout, in, N.act[5], part);
-    k_sum_parts<<<blocks_for(W6_N + B6_N, 256), 256, 0, s>>>(part, nb, W6_N + B6_N, N.G + OFF_W6);
-    k_l6_bwd<<<blocks_for(npx, 128), 128, 0, s>>>(im, dout, in, N.act[5], N.P, N.gA);
-    nl += 3;
-  }
+  const int64_t tasks = (int64_t)((im.W + BW_RUN - 1) / BW_RUN) * im.H, per = BW_THREADS / 32;
+  const int nb = (int)std::max<int64_t>(1, std::min<int64_t>((tasks + per - 1) / per, (int64_t)num_sms() * BW_CTAS));
+  const int64_t jobs = (int64_t)((im.W + TPX - 1) / TPX) * ((im.R + WG_ROWS - 1) / WG_ROWS) * (im.H / im.R);
+  const int gw = (int)std::max<int64_t>(1, std::min<int64_t>(jobs, num_sms()));
+  float* part = ensure_part(N, std::max<int64_t>((int64_t)nb * (W1_N + B1_N), (int64_t)gw * WG_PART), s);
+  k_l6_gate<<<blocks_for(npx, 256), 256, 0, s>>>(npx, dout, in, N.out);
+  k_l6_back<<<nb, BW_THREADS, 0, s>>>(im, N.out, N.act[5], N.P, N.gA, part);
+  sum_parts(part, nb, W6_N + B6_N, 0, N.G + OFF_W6, s);
   bf16* cur = N.gA;
   bf16* nxt = N.gB;
   for (int l = NMID - 1; l >= 0; --l) {
-    const unsigned gw = conv_grid(im, 4);
-    const int nbb = nsm * 4;
-    float* part = ensure_part(N, std::max<int64_t>((int64_t)gw * WM_N, (int64_t)nbb * NC), s);
-    k_conv32_wgrad<<<gw, 128, wgrad_smem(), s>>>(im, N.act[l + 1], cur, part);
-    k_sum_wgrad<<<blocks_for(WM_N, 256), 256, 0, s>>>(part, (int)gw, N.G + off_wm(l));
-    k_bias_grad<<<nbb, 256, 0, s>>>(npx, cur, part);
-    k_sum_parts<<<1, 32, 0, s>>>(part, nbb, NC, N.G + off_wm(l) + WM_N);
+    k_conv32_wgrad<<<gw, WG_THREADS, WG_SMEM, s>>>(conv_map(N.act[l + 1], im, TC_PIX, WG_ROWS),
+                                                   conv_map(cur, im, TPX, WG_ROWS + 2), im, part, N.err);
+    sum_parts(part, gw, WG_PART, WM_N, N.G + off_wm(l), s);
     conv32(im, cur, N.wb + (int64_t)l * WM_N, nullptr, nxt, 0, N.act[l + 1], N.err, s);
     std::swap(cur, nxt);
-    nl += 5;
   }
-  {
-    const int nb = nsm * 4;
-    float* part = ensure_part(N, (int64_t)nb * (W1_N + B1_N), s);
-    k_l1_wgrad<<<nb, 256, 0, s>>>(im, cur, in, part);
-    k_sum_parts<<<blocks_for(W1_N + B1_N, 256), 256, 0, s>>>(part, nb, W1_N + B1_N, N.G + OFF_W1);
-    nl += 2;
-  }
+  k_l1_wgrad<<<nb, BW_THREADS, 0, s>>>(im, cur, in, part);
+  sum_parts(part, nb, W1_N + B1_N, 0, N.G + OFF_W1, s);
+  nl += 5 + 3 * NMID;
   EB_CUDA(cudaGetLastError());
 }
 
@@ -1973,7 +2211,7 @@ int nn_backward(nn_handle* h, int width, int height, int images, const float* in
     ensure_act(N, npx_of(im), stream);
     int64_t nl = 0;
     const float2* in = reinterpret_cast<const float2*>(in_dev);
-    forward(N, im, in, N.out, stream, nl);
+    forward(N, im, in, nullptr, stream, nl);
     backward(N, im, in, dout_dev, stream, nl);
   });
 }
