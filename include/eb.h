@@ -448,7 +448,11 @@ int wave_theta_step(const amg_handle* amg, double dt, double theta, double* u_pr
  * data).  On entry (u_prev, u_cur) = (u^{n-1}, u^n); on exit they hold
  * (u^{n+nsteps-1}, u^{n+nsteps}).  One kernel launch per step; whole chunks of
  * 32 steps run as one launch of a CUDA graph that the handle caches for these
- * fields, prec, dt and tile list (built on first use, which allocates).
+ * fields, prec, dt and tile list (built on first use, which allocates).  Two or
+ * more EB_F32 steps on a 2D grid with beta = 1 and the line-by-line closure run
+ * eight per launch, through a second pair of fields that the handle keeps from
+ * the first such call on (2 x num_nodes floats; calls of one handle on several
+ * streams then take turns); the results are the same.
  * prec: EB_F64 or EB_F32 element type of both fields.  Asynchronous on
  * stream; the fields must not be touched by other work until it completes. */
 int wave_step(const eb_handle* eb, int prec, double dt, void* u_prev_dev, void* u_cur_dev, int nsteps,

@@ -108,6 +108,16 @@ struct LeapfrogGraph {
   void release();
 };
 
+// what a handle keeps for several leapfrog steps per launch (eb_wave.cu); done
+// is created with the rest and recorded after each use
+struct WvTask;
+struct WavePlan {
+  cudaEvent_t done = nullptr;
+  float* buf = nullptr;  // second pair of fields
+  WvTask* task = nullptr;  // strips x chunks of rows that hold a CP
+  int* ntask = nullptr;
+};
+
 struct EBHandle {
   Geometry g;
   eb_levelset ls;
@@ -170,6 +180,7 @@ struct EBHandle {
   int32_t* cut_off = nullptr;    // [num_cp + 1] first cut of CP k
   cudaStream_t home = 0;
   mutable LeapfrogGraph lf_graph;
+  mutable WavePlan* wave = nullptr;
 };
 
 }  // namespace ebk
@@ -278,4 +289,10 @@ void run_tuner(int dim, const std::function<void(const TileDims&)>& retile, cons
                int reps, eb_tune_t* out, cudaStream_t s);
 template <class T>
 int launch_leapfrog(const EBHandle& eb, T* ua, T* ub, int nsteps, double dt, cudaStream_t s, bool use_graph);
+// nsteps >= 2 FP32 leapfrog steps of a 2D grid with beta = 1 and the
+// line-by-line closure, several per launch (eb_wave.cu); the fields hold 0 off
+// the CPs of the active tiles.  false: not done (the second pair of fields could
+// not be allocated), nothing was launched
+bool launch_leapfrog_blocked(const EBHandle& eb, float* ua, float* ub, int nsteps, float c2, cudaStream_t s);
+void wave_plan_free(WavePlan*& W, cudaStream_t s);
 }

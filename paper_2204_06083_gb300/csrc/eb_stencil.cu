@@ -154,7 +154,8 @@ template void launch_apply<__nv_bfloat16>(const EBHandle&, const __nv_bfloat16*,
 
 // -------------------------------------------------------------- leapfrog
 // One leapfrog step per launch: u_new = 2 u - u_old - dt^2 A u, u_new
-// overwriting u_old in place.  A launch boundary is the cheapest grid-wide
+// overwriting u_old in place (2D FP32 runs take eight per launch instead:
+// eb_wave.cu).  A launch boundary is the cheapest grid-wide
 // barrier on this part: a persistent cooperative kernel with a software grid
 // barrier between its steps measured 9.6-14.8 us per step at 4096^2 against
 // 8.3 us for one launch per step inside a CUDA graph.  512-thread CTAs sized
@@ -241,6 +242,14 @@ static unsigned leapfrog_grid(const EBHandle& eb, const void* fn) {
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)ps * num_sms()));
 }
 
+// whether s is being captured (an error of the query counts as yes)
+static bool is_capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+
 void LeapfrogGraph::release() {
   if (exec) cudaGraphExecDestroy(exec);
   exec = nullptr;
@@ -272,6 +281,16 @@ int launch_leapfrog(const EBHandle& eb, T* ua, T* ub, int nsteps, double dt, cud
       k_field_mask<T, 2><<<blocks, LF_THREADS, 0, s>>>(tv, code, ua, ub);
     else
       k_field_mask<T, 3><<<blocks, LF_THREADS, 0, s>>>(tv, code, ua, ub);
+  }
+  if constexpr (std::is_same<T, float>::value) {
+    // FP32 on a 2D grid: several steps per launch (eb_wave.cu).  Not for FP64,
+    // which the FP64 pipe bounds (recomputed halos cost more than the launches
+    // and passes they save: 90 against 47 us per step at 4096^2), nor for RBF
+    // closures (D_k > 0 tells the CPs there), nor during stream capture (the
+    // plan allocates and waits for its last use on another stream).
+    if (use_graph && G.dim == 2 && !eb.has_beta() && eb.closure == EB_CLOSURE_LINE && nsteps >= 2 && tv.pair_node &&
+        !is_capturing(s) && launch_leapfrog_blocked(eb, ua, ub, nsteps, c2, s))
+      return EB_OK;
   }
   int done = 0;
   if (use_graph && nsteps >= LeapfrogGraph::CHUNK) {
