@@ -787,7 +787,7 @@ __global__ void __launch_bounds__(SW_THREADS) k_spd_inverse(double* M, int n, do
       __syncthreads();
       double w = 0.0;
 #pragma unroll
-      for (int k = 0; k < SWB; ++k) w = fma(A[tr][k], B[k][tc], w);
+      for (int k = SWB - 1; k >= 0; --k) w = fma(A[tr][k], B[k][tc], w);
       Wg[i * SWB + tc] = w;
       Pg[i * SWB + tc] = pv;
       if (i < n && j < n) M[i >= j ? (int64_t)i * n + j : (int64_t)j * n + i] = w;

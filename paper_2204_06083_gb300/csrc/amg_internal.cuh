@@ -59,6 +59,7 @@ struct Hierarchy {
   double* coarse_inv = nullptr;  // FP64 inverse of the coarsest matrix
   int64_t nc = 0;
   MatrixFreeP mf;
+  double* cut_dinv = nullptr;    // FP64 V-cycle of a single grid: 1 / (sigma + D_k / h^2) at the cut CPs (full grid)
   VecSet<double> g64;            // level-0 grid vectors (full grid)
   VecSet<float> g32;
   VecSet<__nv_bfloat16> g16;

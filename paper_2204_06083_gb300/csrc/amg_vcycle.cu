@@ -32,16 +32,45 @@ struct CsrV {
   const V* v;
 };
 
-// operator constants in the arithmetic type of the kernel
+// operator constants in the arithmetic type of the kernel; dinv (FP64 V-cycles
+// of single grids): 1 / (sigma + D_k / h^2) of the CPs whose D_k is not 2 dim
 template <class A>
 struct GOp {
   A inv_h2, sigma, dinv_int;
+  const A* dinv = nullptr;
 };
 
 template <class A, class DT>
 __device__ __forceinline__ A inv_diag_t(uint32_t c, const DT* __restrict__ diag, int32_t node, const GOp<A>& o) {
   if (!(c & 0x7F)) return o.dinv_int;
+  // an FP64 division is some ten FP64 operations, run by the whole warp for one
+  // cut cell in it: the same value, formed once at setup
+  if (sizeof(A) == 8 && o.dinv) return __ldg(o.dinv + node);
   return (A)1 / (o.sigma + (A)__ldg(diag + node) * o.inv_h2);
+}
+
+// division by a constant whose correctly rounded reciprocal is known: FP64 by
+// Markstein's correction of the product (IBM J. Res. Dev. 34, 1990), which
+// gives the rounded quotient in three operations; FP32 by the product
+struct DivBy {
+  double d, inv;
+};
+__device__ __forceinline__ double div_by(double a, const DivBy& c) {
+  const double q = a * c.inv;
+  return fma(fma(-q, c.d, a), c.inv, q);
+}
+__device__ __forceinline__ float div_by(float a, const DivBy& c) { return a * (float)c.inv; }
+
+// the values of GOp<double>::dinv
+__global__ void __launch_bounds__(TILE_NODES) k_cut_dinv(PairList pl, const uint8_t* __restrict__ code,
+                                                         const double* __restrict__ diag, double sigma, double inv_h2,
+                                                         double* __restrict__ out) {
+  EB_LIST_LOOP(pl, node) {
+    uint32_t c0, c1;
+    ld_codes(code, node, c0, c1);
+    if ((c0 & CODE_CP) && (c0 & 0x7F)) out[node] = 1.0 / (sigma + diag[node] * inv_h2);
+    if ((c1 & CODE_CP) && (c1 & 0x7F)) out[node + 1] = 1.0 / (sigma + diag[node + 1] * inv_h2);
+  }
 }
 
 // per-tile shift of a batched view (unit spacing, sigma_g per geometry)
@@ -112,7 +141,7 @@ __global__ void __launch_bounds__(TILE_NODES) k_g_cheb_first(TileView tv, const 
                                                              GOp<typename AccOf<V>::type> o,
                                                              const double* __restrict__ r, V* __restrict__ b_out,
                                                              V* __restrict__ x, V* __restrict__ d,
-                                                             typename AccOf<V>::type theta) {
+                                                             DivBy theta) {
   using A = typename AccOf<V>::type;
   EB_SWEEP(DIM, tv, node) {
     const GOp<A> ot = sweep_op<DIM>(tv, tt_, o);
@@ -131,8 +160,8 @@ __global__ void __launch_bounds__(TILE_NODES) k_g_cheb_first(TileView tv, const 
     }
     const A b0 = (c0 & CODE_CP) ? r0 : (A)0, b1 = (c1 & CODE_CP) ? r1 : (A)0;
     if (b_out) st2o(b_out + node, b0, b1);
-    const A v0 = (c0 & CODE_CP) ? inv_diag_t<A>(c0, diag, node, ot) * b0 / theta : (A)0;
-    const A v1 = (c1 & CODE_CP) ? inv_diag_t<A>(c1, diag, node + 1, ot) * b1 / theta : (A)0;
+    const A v0 = (c0 & CODE_CP) ? div_by(inv_diag_t<A>(c0, diag, node, ot) * b0, theta) : (A)0;
+    const A v1 = (c1 & CODE_CP) ? div_by(inv_diag_t<A>(c1, diag, node + 1, ot) * b1, theta) : (A)0;
     st2o(x + node, v0, v1);
     st2o(d + node, v0, v1);
   }
@@ -149,22 +178,34 @@ __global__ void __launch_bounds__(TILE_NODES) k_update_first(PairList pl, PcgUpd
                                                              const typename DiagOf<V>::type* __restrict__ diag,
                                                              GOp<typename AccOf<V>::type> o, V* __restrict__ b_out,
                                                              V* __restrict__ x0, V* __restrict__ d,
-                                                             typename AccOf<V>::type theta) {
+                                                             DivBy theta) {
   using A = typename AccOf<V>::type;
-  __shared__ double sm[32];
+  __shared__ double sm[TILE_NODES];
   __shared__ double s_alpha;
   if (cta_done(u.sc)) {
     if (threadIdx.x == 0) u.rr_part[blockIdx.x] = 0.0;
     return;
+  }
+  double* const x = u.sc->x;
+  // this thread's first pair on its way into L1 during the partial sums
+  const int64_t l0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (l0 < pl.n) {
+    const int32_t nd = __ldg(pl.node + l0);
+    prefetch_l1(u.r + nd);
+    prefetch_l1(u.q + nd);
+    prefetch_l1(u.p + nd);
+    prefetch_l1(x + nd);
+    prefetch_l1(code + nd);
+    if (u.rzo_part) prefetch_l1(u.z + nd);
   }
   const double alpha = pcg_alpha(u.sc, u.pq_part, u.nblk, sm, &s_alpha);
   const double ax = alpha * u.h2;  // q holds h^2 (sigma I + A) p
   double srr = 0.0, srzo = 0.0;
   EB_LIST_LOOP(pl, node) {
     const Two<double> rv = ld2d(u.r + node), qv = LdRO::ld2(u.q + node), pv = LdRO::ld2(u.p + node),
-                      xv = ld2d(u.x + node);
+                      xv = ld2d(x + node);
     const double r0 = rv.x - alpha * qv.x, r1 = rv.y - alpha * qv.y;
-    st2(u.x + node, xv.x + ax * pv.x, xv.y + ax * pv.y);
+    st2(x + node, xv.x + ax * pv.x, xv.y + ax * pv.y);
     st2(u.r + node, r0, r1);
     srr += r0 * r0 + r1 * r1;
     if (u.rzo_part) {
@@ -176,8 +217,8 @@ __global__ void __launch_bounds__(TILE_NODES) k_update_first(PairList pl, PcgUpd
     ld_codes(code, node, c0, c1);
     const A b0 = (c0 & CODE_CP) ? (A)r0 : (A)0, b1 = (c1 & CODE_CP) ? (A)r1 : (A)0;
     if (b_out) st2o(b_out + node, b0, b1);
-    const A v0 = (c0 & CODE_CP) ? inv_diag_t<A>(c0, diag, node, ot) * b0 / theta : (A)0;
-    const A v1 = (c1 & CODE_CP) ? inv_diag_t<A>(c1, diag, node + 1, ot) * b1 / theta : (A)0;
+    const A v0 = (c0 & CODE_CP) ? div_by(inv_diag_t<A>(c0, diag, node, ot) * b0, theta) : (A)0;
+    const A v1 = (c1 & CODE_CP) ? div_by(inv_diag_t<A>(c1, diag, node + 1, ot) * b1, theta) : (A)0;
     st2o(x0 + node, v0, v1);
     st2o(d + node, v0, v1);
   }
@@ -201,11 +242,12 @@ struct UfIn {
   uint32_t c0, c1;
 };
 
-__device__ __forceinline__ void uf_load(UfIn& in, const PcgUpdate& u, const uint8_t* code, int32_t node) {
+__device__ __forceinline__ void uf_load(UfIn& in, const PcgUpdate& u, const double* x, const uint8_t* code,
+                                        int32_t node) {
   df_ld2_rw(u.r, node, in.r0, in.r1);
   df_ld2(u.q, node, in.q0, in.q1);
   df_ld2(u.p, node, in.p0, in.p1);
-  df_ld2_rw(u.x, node, in.xa, in.xb);
+  df_ld2_rw(x, node, in.xa, in.xb);
   in.zv = u.rzo_part ? __ldg(reinterpret_cast<const float2*>(reinterpret_cast<const float*>(u.z) + node))
                      : make_float2(0.0f, 0.0f);
   ld_codes(code, node, in.c0, in.c1);
@@ -234,9 +276,10 @@ __global__ void __launch_bounds__(TILE_NODES) k_update_first_df(PairList pl, Pcg
   }
   const int64_t step = (int64_t)gridDim.x * blockDim.x;
   int64_t li = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  double* const x = u.sc->x;
   UfIn in;
   int32_t node = li < pl.n ? __ldg(pl.node + li) : 0;
-  if (li < pl.n) uf_load(in, u, code, node);
+  if (li < pl.n) uf_load(in, u, x, code, node);
   // alpha from the DF p'q partials (FP64 scalars), split into DF once per CTA
   const double pq = df_sum_parts(u.pq_part, u.nblk, dsm);
   if (threadIdx.x == 0) {
@@ -252,7 +295,7 @@ __global__ void __launch_bounds__(TILE_NODES) k_update_first_df(PairList pl, Pcg
     const int32_t nnode = ln < pl.n ? __ldg(pl.node + ln) : 0;
     // the residual update cancels by design: the accurate DF sum
     const DF r0 = df_sub(in.r0, df_mul(a_df, in.q0)), r1 = df_sub(in.r1, df_mul(a_df, in.q1));
-    df_st2(u.x, node, df_add_fast(in.xa, df_mul(ax_df, in.p0)), df_add_fast(in.xb, df_mul(ax_df, in.p1)));
+    df_st2(x, node, df_add_fast(in.xa, df_mul(ax_df, in.p0)), df_add_fast(in.xb, df_mul(ax_df, in.p1)));
     df_st2(u.r, node, r0, r1);
     df_acc_prod(srr, r0, r0);
     df_acc_prod(srr, r1, r1);
@@ -267,7 +310,7 @@ __global__ void __launch_bounds__(TILE_NODES) k_update_first_df(PairList pl, Pcg
     const float v1 = (c1 & CODE_CP) ? inv_diag_t<float>(c1, diag, node + 1, o) * b1 * inv_theta : 0.0f;
     st2o(x0 + node, v0, v1);
     st2o(d + node, v0, v1);
-    if (ln < pl.n) uf_load(in, u, code, nnode);
+    if (ln < pl.n) uf_load(in, u, x, code, nnode);
     li = ln;
     node = nnode;
   }
@@ -326,7 +369,7 @@ __global__ void __launch_bounds__(TILE_NODES) k_g_cheb_step(TileView tv, const u
     }
   }
   if constexpr (DOT == 1) {
-    __shared__ double sm[32];
+    __shared__ double sm[TILE_NODES];
     const double a = block_sum(srz, sm);
     if (threadIdx.x == 0) part[blockIdx.x] = a;
   } else if constexpr (DOT == 2) {
@@ -562,7 +605,7 @@ struct CoarseFirst {
   const V* dinv = nullptr;
   V* x = nullptr;
   V* d = nullptr;
-  typename AccOf<V>::type theta = 1;
+  DivBy theta{1.0, 1.0};
 };
 
 template <class V>
@@ -571,7 +614,7 @@ __device__ __forceinline__ void store_restricted(V* out, int64_t i, typename Acc
   const V b = cvt<V>(s);
   out[i] = b;
   if (f.dinv) {
-    const V v = cvt<V>(cvt<A>(f.dinv[i]) * cvt<A>(b) / f.theta);
+    const V v = cvt<V>(div_by((A)(cvt<A>(f.dinv[i]) * cvt<A>(b)), f.theta));
     f.x[i] = v;
     f.d[i] = v;
   }
@@ -743,16 +786,36 @@ inline int group_width(int64_t nnz, int64_t n, int epl) {
     }                                                                                            \
   } while (0)
 
-// x = M b with M the FP64 inverse (row-major); one warp per row
+// x = M b with M the FP64 inverse (row-major); one warp per row, four rows per
+// CTA, so that a few hundred rows reach every SM's schedulers (0.4 FP64 lanes
+// per clock each).  A reduced-precision b is widened once per CTA: a conversion
+// costs as much as an FP64 multiply-add.  515 rows, FP32 b: 4.6 -> 3.0 us.
+constexpr int GV_WARPS = 4;
+constexpr int GV_CHUNK = 1024;
 template <class V>
-__global__ void k_dense_gemv(const double* __restrict__ M, int64_t n, const V* __restrict__ b, V* __restrict__ x) {
-  const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+__global__ void __launch_bounds__(32 * GV_WARPS) k_dense_gemv(const double* __restrict__ M, int64_t n,
+                                                              const V* __restrict__ b, V* __restrict__ x) {
   const int lane = threadIdx.x & 31;
-  if (row >= n) return;
-  double s = 0.0;
-  for (int64_t j = lane; j < n; j += 32) s += M[row * n + j] * cvt<double>(b[j]);
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) x[row] = cvt<V>(s);
+  const int64_t row = (int64_t)blockIdx.x * GV_WARPS + (threadIdx.x >> 5);
+  const double* Mr = M + (row < n ? row : 0) * n;
+  double t = 0.0;
+  if constexpr (std::is_same<V, double>::value) {
+#pragma unroll 4
+    for (int64_t j = lane; j < n; j += 32) t += Mr[j] * b[j];
+  } else {
+    __shared__ double sb[GV_CHUNK];
+    for (int64_t j = 16 * lane; j < min(n, (int64_t)GV_CHUNK); j += 512) prefetch_l1(Mr + j);
+    for (int64_t c = 0; c < n; c += GV_CHUNK) {
+      const int m = (int)min((int64_t)GV_CHUNK, n - c);
+      __syncthreads();
+      for (int j = threadIdx.x; j < m; j += 32 * GV_WARPS) sb[j] = cvt<double>(b[c + j]);
+      __syncthreads();
+#pragma unroll 4
+      for (int j = lane; j < m; j += 32) t += Mr[c + j] * sb[j];
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if (lane == 0 && row < n) x[row] = cvt<V>(t);
 }
 
 template <class V>
@@ -846,7 +909,8 @@ static CoarseFirst<V> coarse_first(Solver& S, size_t l) {
   f.dinv = LV::dinv(L);
   f.x = v.x;
   f.d = v.d;
-  f.theta = (typename AccOf<V>::type)cheb_coef(L.rho, S.opts.cheb_degree).theta;
+  const double theta = cheb_coef(L.rho, S.opts.cheb_degree).theta;
+  f.theta = DivBy{theta, 1.0 / theta};
   return f;
 }
 
@@ -864,7 +928,7 @@ static void vcycle_compact(Solver& S, size_t l, cudaStream_t s, bool warm = fals
   const int64_t n = L.A.n;
   if (l + 1 == H.L.size()) {
     S.nlaunch += 1;
-    k_dense_gemv<V><<<blocks_for(n * 32, 256), 256, 0, s>>>(H.coarse_inv, n, v.b, v.x);
+    k_dense_gemv<V><<<blocks_for(n, GV_WARPS), 32 * GV_WARPS, 0, s>>>(H.coarse_inv, n, v.b, v.x);
     return;
   }
   const ChebCoef cc = cheb_coef(L.rho, S.opts.cheb_degree);
@@ -893,6 +957,15 @@ static void vcycle_compact(Solver& S, size_t l, cudaStream_t s, bool warm = fals
     if (mark) S.prof_mark(s, false, PROF_LEVEL1);
     std::swap(v.x, v.x2);
   }
+}
+
+template <class A>
+static GOp<A> grid_op(const Solver& S) {
+  const Geometry& G = S.eb->g;
+  const double inv_h2 = 1.0 / (G.h * G.h);
+  GOp<A> o{(A)inv_h2, (A)S.shift, (A)(1.0 / (S.shift + 2.0 * G.dim * inv_h2))};
+  if constexpr (std::is_same<A, double>::value) o.dinv = S.H->cut_dinv;
+  return o;
 }
 
 // tensor map of a 2D grid array (S columns x R rows, element size es) with boxes of bw x bh
@@ -954,7 +1027,7 @@ static int vcycle_grid(Solver& S, const double* r, double* z, cudaStream_t s, co
     const int64_t n = L0.A.n;
     EB_CUDA(cudaMemsetAsync(z, 0, sizeof(double) * G.num_nodes, s));
     k_gather_cp<V><<<blocks_for(n, 256), 256, 0, s>>>(n, eb.cp_node, r, v.b);
-    k_dense_gemv<V><<<blocks_for(n * 32, 256), 256, 0, s>>>(H.coarse_inv, n, v.b, v.x);
+    k_dense_gemv<V><<<blocks_for(n, GV_WARPS), 32 * GV_WARPS, 0, s>>>(H.coarse_inv, n, v.b, v.x);
     k_scatter_cp<V><<<blocks_for(n, 256), 256, 0, s>>>(n, eb.cp_node, v.x, z);
     EB_CUDA(cudaGetLastError());
     S.nlaunch += 3;
@@ -962,14 +1035,18 @@ static int vcycle_grid(Solver& S, const double* r, double* z, cudaStream_t s, co
   }
   const double inv_h2 = 1.0 / (G.h * G.h);
   const unsigned gb = tile_grid(eb);
-  // list sweeps: one CP pair per thread (the partial-forming launch keeps the
-  // fixed grid gb, whose CTA count is the number of partials)
+  // list sweeps: one CP pair per thread (the partial-forming launch at most
+  // four CTAs per SM)
   constexpr bool LIST = (DIM & DIM_LIST) != 0;
-  const unsigned gl = LIST ? blocks_for(eb.num_pairs, TILE_NODES) : gb;
+  const int th = LIST ? list_threads(eb.num_pairs) : TILE_NODES;
+  const unsigned gl = LIST ? blocks_for(eb.num_pairs, th) : gb;
+  // the launch that forms the r'z partials: DF sums are cheap to repeat, and
+  // that step runs faster on eight CTAs per SM (256^3: 10.3 against 12.5 us)
+  const unsigned gd = LIST ? (unsigned)list_blocks(eb, dot && dot->df ? 8 : 4) : gb;
   const ChebCoef cc = cheb_coef(L0.rho, S.opts.cheb_degree);
   const TileView tv = eb.tv();
   using A = typename AccOf<V>::type;
-  const GOp<A> o{(A)inv_h2, (A)S.shift, (A)(1.0 / (S.shift + 2.0 * G.dim * inv_h2))};
+  const GOp<A> o = grid_op<A>(S);
   const typename DiagOf<V>::type* diag = diag_of<V>(eb);
   S.nlaunch += 3 + 2 * cc.deg;
   VecSet<V>& g = LV::grid(H);
@@ -982,9 +1059,9 @@ static int vcycle_grid(Solver& S, const double* r, double* z, cudaStream_t s, co
   if (first_done)
     S.nlaunch -= 1;  // amg_update_first did it
   else if (rdf)
-    k_g_cheb_first<DIM, V, true><<<gl, TILE_NODES, 0, s>>>(tv, eb.code, diag, o, r, bcopy, x, g.d, (A)cc.theta);
+    k_g_cheb_first<DIM, V, true><<<gl, th, 0, s>>>(tv, eb.code, diag, o, r, bcopy, x, g.d, DivBy{cc.theta, 1.0 / cc.theta});
   else
-    k_g_cheb_first<DIM, V><<<gl, TILE_NODES, 0, s>>>(tv, eb.code, diag, o, r, bcopy, x, g.d, (A)cc.theta);
+    k_g_cheb_first<DIM, V><<<gl, th, 0, s>>>(tv, eb.code, diag, o, r, bcopy, x, g.d, DivBy{cc.theta, 1.0 / cc.theta});
   // the tensor-copy step (batched 2D views, FP32 storage) or the sweep kernel
   auto step = [&](const V* xin, V* xout, int k) {
     if constexpr (std::is_same<V, float>::value && (DIM & (DIM_VB | DIM_LIST)) == 0 && dim_of(DIM) == 2) {
@@ -993,7 +1070,7 @@ static int vcycle_grid(Solver& S, const double* r, double* z, cudaStream_t s, co
         return;
       }
     }
-    k_g_cheb_step<DIM, V, V><<<gl, TILE_NODES, 0, s>>>(tv, eb.code, diag, o, b, xin, xout, g.d, (A)cc.c1[k],
+    k_g_cheb_step<DIM, V, V><<<gl, th, 0, s>>>(tv, eb.code, diag, o, b, xin, xout, g.d, (A)cc.c1[k],
                                                        (A)cc.c2[k]);
   };
   for (int k = 1; k < cc.deg; ++k) {
@@ -1002,7 +1079,7 @@ static int vcycle_grid(Solver& S, const double* r, double* z, cudaStream_t s, co
     S.prof_mark(s, false);
     std::swap(x, x2);
   }
-  k_g_resid<DIM, V><<<gl, TILE_NODES, 0, s>>>(tv, eb.code, diag, o, b, x, g.r);
+  k_g_resid<DIM, V><<<gl, th, 0, s>>>(tv, eb.code, diag, o, b, x, g.r);
   Level& C = H.L[1];
   VecSet<V>& cv = LV::vec(C);
   const CsrV<V> R0 = LV::R(L0), P0 = LV::P(L0);
@@ -1017,7 +1094,7 @@ static int vcycle_grid(Solver& S, const double* r, double* z, cudaStream_t s, co
   vcycle_compact<V>(S, 1, s);
   if (S.opts.cycle == 2 && H.L.size() > 2) vcycle_compact<V>(S, 1, s, true);  // W-cycle
   if (M.on)
-    k_prolong_mf<DIM, V, SC><<<gl, TILE_NODES, 0, s>>>(tv, eb.code, diag, o, (A)M.omega, M.agg_node, sc, cv.x, x);
+    k_prolong_mf<DIM, V, SC><<<gl, th, 0, s>>>(tv, eb.code, diag, o, (A)M.omega, M.agg_node, sc, cv.x, x);
   else
     EB_GROUP_LAUNCH(gP, k_prolong0, V, P0.n, s, P0.n, P0.rp, P0.ci, P0.v, eb.cp_node, cv.x, x);
   for (int k = 0; k < cc.deg; ++k) {
@@ -1026,14 +1103,14 @@ static int vcycle_grid(Solver& S, const double* r, double* z, cudaStream_t s, co
     const bool mark = !(k == cc.deg - 1 && dot);
     if (mark) S.prof_mark(s, true);
     if (k == cc.deg - 1 && rdf && dot->part)  // z in FP32 for the DF outer iteration, with the r'z partials
-      k_g_cheb_step<DIM, V, float, 2><<<gb, TILE_NODES, 0, s>>>(tv, eb.code, diag, o, b, x,
+      k_g_cheb_step<DIM, V, float, 2><<<gd, th, 0, s>>>(tv, eb.code, diag, o, b, x,
                                                                 reinterpret_cast<float*>(z), g.d, (A)cc.c1[k],
                                                                 (A)cc.c2[k], dot->r, dot->part);
     else if (k == cc.deg - 1 && rdf)  // z in FP32 on every node of the active tiles, 0 off the CPs
       k_g_cheb_step<(DIM & ~DIM_LIST), V, float><<<gb, TILE_NODES, 0, s>>>(
           tiles_only(tv), eb.code, diag, o, b, x, reinterpret_cast<float*>(z), g.d, (A)cc.c1[k], (A)cc.c2[k]);
     else if (k == cc.deg - 1 && dot)
-      k_g_cheb_step<DIM, V, double, 1><<<gb, TILE_NODES, 0, s>>>(tv, eb.code, diag, o, b, x, z, g.d, (A)cc.c1[k],
+      k_g_cheb_step<DIM, V, double, 1><<<gd, th, 0, s>>>(tv, eb.code, diag, o, b, x, z, g.d, (A)cc.c1[k],
                                                                  (A)cc.c2[k], dot->r, dot->part);
     else if (k == cc.deg - 1)  // z for a caller (amg_vcycle): every node of the active tiles, 0 off the CPs
       k_g_cheb_step<(DIM & ~DIM_LIST), V, double>
@@ -1046,7 +1123,7 @@ static int vcycle_grid(Solver& S, const double* r, double* z, cudaStream_t s, co
   g.x = x;
   g.x2 = x2;
   EB_CUDA(cudaGetLastError());
-  return (dot && dot->part) ? (int)gb : 0;
+  return (dot && dot->part) ? (int)gd : 0;
 }
 
 int amg_vcycle_grid(Solver& S, const double* r, double* z, cudaStream_t s, const VcycleDot* dot, bool first_done) {
@@ -1076,18 +1153,18 @@ static void update_first(Solver& S, const PcgUpdate& u, cudaStream_t s) {
   const Geometry& G = eb.g;
   const double inv_h2 = 1.0 / (G.h * G.h);
   const ChebCoef cc = cheb_coef(H.L[0].rho, S.opts.cheb_degree);
-  const GOp<A> o{(A)inv_h2, (A)S.shift, (A)(1.0 / (S.shift + 2.0 * G.dim * inv_h2))};
+  const GOp<A> o = grid_op<A>(S);
   VecSet<V>& g = LV::grid(H);
   V* bcopy = std::is_same<V, double>::value ? nullptr : g.b;
   if constexpr (!std::is_same<V, double>::value) {
     if (u.df) {
-      k_update_first_df<DIM, V><<<(unsigned)u.nblk, TILE_NODES, 0, s>>>(eb.pairs(), u, eb.code, diag_of<V>(eb), o,
+      k_update_first_df<DIM, V><<<(unsigned)u.nblk, S.iter_threads(), 0, s>>>(eb.pairs(), u, eb.code, diag_of<V>(eb), o,
                                                                         bcopy, g.x, g.d, (float)(1.0 / cc.theta));
       return;
     }
   }
-  k_update_first<DIM, V><<<(unsigned)u.nblk, TILE_NODES, 0, s>>>(eb.pairs(), u, eb.code, diag_of<V>(eb), o, bcopy,
-                                                                 g.x, g.d, (A)cc.theta);
+  k_update_first<DIM, V><<<(unsigned)u.nblk, S.iter_threads(), 0, s>>>(eb.pairs(), u, eb.code, diag_of<V>(eb), o, bcopy,
+                                                                 g.x, g.d, DivBy{cc.theta, 1.0 / cc.theta});
 }
 
 int amg_levels(const Solver& S) { return S.H ? (int)S.H->L.size() : 0; }
@@ -1162,6 +1239,12 @@ void amg_alloc_vcycle(Solver& S, cudaStream_t s) {
     }
   } else {
     alloc_set(H.g64, nn, false, s);
+    const EBHandle& eb = *S.eb;
+    if (eb.pair_node && H.L.size() > 1) {
+      H.cut_dinv = dalloc<double>(nn, s, false);
+      k_cut_dinv<<<list_blocks(eb), list_threads(eb.num_pairs), 0, s>>>(eb.pairs(), eb.code, eb.diag, S.shift,
+                                                                        1.0 / (eb.g.h * eb.g.h), H.cut_dinv);
+    }
     for (size_t l = first; l < H.L.size(); ++l) alloc_set(H.L[l].v64, H.L[l].A.n, true, s);
   }
   EB_CUDA(cudaGetLastError());
@@ -1171,6 +1254,7 @@ void amg_free_vcycle(Hierarchy& H, cudaStream_t s) {
   free_set(H.g64, s);
   free_set(H.g32, s);
   free_set(H.g16, s);
+  dfree(H.cut_dinv, s);
   for (Level& L : H.L) {
     free_set(L.v64, s);
     free_set(L.v32, s);
@@ -1212,12 +1296,12 @@ static void smoother_step(Solver& S, int level, cudaStream_t s) {
     const EBHandle& eb = *S.eb;
     const Geometry& G = eb.g;
     const double inv_h2 = 1.0 / (G.h * G.h);
-    const GOp<A> o{(A)inv_h2, (A)S.shift, (A)(1.0 / (S.shift + 2.0 * G.dim * inv_h2))};
+    const GOp<A> o = grid_op<A>(S);
     VecSet<V>& g = LV::grid(H);
     const V* b = std::is_same<V, double>::value ? reinterpret_cast<const V*>(S.r) : g.b;
     dim_dispatch(eb, [&](auto D) {
       if (eb.pair_node)
-        k_g_cheb_step<D.value | DIM_LIST, V, V><<<blocks_for(eb.num_pairs, TILE_NODES), TILE_NODES, 0, s>>>(
+        k_g_cheb_step<D.value | DIM_LIST, V, V><<<blocks_for(eb.num_pairs, list_threads(eb.num_pairs)), list_threads(eb.num_pairs), 0, s>>>(
             eb.tv(), eb.code, diag_of<V>(eb), o, b, g.x, g.x2, g.d, (A)cc.c1[k], (A)cc.c2[k]);
       else
         k_g_cheb_step<D.value, V, V><<<tile_grid(eb), TILE_NODES, 0, s>>>(eb.tv(), eb.code, diag_of<V>(eb), o, b,

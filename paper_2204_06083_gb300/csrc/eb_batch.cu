@@ -56,8 +56,6 @@ struct Batch {
   cudaStream_t home = 0;
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t gexec = nullptr;
-  const double* g_b = nullptr;
-  double* g_x = nullptr;
   int64_t g_launches = 0, nlaunch = 0;
   // event timing of the level-0 smoother launches inside the captured iteration
   bool profile = false;
@@ -74,8 +72,6 @@ struct Batch {
   int g_df = -1, l_df = -1;
   // the whole loop on the device (conditional WHILE node) when not profiling
   cudaGraphExec_t lexec = nullptr;
-  const double* l_b = nullptr;
-  double* l_x = nullptr;
   int64_t l_launches = 0;
   int ngeo() const { return (int)geo.size(); }
 };
@@ -211,8 +207,6 @@ static void batch_tiles(Batch& B, cudaStream_t s) {
   B.gexec = nullptr;
   if (B.lexec) cudaGraphExecDestroy(B.lexec);
   B.lexec = nullptr;
-  B.l_b = nullptr;
-  B.l_x = nullptr;
   dfree(V.tile_base, s); dfree(V.tile_lim, s); dfree(V.tile_shift64, s); dfree(V.tile_shift32, s);
   dfree(B.tile_geo, s); dfree(B.geo_tile0, s); dfree(B.part, s);
   V.num_tiles = 0;
@@ -396,9 +390,10 @@ __global__ void __launch_bounds__(BT) k_b_xpby_apply(TileView tv, const int32_t*
 // CG), r.z for the new r and the z still in place (the r.zold term of the
 // Polak-Ribiere beta), as pairs; without z, single r.r partials
 __global__ void __launch_bounds__(BT) k_b_update_xr(TileView tv, const int32_t* tile_geo, const PcgScalars* sc,
-                                                    double* x, double* r, const double* p, const double* q,
+                                                    double* r, const double* p, const double* q,
                                                     const double* z, double* part) {
   __shared__ double sm[BT / 32];
+  double* const x = sc->x;
   for (int64_t tt = blockIdx.x; tt < tv.ntiles; tt += gridDim.x) {
     const PcgScalars& S = sc[tile_geo[tt]];
     if (S.done) continue;
@@ -497,10 +492,11 @@ __global__ void __launch_bounds__(BT) k_b_heat_rhs(TileView tv, const int32_t* t
 // x += alpha p, r -= alpha q in DF; per-tile DF partials r.r and, with z
 // (flexible CG), r.zold as pairs, else r.r alone (k_b_update_xr's layout)
 __global__ void __launch_bounds__(BT) k_b_update_xr_df(TileView tv, const int32_t* tile_geo, const PcgScalars* sc,
-                                                       double* x, double* r, const double* p, const double* q,
+                                                       double* r, const double* p, const double* q,
                                                        const float* z, double* part) {
   __shared__ DF dsm[BT / 32];
   __shared__ DF s_a;
+  double* const x = sc->x;
   for (int64_t tt = blockIdx.x; tt < tv.ntiles; tt += gridDim.x) {
     const PcgScalars& S = sc[tile_geo[tt]];
     if (S.done) continue;
@@ -822,25 +818,25 @@ static void b_xpby_apply(Batch& B, int first, cudaStream_t s) {
 // One batched iteration: alpha from the p.q partials of the previous
 // k_b_xpby_apply, the x/r update (with r.zold when flexible), r.r and the
 // convergence test, the V-cycle and r.z, beta, then p and the next q.
-static void b_iteration(Batch& B, double* x, bool flex, cudaStream_t s) {
+static void b_iteration(Batch& B, bool flex, cudaStream_t s) {
   Solver& S = *B.S;
   const TileView tv = B.view.tv();
   const unsigned gb = bgrid(B);
   ++B.nlaunch;
   b_finalize(B, FIN_ALPHA, s);
   if (B.df)
-    k_b_update_xr_df<<<gb, BT, 0, s>>>(tv, B.tile_geo, B.sc, x, S.r, S.p, S.q,
+    k_b_update_xr_df<<<gb, BT, 0, s>>>(tv, B.tile_geo, B.sc, S.r, S.p, S.q,
                                        flex ? reinterpret_cast<const float*>(S.z) : nullptr, B.part);
   else
-    k_b_update_xr<<<gb, BT, 0, s>>>(tv, B.tile_geo, B.sc, x, S.r, S.p, S.q, flex ? S.z : nullptr, B.part);
+    k_b_update_xr<<<gb, BT, 0, s>>>(tv, B.tile_geo, B.sc, S.r, S.p, S.q, flex ? S.z : nullptr, B.part);
   b_finalize(B, flex ? FIN_RRF : FIN_RR, s);
   b_precondition(B, S.r, S.z, s);
   b_finalize(B, flex ? FIN_BETAF : FIN_BETA, s);
   b_xpby_apply(B, 0, s);
 }
 
-static void b_graph_prepare(Batch& B, const double* b, double* x, bool flex, cudaStream_t s) {
-  if (B.gexec && B.g_b == b && B.g_x == x && B.g_prof == (int)B.profile && B.g_df == (int)B.df) return;
+static void b_graph_prepare(Batch& B, bool flex, cudaStream_t s) {
+  if (B.gexec && B.g_prof == (int)B.profile && B.g_df == (int)B.df) return;
   Solver& S = *B.S;
   if (B.gexec) cudaGraphExecDestroy(B.gexec);
   B.gexec = nullptr;
@@ -854,7 +850,7 @@ static void b_graph_prepare(Batch& B, const double* b, double* x, bool flex, cud
   S.prof_on = B.profile;
   S.prof_n = 0;
   EB_CUDA(cudaStreamBeginCapture(B.cap_stream, cudaStreamCaptureModeThreadLocal));
-  b_iteration(B, x, flex, B.cap_stream);
+  b_iteration(B, flex, B.cap_stream);
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamEndCapture(B.cap_stream, &graph);
   S.prof_on = false;
@@ -867,8 +863,6 @@ static void b_graph_prepare(Batch& B, const double* b, double* x, bool flex, cud
   EB_CUDA(e);
   B.g_launches = B.nlaunch - n0;
   B.nlaunch = n0;
-  B.g_b = b;
-  B.g_x = x;
   B.g_df = (int)B.df;
 }
 
@@ -883,24 +877,20 @@ __global__ void k_b_loop_cond(cudaGraphConditionalHandle h, const PcgScalars* sc
 static void b_loop_release(Batch& B) {
   if (B.lexec) cudaGraphExecDestroy(B.lexec);
   B.lexec = nullptr;
-  B.l_b = nullptr;
-  B.l_x = nullptr;
 }
 
-static void b_loop_prepare(Batch& B, const double* b, double* x, bool flex) {
-  if (B.lexec && B.l_b == b && B.l_x == x && B.l_df == (int)B.df) return;
+static void b_loop_prepare(Batch& B, bool flex) {
+  if (B.lexec && B.l_df == (int)B.df) return;
   b_loop_release(B);
   if (!B.cap_stream) EB_CUDA(cudaStreamCreateWithFlags(&B.cap_stream, cudaStreamNonBlocking));
   const int64_t n0 = B.nlaunch;
   B.lexec = build_while_graph(B.cap_stream, [&](cudaStream_t cs, cudaGraphConditionalHandle h) {
-    b_iteration(B, x, flex, cs);
+    b_iteration(B, flex, cs);
     k_b_loop_cond<<<1, 256, 0, cs>>>(h, B.sc, B.ngeo());
     ++B.nlaunch;
   });
   B.l_launches = B.nlaunch - n0;
   B.nlaunch = n0;
-  B.l_b = b;
-  B.l_x = x;
   B.l_df = (int)B.df;
 }
 
@@ -932,6 +922,7 @@ static int batch_pcg(Batch& B, const double* b, double* x, double rtol, int maxi
   for (auto& p : init) {
     p = PcgScalars{};
     p.tol2 = rtol * rtol;
+    p.x = xi;
   }
   std::vector<int> iters(ng, 0), flags(ng, 0), conv(ng, 0);
   std::vector<double> rel(ng, 0.0);
@@ -971,7 +962,7 @@ static int batch_pcg(Batch& B, const double* b, double* x, double rtol, int maxi
       b_xpby_apply(B, 1, s);
       int it = 0;
       if (!B.profile) {  // the whole loop on the device
-        b_loop_prepare(B, b, xi, flex);
+        b_loop_prepare(B, flex);
         EB_CUDA(cudaGraphLaunch(B.lexec, s));
         EB_CUDA(cudaMemcpyAsync(B.sc_host, B.sc, sizeof(PcgScalars) * ng, cudaMemcpyDeviceToHost, s));
         EB_CUDA(cudaStreamSynchronize(s));
@@ -982,7 +973,7 @@ static int batch_pcg(Batch& B, const double* b, double* x, double rtol, int maxi
       }
       while (true) {
         if (its + it >= maxit) break;
-        b_graph_prepare(B, b, xi, flex, s);
+        b_graph_prepare(B, flex, s);
         EB_CUDA(cudaGraphLaunch(B.gexec, s));
         B.nlaunch += B.g_launches;
         ++it;
@@ -1144,7 +1135,7 @@ int batch_rhs(const batch_handle* b, const double* f_all, const double* ug_all, 
 // summation order: deterministic)
 __global__ void __launch_bounds__(256) k_b_wsum(const int64_t* node_off, const int32_t* n0, const int32_t* n1,
                                                 int64_t stride, const double* w, const double* u, double* out) {
-  __shared__ double sm[32];
+  __shared__ double sm[256];
   const int g = blockIdx.x;
   const int64_t base = node_off[g];
   const int64_t nx = n0[g], cnt = nx * n1[g];

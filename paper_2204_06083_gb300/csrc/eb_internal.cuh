@@ -5,6 +5,7 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <functional>
 #include <string>
@@ -260,6 +261,20 @@ inline int num_sms() {
 inline unsigned tile_grid(const EBHandle& eb, int per_sm = 8) {
   int64_t b = eb.num_tiles < (int64_t)num_sms() * per_sm ? eb.num_tiles : (int64_t)num_sms() * per_sm;
   return (unsigned)(b < 1 ? 1 : b);
+}
+
+inline unsigned blocks_for(int64_t n, int threads);
+
+// Threads per CTA of a kernel that takes the CP pair list one pair per thread:
+// small CTAs while they all fit on the GPU at once, so that a small grid's FP64
+// work spreads over every SM's schedulers (128^2: 1,500 pairs are 24 CTAs of 64
+// threads, not 6 of 256; one FP64 Chebyshev step 4.4 -> 2.4 us)
+inline int list_threads(int64_t pairs) { return pairs < (int64_t)num_sms() * 256 ? 64 : 256; }
+// CTAs of the list kernels that form reduction partials: at most four per SM
+// (every CTA of the next launch sums the partials again)
+inline int list_blocks(const EBHandle& eb, int per_sm = 4) {
+  const int t = list_threads(eb.num_pairs);
+  return (int)std::max<int64_t>(1, std::min<int64_t>((eb.num_pairs + t - 1) / t, (int64_t)num_sms() * per_sm));
 }
 
 inline unsigned blocks_for(int64_t n, int threads) {

@@ -56,7 +56,7 @@ __device__ __forceinline__ void op_pair_unit(const TileView& tv, const double* x
 template <int DIM>
 __global__ void __launch_bounds__(TILE_NODES) k_resid(TileView tv, const uint8_t* code, const double* diag, OpParams o,
                                                       const double* b, const double* x, double* r, double* part) {
-  __shared__ double sm[32];
+  __shared__ double sm[TILE_NODES];
   double sbb = 0.0, srr = 0.0;
   EB_PAIR_LOOP(DIM, tv, node) {
     uint32_t c0, c1;
@@ -85,16 +85,17 @@ __global__ void __launch_bounds__(TILE_NODES) k_resid(TileView tv, const uint8_t
 // of r.z for the new r and the z of the iteration ending (still in z): the
 // r.zold term of the Polak-Ribiere beta.
 template <int DIM>
-__global__ void __launch_bounds__(TILE_NODES) k_update_xr(PairList pl, PcgScalars* sc, double* x, double* r,
+__global__ void __launch_bounds__(TILE_NODES) k_update_xr(PairList pl, PcgScalars* sc, double* r,
                                                           const double* p, const double* q, const double* pq_part,
                                                           int nblk, double* part, double h2, const double* z,
                                                           double* rzo_part) {
-  __shared__ double sm[32];
+  __shared__ double sm[TILE_NODES];
   __shared__ double s_alpha;
   if (cta_done(sc)) {
     if (threadIdx.x == 0) part[blockIdx.x] = 0.0;
     return;
   }
+  double* const x = sc->x;
   const double alpha = pcg_alpha(sc, pq_part, nblk, sm, &s_alpha);
   const double ax = alpha * h2;
   double s = 0.0, so = 0.0;
@@ -121,7 +122,7 @@ __global__ void __launch_bounds__(TILE_NODES) k_update_xr(PairList pl, PcgScalar
 template <int DIM>
 __global__ void __launch_bounds__(TILE_NODES) k_jacobi_dot(TileView tv, const uint8_t* code, const double* diag,
                                                            OpParams o, const double* r, double* z, double* part) {
-  __shared__ double sm[32];
+  __shared__ double sm[TILE_NODES];
   double s = 0.0;
   EB_PAIR_LOOP(DIM, tv, node) {
     uint32_t c0, c1;
@@ -138,7 +139,7 @@ __global__ void __launch_bounds__(TILE_NODES) k_jacobi_dot(TileView tv, const ui
 
 template <int DIM>
 __global__ void __launch_bounds__(TILE_NODES) k_dot(TileView tv, const double* a, const double* b, double* part) {
-  __shared__ double sm[32];
+  __shared__ double sm[TILE_NODES];
   double s = 0.0;
   EB_PAIR_LOOP(DIM, tv, node) {
     const Two<double> av = LdRO::ld2(a + node), bv = LdRO::ld2(b + node);
@@ -172,16 +173,33 @@ __global__ void __launch_bounds__(TILE_NODES) k_xpby_apply(TileView tv, PairList
                                                            const double* rz_part, int nrz, const double* rzo_part,
                                                            int nupd, double* pq_part, const double* rr_part,
                                                            cudaGraphConditionalHandle h) {
-  __shared__ double sm[32];
+  __shared__ double sm[TILE_NODES + 2];
   __shared__ double s_beta;
   if (cta_done(sc)) {
     if (COND && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(h, 0u);
     return;
   }
+  // this thread's first pair on its way into L1 during the partial sums
+  const int64_t l0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (l0 < pl.n) {
+    const int32_t nd = __ldg(pl.node + l0);
+    prefetch_l1(z + nd);
+    prefetch_l1(z + max(nd - tv.sy, 0));
+    prefetch_l1(z + min(nd + tv.sy, tv.nn - 1));
+    if (dim_of(DIM) == 3) {
+      prefetch_l1(z + max(nd - tv.sz, 0));
+      prefetch_l1(z + min(nd + tv.sz, tv.nn - 1));
+    }
+    prefetch_l1(code + nd);
+    if (!first) {
+      prefetch_l1(p + nd);
+      prefetch_l1(q + nd);
+    }
+  }
   if (!first) {
-    const double v = sum_parts(rz_part, nrz, 1, sm);
-    __syncthreads();
-    const double t = rzo_part ? sum_parts(rzo_part, nupd, 1, sm) : 0.0;
+    double v, t = 0.0;
+    if (rzo_part) sum_parts2(rz_part, nrz, rzo_part, nupd, sm, v, t);
+    else v = sum_parts(rz_part, nrz, sm);
     if (threadIdx.x == 0) {
       const int k = sc->slot;  // not sc->iters: CTA 0 of this launch may advance it
       const bool ok = v > 0.0;
@@ -204,7 +222,7 @@ __global__ void __launch_bounds__(TILE_NODES) k_xpby_apply(TileView tv, PairList
     // this iteration's update, then continue while not converged (or broken
     // down) and below the iteration limit.  CTAs that start after it and see
     // done skip the p, q update, which a finished loop does not use.
-    const double v = sum_parts(rr_part, nupd, 1, sm);
+    const double v = sum_parts(rr_part, nupd, sm);
     if (threadIdx.x == 0) {
       if (!sc->done) {
         sc->rr = v;
@@ -674,10 +692,11 @@ void Solver::alloc_work(cudaStream_t s) {
   q = dalloc<double>(nn, s);
   tmp = dalloc<double>(nn, s);
   nblk = (int)std::min<int64_t>(std::max<int64_t>(eb->num_tiles, 1), (int64_t)num_sms() * 4);
-  // p'q and r'r regions of 2 nblk, r'z of 2 max(nblk, 8 SMs) (the V-cycle's
-  // grid sweeps use at most 8 CTAs per SM), then r'zold of nblk
+  // p'q and r'r regions of 2 npart, r'z of 2 max(nblk, 8 SMs) (the V-cycle's
+  // grid sweeps use at most 8 CTAs per SM), then r'zold of npart
   rz_cap = 2 * std::max<int64_t>(nblk, (int64_t)num_sms() * 8);
-  part = dalloc<double>(5 * (int64_t)nblk + rz_cap, s);
+  npart = std::max(nblk, nblk_iter());
+  part = dalloc<double>(5 * (int64_t)npart + rz_cap, s);
   sc = dalloc<PcgScalars>(1, s);
   EB_CUDA(cudaMallocHost((void**)&sc_host, sizeof(PcgScalars)));
 }
@@ -784,6 +803,7 @@ int Solver::pcg(const double* b, double* x, double rtol, int maxit, const pcg_op
   auto t0 = std::chrono::steady_clock::now();
   PcgScalars init{};
   init.tol2 = rtol * rtol;
+  init.x = xi;
   int total_iters = 0;
   const int pcg_maxit = maxit;
   bool converged = false;
@@ -832,7 +852,7 @@ int Solver::pcg(const double* b, double* x, double rtol, int maxit, const pcg_op
     int it = 0;
     bool stop = false;
     if (o.use_graph == 1 && !prof_on) {  // the whole loop on the device
-      loop_prepare(kind, b, xi, s);
+      loop_prepare(kind);
       EB_CUDA(cudaGraphLaunch(lexec, s));
       EB_CUDA(cudaMemcpyAsync(sc_host, sc, sizeof(PcgScalars), cudaMemcpyDeviceToHost, s));
       EB_CUDA(cudaStreamSynchronize(s));
@@ -843,13 +863,13 @@ int Solver::pcg(const double* b, double* x, double rtol, int maxit, const pcg_op
       const int nb = std::min(check, maxit - (total_iters + it));
       bool graphed = false;
       if (o.use_graph && nb == check) {
-        graph_prepare(kind, b, xi, check, prof_on ? prof_what : 0, s);
+        graph_prepare(kind, check, prof_on ? prof_what : 0, s);
         EB_CUDA(cudaGraphLaunch(gexec, s));
         nlaunch += g_launches;
         graphed = true;
         it += nb;
       } else {
-        for (int j = 0; j < nb; ++j, ++it) iteration(kind, b, xi, s);
+        for (int j = 0; j < nb; ++j, ++it) iteration(kind, s);
       }
       EB_CUDA(cudaGetLastError());
       EB_CUDA(cudaMemcpyAsync(sc_host, sc, sizeof(PcgScalars), cudaMemcpyDeviceToHost, s));
@@ -969,7 +989,7 @@ static void launch_xpby_apply(const EBHandle& eb, unsigned g, cudaStream_t s, co
                               const double* rzo, int nupd, double* pq, const double* rr,
                               cudaGraphConditionalHandle h) {
   dim_dispatch(eb, [&](auto D) {
-    k_xpby_apply<D.value, SHIFT, COND><<<g, TILE_NODES, 0, s>>>(tv, pl, sc, code, diag, op, z, p, q, first, rz, nrz,
+    k_xpby_apply<D.value, SHIFT, COND><<<g, list_threads(pl.n), 0, s>>>(tv, pl, sc, code, diag, op, z, p, q, first, rz, nrz,
                                                                 rzo, nupd, pq, rr, h);
   });
 }
@@ -991,14 +1011,14 @@ void Solver::xpby_apply(const OpParams& op, bool flex, int first, cudaStream_t s
       DfBeta bdf;
       for (int a = 0; a < 3; ++a) bdf.b[a] = beta_df[a];
       dim_dispatch(*eb, [&](auto D) {
-        k_xpby_apply_df<D.value, SH, CO><<<g, TILE_NODES, 0, s>>>(tv, pl, sc, eb->code, diag_df, sig, zf, p, q, first,
+        k_xpby_apply_df<D.value, SH, CO><<<g, iter_threads(), 0, s>>>(tv, pl, sc, eb->code, diag_df, sig, zf, p, q, first,
                                                                   part_rz(), rz_n, rzo, (int)g, part_pq(), part_rr(),
                                                                   h, bdf);
       });
       return;
     }
     launch_xpby_apply<SH, CO>(*eb, g, s, tv, pl, sc, eb->code, eb->diag, op, z, p, q, first, part_rz(), rz_n, rzo,
-                              nblk, part_pq(), part_rr(), h);
+                              (int)g, part_pq(), part_rr(), h);
   };
   using T = std::true_type;
   using F = std::false_type;
@@ -1011,9 +1031,7 @@ void Solver::xpby_apply(const OpParams& op, bool flex, int first, cudaStream_t s
   }
 }
 
-void Solver::iteration(int kind, const double* b, double* x, cudaStream_t s,
-                       const cudaGraphConditionalHandle* cond) {
-  (void)b;
+void Solver::iteration(int kind, cudaStream_t s, const cudaGraphConditionalHandle* cond) {
   const int dim = eb->g.dim;
   const OpParams op = op_params(*this);
   const bool flex = flex_for(kind);
@@ -1025,7 +1043,6 @@ void Solver::iteration(int kind, const double* b, double* x, cudaStream_t s,
   if (kind == EB_PC_AMG && H) {
     PcgUpdate u;
     u.sc = sc;
-    u.x = x;
     u.r = r;
     u.p = p;
     u.q = q;
@@ -1040,9 +1057,16 @@ void Solver::iteration(int kind, const double* b, double* x, cudaStream_t s,
     if (fused) ++nlaunch;
   }
   EB_REQUIRE(fused || !df_on, EB_ERR_INVALID, "pcg: the DF outer iteration needs the fused x/r update");
-  if (!fused)
-    EB_DIM_LAUNCH(dim, k_update_xr, nblk, eb->pairs(), sc, x, r, p, q, part_pq(), nblk, part_rr(), eb->g.h * eb->g.h, z,
-                  flex ? part_rzo() : nullptr);
+  if (!fused) {
+    ++nlaunch;
+    const int nb = nblk_iter();
+    const double h2 = eb->g.h * eb->g.h;
+    double* rzo = flex ? part_rzo() : nullptr;
+    if (dim == 2)
+      k_update_xr<2><<<nb, iter_threads(), 0, s>>>(eb->pairs(), sc, r, p, q, part_pq(), nb, part_rr(), h2, z, rzo);
+    else
+      k_update_xr<3><<<nb, iter_threads(), 0, s>>>(eb->pairs(), sc, r, p, q, part_pq(), nb, part_rr(), h2, z, rzo);
+  }
   prof_mark(s, false, PROF_UPDATE);
   precondition(kind, r, z, s, fused);
   // r'r and the convergence test end the iteration: in the device-side loop
@@ -1056,8 +1080,8 @@ void Solver::iteration(int kind, const double* b, double* x, cudaStream_t s,
 // Captures `iters` iterations into a CUDA graph (once per argument set).  The
 // capture runs on a private stream forked from s, so s may be the legacy
 // default stream.
-void Solver::graph_prepare(int kind, const double* b, double* x, int iters, int profile, cudaStream_t s) {
-  if (gexec && g_b == b && g_x == x && g_iters == iters && g_kind == kind && g_prof == profile && g_nn == nn &&
+void Solver::graph_prepare(int kind, int iters, int profile, cudaStream_t s) {
+  if (gexec && g_iters == iters && g_kind == kind && g_prof == profile && g_nn == nn &&
       g_nn_mode == nn_mode && g_tile_gen == eb->tile_gen && g_df == (int)df_on)
     return;
   if (prof_on) {  // settle event pairs recorded so far before the capture reuses them
@@ -1073,7 +1097,7 @@ void Solver::graph_prepare(int kind, const double* b, double* x, int iters, int 
   const int64_t n0 = nlaunch;
   prof_n = 0;
   EB_CUDA(cudaStreamBeginCapture(cap_stream, cudaStreamCaptureModeThreadLocal));
-  for (int j = 0; j < iters; ++j) iteration(kind, b, x, cap_stream);
+  for (int j = 0; j < iters; ++j) iteration(kind, cap_stream);
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamEndCapture(cap_stream, &graph);
   cudaEventDestroy(fork);
@@ -1084,8 +1108,6 @@ void Solver::graph_prepare(int kind, const double* b, double* x, int iters, int 
   g_launches = nlaunch - n0;
   nlaunch = n0;
   g_pairs = prof_n;
-  g_b = b;
-  g_x = x;
   g_iters = iters;
   g_kind = kind;
   g_prof = profile;
@@ -1099,8 +1121,6 @@ void Solver::graph_release() {
   if (gexec) cudaGraphExecDestroy(gexec);
   gexec = nullptr;
   g_pairs = 0;
-  g_b = nullptr;
-  g_x = nullptr;
 }
 
 cudaGraphExec_t build_while_graph(cudaStream_t cap,
@@ -1139,20 +1159,17 @@ cudaGraphExec_t build_while_graph(cudaStream_t cap,
 
 // Captures the device-side loop { while (!done && iters < maxit) iteration }
 // (once per argument set).
-void Solver::loop_prepare(int kind, const double* b, double* x, cudaStream_t s) {
-  if (lexec && l_b == b && l_x == x && l_kind == kind && l_nn == nn && l_nn_mode == nn_mode &&
+void Solver::loop_prepare(int kind) {
+  if (lexec && l_kind == kind && l_nn == nn && l_nn_mode == nn_mode &&
       l_tile_gen == eb->tile_gen && l_df == (int)df_on)
     return;
   loop_release();
-  (void)s;  // capturing runs nothing; the graph is launched on s
   if (!cap_stream) EB_CUDA(cudaStreamCreateWithFlags(&cap_stream, cudaStreamNonBlocking));
   const int64_t n0 = nlaunch;
   lexec = build_while_graph(cap_stream,
-                            [&](cudaStream_t cs, cudaGraphConditionalHandle h) { iteration(kind, b, x, cs, &h); });
+                            [&](cudaStream_t cs, cudaGraphConditionalHandle h) { iteration(kind, cs, &h); });
   l_launches = nlaunch - n0;
   nlaunch = n0;
-  l_b = b;
-  l_x = x;
   l_kind = kind;
   l_nn = nn;
   l_nn_mode = nn_mode;
@@ -1163,8 +1180,6 @@ void Solver::loop_prepare(int kind, const double* b, double* x, cudaStream_t s) 
 void Solver::loop_release() {
   if (lexec) cudaGraphExecDestroy(lexec);
   lexec = nullptr;
-  l_b = nullptr;
-  l_x = nullptr;
 }
 
 static bool capturing(cudaStream_t s) {

@@ -33,6 +33,7 @@ struct PcgScalars {
   // p update, whose launch may also advance iters (device-side loop)
   int slot;
   double rzo;  // batched flexible PCG: r'zold of the iteration (FIN_RRF)
+  double* x;   // the vector the solve updates: captured iterations serve any
 };
 
 struct Hierarchy;  // AMG levels (amg.cu)
@@ -56,18 +57,19 @@ struct Solver {
   bool flex_for(int kind) const { return kind == EB_PC_AMG_NN || (kind == EB_PC_AMG && flexible()); }
   nn_handle* nn = nullptr;  // learned stage of EB_PC_AMG_NN (set for one solve)
   int nn_mode = 0;          // eb_nn_mode of that stage
-  // reduction partials: [p'q | r'r] regions of 2 nblk each, then the r'z region
-  // of 2 max(nblk, 8 SMs): r'z comes from the PCG's own dot kernel (nblk
-  // partials) or from the V-cycle's last smoothing launch (one per CTA of it),
-  // then the r'zold region of nblk
+  // reduction partials: [p'q | r'r] regions of 2 npart each, then the r'z region
+  // (nblk partials from the PCG's own dot kernel, one per CTA of the V-cycle's
+  // last smoothing launch), then the r'zold region of npart
+  int npart = 1;  // max(nblk, nblk_iter())
   double* part = nullptr;
   double* part_pq() const { return part; }
-  double* part_rr() const { return part + 2 * (int64_t)nblk; }
-  double* part_rz() const { return part + 4 * (int64_t)nblk; }
-  // r'zold partials of the flexible beta (nblk, from the x/r update)
-  double* part_rzo() const { return part + 4 * (int64_t)nblk + rz_cap; }
+  double* part_rr() const { return part + 2 * (int64_t)npart; }
+  double* part_rz() const { return part + 4 * (int64_t)npart; }
+  // r'zold partials of the flexible beta (from the x/r update)
+  double* part_rzo() const { return part + 4 * (int64_t)npart + rz_cap; }
   // CTAs (= partials) of the iteration's x/r update and p update + apply
-  int nblk_iter() const { return nblk; }
+  int nblk_iter() const { return list_blocks(*eb); }
+  int iter_threads() const { return list_threads(eb->num_pairs); }
   int64_t rz_cap = 0;
   int nblk = 1;
   int rz_n = 1;  // r'z partials written by the last precondition()
@@ -81,11 +83,10 @@ struct Solver {
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> prof_ev;
   double prof_acc_ms = 0.0;
   int prof_acc_n = 0;
-  // captured PCG iteration (CUDA graph), keyed by its arguments
+  // captured PCG iteration (CUDA graph), keyed by what it depends on: neither b
+  // nor x, whose address the iteration takes from sc
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t gexec = nullptr;
-  const double* g_b = nullptr;
-  double* g_x = nullptr;
   const nn_handle* g_nn = nullptr;
   int g_tile_gen = -1;
   int g_nn_mode = -1;
@@ -94,8 +95,6 @@ struct Solver {
   // the whole iteration loop on the device: a conditional WHILE node whose
   // body is one iteration (no host round trip per iteration)
   cudaGraphExec_t lexec = nullptr;
-  const double* l_b = nullptr;
-  double* l_x = nullptr;
   int l_kind = -1, l_nn_mode = -1, l_tile_gen = -1;
   const nn_handle* l_nn = nullptr;
   int64_t l_launches = 0;  // kernel launches per loop iteration
@@ -133,15 +132,14 @@ struct Solver {
   void prof_end(pcg_stats* st, cudaStream_t s);
   void prof_release();
   // cond: inside the device-side loop, the handle its last launch sets
-  void iteration(int kind, const double* b, double* x, cudaStream_t s,
-                 const cudaGraphConditionalHandle* cond = nullptr);
+  void iteration(int kind, cudaStream_t s, const cudaGraphConditionalHandle* cond = nullptr);
   // p = z + beta p and q = h^2 (sigma I + A) z + beta q with the p.q partials
   // (eb_solve.cu); flex: the Polak-Ribiere beta (r'zold partials in part_rzo)
   void xpby_apply(const OpParams& op, bool flex, int first, cudaStream_t s,
                   const cudaGraphConditionalHandle* cond = nullptr);
-  void graph_prepare(int kind, const double* b, double* x, int iters, int profile, cudaStream_t s);
+  void graph_prepare(int kind, int iters, int profile, cudaStream_t s);
   void graph_release();
-  void loop_prepare(int kind, const double* b, double* x, cudaStream_t s);
+  void loop_prepare(int kind);
   void loop_release();
 };
 
@@ -155,18 +153,24 @@ cudaGraphExec_t build_while_graph(cudaStream_t cap,
 // AMG (amg.cu)
 void amg_build(Solver& S, cudaStream_t s);
 void amg_free(Solver& S);
-// Sum of v over the CTA (warp shuffles, then the warps in order); thread 0
-// holds the result.  Every reduction partial of the PCG is formed this way.
-__device__ __forceinline__ double block_sum(double v, double* sm) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) sm[w] = v;
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x == 0)
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += sm[i];
+// Sum of v over the CTA: through shared memory, one warp adding the columns
+// and then its lanes; thread 0 holds the result.  Every reduction partial of
+// the PCG is formed this way.  GB300 issues 0.4 FP64 lanes per clock and
+// scheduler, so a warp-wide FP64 addition occupies one for 80 clocks: a CTA of
+// 256 threads spends 12 of them here, where shuffle trees in all its warps and
+// a serial end take 48.  sm: blockDim.x doubles.
+__device__ __forceinline__ double warp_column_sum(const double* sm, int n) {
+  double s = sm[threadIdx.x & 31];
+  for (int i = (threadIdx.x & 31) + 32; i < n; i += 32) s += sm[i];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   return s;
+}
+
+__device__ __forceinline__ double block_sum(double v, double* sm) {
+  __syncthreads();
+  sm[threadIdx.x] = v;
+  __syncthreads();
+  return threadIdx.x < 32 ? warp_column_sum(sm, (int)blockDim.x) : 0.0;
 }
 
 // sc->done as thread 0 of the CTA reads it, the same for all its threads (CTA
@@ -180,13 +184,48 @@ __device__ __forceinline__ bool cta_done(const PcgScalars* sc) {
   return s_done != 0;
 }
 
-// sum of n partials (stride apart) in a fixed order, the same in every CTA;
-// thread 0 holds the result
-__device__ __forceinline__ double sum_parts(const double* part, int n, int stride, double* sm) {
+// sum of n partials in a fixed order, the same in every CTA of a launch;
+// thread 0 holds the result.  Four warps load (as many as the FP64 additions
+// keep busy: every CTA repeats the sum), one combines.  sm: 128 doubles.
+__device__ __forceinline__ double sum_parts(const double* part, int n, double* sm) {
+  const int w = min((int)blockDim.x, 128);
   double a = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) a += part[stride * i];
-  return block_sum(a, sm);
+  if ((int)threadIdx.x < w) {
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += w) a += part[i];
+  }
+  __syncthreads();
+  if ((int)threadIdx.x < w) sm[threadIdx.x] = a;
+  __syncthreads();
+  return threadIdx.x < 32 ? warp_column_sum(sm, w) : 0.0;
 }
+
+// two such sums side by side, by the two halves of the CTA (blockDim.x >= 64);
+// thread 0 holds both.  sm: 258 doubles.
+__device__ __forceinline__ void sum_parts2(const double* pa, int na, const double* pb, int nb, double* sm, double& a,
+                                           double& b) {
+  const int half = (int)blockDim.x >> 1, g = (int)threadIdx.x >= half, l = (int)threadIdx.x - g * half;
+  const int w = min(half, 128), n = g ? nb : na;
+  const double* p = g ? pb : pa;
+  double v = 0.0;
+  if (l < w) {
+#pragma unroll 4
+    for (int i = l; i < n; i += w) v += p[i];
+  }
+  __syncthreads();
+  if (l < w) sm[128 * g + l] = v;
+  __syncthreads();
+  if (l < 32) {
+    const double s = warp_column_sum(sm + 128 * g, w);
+    if (l == 0) sm[256 + g] = s;
+  }
+  __syncthreads();
+  a = sm[256];
+  b = sm[257];
+}
+
+// into L1 ahead of a load (the reduction sums between hide the latency)
+__device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 
 // alpha = rz / p'q from the nblk partials of k_xpby_apply (q scaled by h^2:
 // the CG step length over h^2), formed by every CTA in
@@ -211,7 +250,7 @@ __device__ __forceinline__ double pcg_alpha_from(PcgScalars* sc, double pq) {
 
 __device__ __forceinline__ double pcg_alpha(PcgScalars* sc, const double* pq_part, int nblk, double* sm,
                                             double* s_alpha) {
-  const double pq = sum_parts(pq_part, nblk, 1, sm);
+  const double pq = sum_parts(pq_part, nblk, sm);
   if (threadIdx.x == 0) *s_alpha = pcg_alpha_from(sc, pq);
   __syncthreads();
   return *s_alpha;
@@ -223,7 +262,7 @@ __device__ __forceinline__ double pcg_alpha(PcgScalars* sc, const double* pq_par
 // such step (a single level), else the launch was issued.
 struct PcgUpdate {
   PcgScalars* sc = nullptr;
-  double *x = nullptr, *r = nullptr;
+  double* r = nullptr;  // x is sc->x
   const double *p = nullptr, *q = nullptr, *pq_part = nullptr;
   int nblk = 0;
   double* rr_part = nullptr;

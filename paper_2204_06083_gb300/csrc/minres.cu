@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(TILE_NODES) k_mr_init(TileView tv, PairList pl
                                                         const double* diag, MrOp o, const double* b, const double* x,
                                                         double* v, double* v_prev, double* w, double* w_prev,
                                                         double* part) {
-  __shared__ double sm[32];
+  __shared__ double sm[TILE_NODES];
   double sbb = 0.0;
   EB_LIST_LOOP(pl, node) {
     uint32_t c0, c1;
@@ -78,10 +78,10 @@ __global__ void __launch_bounds__(TILE_NODES) k_mr_init(TileView tv, PairList pl
 // and eta = gamma_1 (one CTA)
 __global__ void k_mr_start(MrScalars* sc, const double* bb_part, int nbb, const double* vz_part, int nvz, double rtol,
                            int maxit) {
-  __shared__ double sm[32];
-  const double bb = sum_parts(bb_part, nbb, 1, sm);
+  __shared__ double sm[TILE_NODES];
+  const double bb = sum_parts(bb_part, nbb, sm);
   __syncthreads();
-  const double vz = sum_parts(vz_part, nvz, 1, sm);
+  const double vz = sum_parts(vz_part, nvz, sm);
   if (threadIdx.x == 0) {
     MrScalars m{};
     MrRot& r = m.st[0];
@@ -129,7 +129,7 @@ template <int DIM>
 __global__ void __launch_bounds__(TILE_NODES) k_mr_apply(TileView tv, PairList pl, const uint8_t* code,
                                                          const double* diag, MrOp o, const MrScalars* sc,
                                                          const double* z, double* zs, double* az, double* part) {
-  __shared__ double sm[32];
+  __shared__ double sm[TILE_NODES];
   const MrRot m = mr_view(sc, -1);
   if (m.done) {
     if (threadIdx.x == 0) part[blockIdx.x] = 0.0;
@@ -155,11 +155,11 @@ __global__ void __launch_bounds__(TILE_NODES) k_mr_apply(TileView tv, PairList p
 
 __global__ void __launch_bounds__(TILE_NODES) k_mr_lanczos(PairList pl, MrScalars* sc, const double* d_part, int nd,
                                                            const double* az, double* v, double* v_prev) {
-  __shared__ double sm[32];
+  __shared__ double sm[TILE_NODES];
   __shared__ double s_delta;
   const MrRot m = mr_view(sc, -1);
   if (m.done) return;
-  const double delta = sum_parts(d_part, nd, 1, sm);
+  const double delta = sum_parts(d_part, nd, sm);
   if (threadIdx.x == 0) {
     s_delta = delta;
     if (blockIdx.x == 0) {
@@ -182,7 +182,7 @@ template <bool COND>
 __global__ void __launch_bounds__(TILE_NODES) k_mr_update(PairList pl, MrScalars* sc, const double* vz_part, int nvz,
                                                           const double* zs, double* w, double* w_prev, double* x,
                                                           cudaGraphConditionalHandle h) {
-  __shared__ double sm[32];
+  __shared__ double sm[TILE_NODES];
   __shared__ double s_k[4];  // a2, a3, 1 / a1, c_{j+1} eta
   __shared__ int s_slot;
   if (threadIdx.x == 0) s_slot = *(volatile const int*)&sc->slot;  // written by the launch before
@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(TILE_NODES) k_mr_update(PairList pl, MrScalars
     if (COND && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(h, 0u);
     return;
   }
-  const double vz = sum_parts(vz_part, nvz, 1, sm);
+  const double vz = sum_parts(vz_part, nvz, sm);
   if (threadIdx.x == 0) {
     const double delta = sc->delta;  // written by the launch before
     const bool ok = vz >= 0.0 && isfinite(vz);
@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(TILE_NODES) k_mr_update(PairList pl, MrScalars
 
 // partials of a'b over the CP pairs
 __global__ void __launch_bounds__(TILE_NODES) k_mr_dot(PairList pl, const double* a, const double* b, double* part) {
-  __shared__ double sm[32];
+  __shared__ double sm[TILE_NODES];
   double s = 0.0;
   EB_LIST_LOOP(pl, node) {
     const Two<double> av = LdRO::ld2(a + node), bv = LdRO::ld2(b + node);
@@ -275,7 +275,7 @@ template <int DIM>
 __global__ void __launch_bounds__(TILE_NODES) k_mr_resid(TileView tv, PairList pl, const uint8_t* code,
                                                          const double* diag, MrOp o, const double* b, const double* x,
                                                          double* part) {
-  __shared__ double sm[32];
+  __shared__ double sm[TILE_NODES];
   double srr = 0.0;
   EB_LIST_LOOP(pl, node) {
     uint32_t c0, c1;
@@ -292,8 +292,8 @@ __global__ void __launch_bounds__(TILE_NODES) k_mr_resid(TileView tv, PairList p
 }
 
 __global__ void k_mr_sum(const double* part, int n, double* out) {
-  __shared__ double sm[32];
-  const double v = sum_parts(part, n, 1, sm);
+  __shared__ double sm[TILE_NODES];
+  const double v = sum_parts(part, n, sm);
   if (threadIdx.x == 0) *out = v;
 }
 
