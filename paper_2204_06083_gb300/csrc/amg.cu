@@ -635,7 +635,7 @@ __global__ void k_row_sort(DCsr C) {
   }
 }
 
-static DCsr transpose(const DCsr& A, cudaStream_t s) {
+DCsr transpose(const DCsr& A, cudaStream_t s) {
   DCsr T;
   T.n = A.m;
   T.m = A.n;
@@ -1058,7 +1058,7 @@ void amg_build_from(Solver& S, DCsr A0, cudaStream_t s) {
       }
       DCsr AP = spgemm(A, L.P, s);
       DCsr Ac = spgemm(L.R, AP, s);
-      csr_free(AP, s);
+      L.AP = AP;
       A = Ac;
       continue;
     }
@@ -1125,7 +1125,7 @@ void amg_build_from(Solver& S, DCsr A0, cudaStream_t s) {
     }
     DCsr AP = spgemm(A, L.P, s);
     DCsr Ac = spgemm(L.R, AP, s);
-    csr_free(AP, s);
+    L.AP = AP;
     A = Ac;
   }
   // coarsest level
@@ -1146,6 +1146,7 @@ void amg_free(Solver& S) {
     csr_free(L.A, s);
     csr_free(L.P, s);
     csr_free(L.R, s);
+    csr_free(L.AP, s);
     dfree(L.R0node, s); dfree(L.agg, s); dfree(L.dinv, s);
   }
   dfree(H->coarse_inv, s);

@@ -28,8 +28,21 @@ struct VecSet {
   V *b = nullptr, *x = nullptr, *x2 = nullptr, *d = nullptr, *r = nullptr;
 };
 
+// Two matrices of one sparsity pattern (that of the first, which contains the
+// other's), values in the storage type of a reduced-precision V-cycle
+struct PairCsr {
+  int64_t n = 0, nnz = 0;
+  int32_t *rp = nullptr, *ci = nullptr;
+  void *a = nullptr, *c = nullptr;
+};
+
 struct Level {
   DCsr A, P, R;               // FP64 hierarchy (exact setup)
+  // reduced-precision V-cycles: (A P, P) for the prolongation that also does
+  // the first post-smoothing step, and, on compact levels, ((A P)^T, P^T) for
+  // the restriction that needs no residual
+  DCsr AP;                    // setup only
+  PairCsr Q, T;
   int32_t* R0node = nullptr;  // level 0 only: R's columns as grid node indices
   int32_t* agg = nullptr;
   double* dinv = nullptr;     // compact levels
@@ -67,6 +80,7 @@ struct Hierarchy {
 
 DCsr level0_csr(const EBHandle& eb, double sigma, cudaStream_t s);
 void amg_build_from(Solver& S, DCsr A0, cudaStream_t s);
+DCsr transpose(const DCsr& A, cudaStream_t s);
 void amg_alloc_vcycle(Solver& S, cudaStream_t s);
 void amg_free_vcycle(Hierarchy& H, cudaStream_t s);
 

@@ -764,6 +764,158 @@ __global__ void k_c_prolong_add(CsrV<V> P, const V* e, V* x) {
   if (i < P.n && g == 0) x[i] = cvt<V>(cvt<A>(x[i]) + s);
 }
 
+// Pairs of matrices of one pattern -------------------------------------------
+template <class V>
+struct PairV {
+  int64_t n;
+  const int32_t *rp, *ci;
+  const V *a, *c;
+};
+
+// Lane g's parts of sum_e a[e] x[ci[e]] and sum_e c[e] y[ci[e]] (csr_dot's order)
+template <int G, class V>
+__device__ __forceinline__ void pair_dot(const PairV<V>& M, const V* x, const V* y, int32_t beg, int32_t end, int g,
+                                         typename AccOf<V>::type& sa, typename AccOf<V>::type& sc) {
+  using A = typename AccOf<V>::type;
+  sa = sc = 0;
+  for (int32_t e0 = beg + g; e0 < end; e0 += CSR_UNROLL * G) {
+    int32_t k[CSR_UNROLL];
+    A wa[CSR_UNROLL], wc[CSR_UNROLL];
+#pragma unroll
+    for (int u = 0; u < CSR_UNROLL; ++u) {
+      const int32_t e = e0 + u * G;
+      k[u] = e < end ? __ldg(M.ci + e) : -1;
+      wa[u] = e < end ? cvt<A>(M.a[e]) : (A)0;
+      wc[u] = e < end ? cvt<A>(M.c[e]) : (A)0;
+    }
+#pragma unroll
+    for (int u = 0; u < CSR_UNROLL; ++u)
+      if (k[u] >= 0) {
+        sa += wa[u] * cvt<A>(x[k[u]]);
+        sc += wc[u] * cvt<A>(y[k[u]]);
+      }
+  }
+}
+
+// The coarse correction and the first post-smoothing step in one launch: with
+// r = b - A x left by the restriction's launch and Q = (A P, P),
+//   x' = x + P e,  d = c2 D^-1 (b - A x') = c2 D^-1 (r - A P e),  xo = x' + d,
+// so the step needs no pass over A (whose rows are longer than A P's) after x'.
+template <int G, class V>
+__global__ void k_c_prolong_step(PairV<V> Q, const V* dinv, const V* e, const V* x, const V* r, V* xo, V* d,
+                                 typename AccOf<V>::type c2) {
+  using A = typename AccOf<V>::type;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t i = t / G;
+  const int g = (int)(t % G);
+  A di = 0, ri = 0, xi = 0, sa = 0, sc = 0;
+  if (i < Q.n) {
+    if (g == 0) {
+      di = cvt<A>(dinv[i]);
+      ri = cvt<A>(r[i]);
+      xi = cvt<A>(x[i]);
+    }
+    pair_dot<G>(Q, e, e, Q.rp[i], Q.rp[i + 1], g, sa, sc);
+  }
+  sa = group_reduce<G>(sa);
+  sc = group_reduce<G>(sc);
+  if (i >= Q.n || g != 0) return;
+  const A dv = c2 * (di * (ri - sa));
+  d[i] = cvt<V>(dv);
+  xo[i] = cvt<V>((xi + sc) + dv);
+}
+
+// The same on level 0: row i of Q is the CP at node cp_node[i]
+template <int G, class V>
+__global__ void k_prolong0_step(PairV<V> Q, const int32_t* __restrict__ cp_node, const uint8_t* __restrict__ code,
+                                const typename DiagOf<V>::type* __restrict__ diag, GOp<typename AccOf<V>::type> o,
+                                const V* e, const V* x, const V* r, V* xo, V* d, typename AccOf<V>::type c2) {
+  using A = typename AccOf<V>::type;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t i = t / G;
+  const int g = (int)(t % G);
+  A ri = 0, xi = 0, sa = 0, sc = 0;
+  int32_t node = 0;
+  uint32_t k = 0;
+  if (i < Q.n) {
+    if (g == 0) {
+      node = __ldg(cp_node + i);
+      k = __ldg(code + node);
+      ri = cvt<A>(r[node]);
+      xi = cvt<A>(x[node]);
+    }
+    pair_dot<G>(Q, e, e, Q.rp[i], Q.rp[i + 1], g, sa, sc);
+  }
+  sa = group_reduce<G>(sa);
+  sc = group_reduce<G>(sc);
+  if (i >= Q.n || g != 0) return;
+  const A dv = c2 * (inv_diag_t<A>(k, diag, node, o) * (ri - sa));
+  d[node] = cvt<V>(dv);
+  xo[node] = cvt<V>((xi + sc) + dv);
+}
+
+// Residual and restriction in one launch: the first nbf CTAs form r = b - A x
+// (the post-smoothing needs it), the others, from x and not from r, the coarse
+// right-hand side P^T (b - A x) = P^T b - (A P)^T x and the coarse level's first
+// step.  T = ((A P)^T, P^T), rows by groups of GT lanes.
+template <int G, class V>
+__global__ void k_c_resid_restrict(CsrV<V> M, const V* b, const V* x, V* r, unsigned nbf, PairV<V> T, int GT, V* bc,
+                                   CoarseFirst<V> f) {
+  using A = typename AccOf<V>::type;
+  if (blockIdx.x < nbf) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t i = t / G;
+    const int g = (int)(t % G);
+    const A ax = csr_row<G>(M, x, i, g);
+    if (i < M.n && g == 0) r[i] = cvt<V>(cvt<A>(b[i]) - ax);
+    return;
+  }
+  const int64_t t = (int64_t)(blockIdx.x - nbf) * blockDim.x + threadIdx.x;
+  const int64_t i = t / GT;
+  const int g = (int)(t % GT);
+  A s = 0;
+  if (i < T.n) {
+    const int32_t beg = T.rp[i], end = T.rp[i + 1];
+    for (int32_t e0 = beg + g; e0 < end; e0 += 4 * GT) {
+      int32_t k[4];
+      A wa[4], wc[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int32_t e = e0 + u * GT;
+        k[u] = e < end ? __ldg(T.ci + e) : -1;
+        wa[u] = e < end ? cvt<A>(T.a[e]) : (A)0;
+        wc[u] = e < end ? cvt<A>(T.c[e]) : (A)0;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (k[u] >= 0) s += wc[u] * cvt<A>(b[k[u]]) - wa[u] * cvt<A>(x[k[u]]);
+    }
+  }
+  for (int o = GT / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, 32);
+  if (i < T.n && g == 0) store_restricted(bc, i, s, f);
+}
+
+// out[e] = the value of B at the places of A's pattern (rows sorted by column;
+// B's pattern is contained in A's), 0 elsewhere: one warp per row
+template <class V>
+__global__ void k_pair_values(DCsr A, DCsr B, V* __restrict__ a, V* __restrict__ c) {
+  const int lane = threadIdx.x & 31;
+  const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (i >= A.n) return;
+  const int32_t a0 = A.rp[i], a1 = A.rp[i + 1], b0 = B.rp[i], b1 = B.rp[i + 1];
+  for (int32_t e = a0 + lane; e < a1; e += 32) {
+    const int32_t k = A.ci[e];
+    int32_t lo = b0, hi = b1;
+    while (lo < hi) {
+      const int32_t mid = (lo + hi) >> 1;
+      if (B.ci[mid] < k) lo = mid + 1;
+      else hi = mid;
+    }
+    a[e] = cvt<V>(A.v[e]);
+    c[e] = (lo < b1 && B.ci[lo] == k) ? cvt<V>(B.v[lo]) : cvt<V>(0.0);
+  }
+}
+
 // group width for a CSR matrix: the largest power of two G <= 32 with
 // G * epl <= its mean row length (epl: entries per lane, tuned per solver)
 inline int group_width(int64_t nnz, int64_t n, int epl) {
@@ -773,9 +925,11 @@ inline int group_width(int64_t nnz, int64_t n, int epl) {
   return g;
 }
 
-#define EB_GROUP_LAUNCH(G, kernel, V, rows, s, ...)                                               \
+#define EB_GROUP_LAUNCH(G, kernel, V, rows, s, ...) \
+  EB_GROUP_GRID(G, kernel, V, blocks_for((int64_t)(rows) * (G), 256), s, __VA_ARGS__)
+#define EB_GROUP_GRID(G, kernel, V, blocks, s, ...)                                               \
   do {                                                                                           \
-    const unsigned nb_ = blocks_for((int64_t)(rows) * (G), 256);                                 \
+    const unsigned nb_ = (blocks);                                                               \
     switch (G) {                                                                                 \
       case 1: kernel<1, V><<<nb_, 256, 0, s>>>(__VA_ARGS__); break;                              \
       case 2: kernel<2, V><<<nb_, 256, 0, s>>>(__VA_ARGS__); break;                              \
@@ -896,6 +1050,11 @@ struct LevelView<__nv_bfloat16> {
   static const __nv_bfloat16* dinv(const Level& L) { return L.dinv16; }
 };
 
+template <class V>
+static PairV<V> pair_view(const PairCsr& M) {
+  return {M.n, M.rp, M.ci, static_cast<const V*>(M.a), static_cast<const V*>(M.c)};
+}
+
 // the first-step outputs for compact level l, or none if l is the coarsest
 // (its dense solve replaces smoothing)
 template <class V>
@@ -932,7 +1091,9 @@ static void vcycle_compact(Solver& S, size_t l, cudaStream_t s, bool warm = fals
     return;
   }
   const ChebCoef cc = cheb_coef(L.rho, S.opts.cheb_degree);
-  S.nlaunch += 2 + 2 * cc.deg + (warm ? 1 : 0);  // pre steps, residual, restriction, prolongation, deg steps
+  const bool mr = L.T.rp != nullptr, mp = L.Q.rp != nullptr;  // merged launches (make_pairs)
+  // pre steps, residual, restriction, prolongation, deg steps
+  S.nlaunch += 2 - (int)mr - (int)mp + 2 * cc.deg + (warm ? 1 : 0);
   const CsrV<V> A = LV::A(L);
   const int e = S.csr_epl;
   const int gA = group_width(L.A.nnz, L.A.n, e), gP = group_width(L.P.nnz, L.P.n, e),
@@ -944,14 +1105,28 @@ static void vcycle_compact(Solver& S, size_t l, cudaStream_t s, bool warm = fals
     if (mark) S.prof_mark(s, false, PROF_LEVEL1);
     std::swap(v.x, v.x2);
   }
-  EB_GROUP_LAUNCH(gA, k_c_resid, V, n, s, A, v.b, v.x, v.r);
   Level& C = H.L[l + 1];
   VecSet<V>& cv = LV::vec(C);
-  EB_GROUP_LAUNCH(gR, k_c_spmv, V, C.A.n, s, LV::R(L), v.r, cv.b, coarse_first<V>(S, l + 1));
+  if (mr) {
+    const int gT = group_width(L.T.nnz, L.T.n, e);
+    const unsigned nbf = blocks_for(n * gA, 256), nbc = blocks_for(L.T.n * gT, 256);
+    EB_GROUP_GRID(gA, k_c_resid_restrict, V, nbf + nbc, s, A, v.b, v.x, v.r, nbf, pair_view<V>(L.T), gT, cv.b,
+                  coarse_first<V>(S, l + 1));
+  } else {
+    EB_GROUP_LAUNCH(gA, k_c_resid, V, n, s, A, v.b, v.x, v.r);
+    EB_GROUP_LAUNCH(gR, k_c_spmv, V, C.A.n, s, LV::R(L), v.r, cv.b, coarse_first<V>(S, l + 1));
+  }
   vcycle_compact<V>(S, l + 1, s);
   if (S.opts.cycle == 2 && l + 2 < H.L.size()) vcycle_compact<V>(S, l + 1, s, true);
-  EB_GROUP_LAUNCH(gP, k_c_prolong_add, V, n, s, LV::P(L), cv.x, v.x);
-  for (int k = 0; k < cc.deg; ++k) {
+  if (mp) {
+    const int gQ = group_width(L.Q.nnz, L.Q.n, e);
+    EB_GROUP_LAUNCH(gQ, k_c_prolong_step, V, n, s, pair_view<V>(L.Q), LV::dinv(L), cv.x, v.x, v.r, v.x2, v.d,
+                    cc.c2[0]);
+    std::swap(v.x, v.x2);
+  } else {
+    EB_GROUP_LAUNCH(gP, k_c_prolong_add, V, n, s, LV::P(L), cv.x, v.x);
+  }
+  for (int k = mp ? 1 : 0; k < cc.deg; ++k) {
     if (mark) S.prof_mark(s, true, PROF_LEVEL1);
     EB_GROUP_LAUNCH(gA, k_c_cheb_step, V, n, s, A, LV::dinv(L), v.b, v.x, v.x2, v.d, cc.c1[k], cc.c2[k]);
     if (mark) S.prof_mark(s, false, PROF_LEVEL1);
@@ -1093,11 +1268,22 @@ static int vcycle_grid(Solver& S, const double* r, double* z, cudaStream_t s, co
   EB_GROUP_LAUNCH(gR, k_restrict0, V, C.A.n, s, C.A.n, R0.rp, L0.R0node, R0.v, g.r, cv.b, coarse_first<V>(S, 1));
   vcycle_compact<V>(S, 1, s);
   if (S.opts.cycle == 2 && H.L.size() > 2) vcycle_compact<V>(S, 1, s, true);  // W-cycle
-  if (M.on)
+  // the correction with the first post-smoothing step, unless that step is the
+  // last (which forms z)
+  const bool merged = L0.Q.rp != nullptr && cc.deg > 1;
+  if (merged) {
+    if constexpr (!std::is_same<V, double>::value) {
+      const int gQ = group_width(L0.Q.nnz, L0.Q.n, S.csr_epl);
+      EB_GROUP_LAUNCH(gQ, k_prolong0_step, V, L0.Q.n, s, pair_view<V>(L0.Q), eb.cp_node, eb.code, diag, o, cv.x, x,
+                      g.r, x2, g.d, (A)cc.c2[0]);
+      std::swap(x, x2);
+      S.nlaunch -= 1;
+    }
+  } else if (M.on)
     k_prolong_mf<DIM, V, SC><<<gl, th, 0, s>>>(tv, eb.code, diag, o, (A)M.omega, M.agg_node, sc, cv.x, x);
   else
     EB_GROUP_LAUNCH(gP, k_prolong0, V, P0.n, s, P0.n, P0.rp, P0.ci, P0.v, eb.cp_node, cv.x, x);
-  for (int k = 0; k < cc.deg; ++k) {
+  for (int k = merged ? 1 : 0; k < cc.deg; ++k) {
     // the launch that also forms the r'z partials is a different kernel: not
     // part of the smoother-step timing
     const bool mark = !(k == cc.deg - 1 && dot);
@@ -1206,6 +1392,56 @@ static float* to_f32(const double* a, int64_t n, cudaStream_t s) {
   return b;
 }
 
+// the pair (A, B) of one pattern, A's, whose structure it takes over
+template <class V>
+static void make_pair(PairCsr& M, DCsr& A, const DCsr& B, cudaStream_t s) {
+  M.n = A.n;
+  M.nnz = A.nnz;
+  M.a = dalloc<V>(A.nnz, s, false);
+  M.c = dalloc<V>(A.nnz, s, false);
+  k_pair_values<V><<<blocks_for(A.n * 32, 256), 256, 0, s>>>(A, B, static_cast<V*>(M.a), static_cast<V*>(M.c));
+  M.rp = A.rp;
+  M.ci = A.ci;
+  A.rp = nullptr;
+  A.ci = nullptr;
+  csr_free(A, s);
+}
+
+// The merged transfers of a reduced-precision V-cycle.  k_c_prolong_step pays
+// on every compact level: A P's rows are shorter than A's (level 1 of 256^3:
+// 11.6 against 4.0 + 13.4 us; of 64 stars: 7.6 against 4.5 + 13.8).  The other
+// two trade a launch (some 2 us) for more bytes, so they stay with matrices
+// that the launches and not the bytes bound: k_prolong0_step in 2D (1022^2: 5.7
+// against 4.1 + 2.8 us; 256^3, whose A P has three times the entries per row:
+// 67 against 18.3 + 7.8), k_c_resid_restrict with short rows of (A P)^T, a warp
+// or less each (1022^2: 2.9 against 2.3 + 2.1 us; 256^3, 700 entries per row:
+// 25 against 11.6 + 4.6).
+constexpr int64_t PAIR_NNZ = 2000000;
+constexpr int64_t PAIR_ROW = 128;
+template <class V>
+static void make_pairs(Solver& S, cudaStream_t s) {
+  Hierarchy& H = *S.H;
+  for (size_t l = 0; l + 1 < H.L.size(); ++l) {
+    Level& L = H.L[l];
+    const bool small = L.A.nnz <= PAIR_NNZ;
+    if (l == 0 && !(small && S.eb->pair_node && S.eb->g.dim == 2)) continue;
+    if (l > 0 && small && L.AP.nnz <= PAIR_ROW * L.AP.m) {
+      DCsr T = transpose(L.AP, s);
+      make_pair<V>(L.T, T, L.R, s);
+    }
+    make_pair<V>(L.Q, L.AP, L.P, s);
+  }
+}
+
+static void free_pair(PairCsr& M, cudaStream_t s) {
+  dfree(M.rp, s);
+  dfree(M.ci, s);
+  char *a = static_cast<char*>(M.a), *c = static_cast<char*>(M.c);
+  dfree(a, s);
+  dfree(c, s);
+  M = PairCsr{};
+}
+
 static __nv_bfloat16* to_bf16(const double* a, int64_t n, cudaStream_t s) {
   __nv_bfloat16* b = dalloc<__nv_bfloat16>(n, s, false);
   if (n > 0) k_to_bf16<<<blocks_for(n, 256), 256, 0, s>>>(n, a, b);
@@ -1227,6 +1463,7 @@ void amg_alloc_vcycle(Solver& S, cudaStream_t s) {
       if (L.P.v) L.P32 = to_f32(L.P.v, L.P.nnz, s);
       if (L.R.v) L.R32 = to_f32(L.R.v, L.R.nnz, s);
     }
+    make_pairs<float>(S, s);
   } else if (S.opts.vcycle_prec == EB_BF16) {
     alloc_set(H.g16, nn, true, s);
     for (size_t l = first; l < H.L.size(); ++l) alloc_set(H.L[l].v16, H.L[l].A.n, true, s);
@@ -1237,6 +1474,7 @@ void amg_alloc_vcycle(Solver& S, cudaStream_t s) {
       if (L.P.v) L.P16 = to_bf16(L.P.v, L.P.nnz, s);
       if (L.R.v) L.R16 = to_bf16(L.R.v, L.R.nnz, s);
     }
+    make_pairs<__nv_bfloat16>(S, s);
   } else {
     alloc_set(H.g64, nn, false, s);
     const EBHandle& eb = *S.eb;
@@ -1247,6 +1485,7 @@ void amg_alloc_vcycle(Solver& S, cudaStream_t s) {
     }
     for (size_t l = first; l < H.L.size(); ++l) alloc_set(H.L[l].v64, H.L[l].A.n, true, s);
   }
+  for (Level& L : H.L) csr_free(L.AP, s);
   EB_CUDA(cudaGetLastError());
 }
 
@@ -1260,6 +1499,8 @@ void amg_free_vcycle(Hierarchy& H, cudaStream_t s) {
     free_set(L.v32, s);
     free_set(L.v16, s);
     dfree(L.A32, s); dfree(L.P32, s); dfree(L.R32, s); dfree(L.dinv32, s);
+    free_pair(L.Q, s);
+    free_pair(L.T, s);
     dfree(L.A16, s); dfree(L.P16, s); dfree(L.R16, s); dfree(L.dinv16, s);
   }
 }
