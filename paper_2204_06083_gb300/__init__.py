@@ -221,10 +221,31 @@ def _check(code: int, allow=()):
     return code
 
 
-def _stream(stream=None):
+# The calls on device vectors are asynchronous and short (a few microseconds on
+# the GPU), so their marshalling is kept to plain integers: addresses and the
+# raw handle of the current stream (ctypes takes an int for a void *).
+_raw_stream = None   # () -> the current stream's raw handle
+_apply_prec = None   # torch element type -> eb_prec
+
+
+def _bind_torch():
+    global _raw_stream, _apply_prec
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    _apply_prec = {torch.float64: EB_F64, torch.float32: EB_F32, torch.bfloat16: EB_BF16}
+    get, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+    if get is None or dev is None:
+        _raw_stream = lambda: torch.cuda.current_stream().cuda_stream
+    else:
+        torch.cuda.current_stream()  # initialises CUDA in this process
+        _raw_stream = lambda: get(dev())
+
+
+def _stream(stream=None):
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        _bind_torch()
+    return _raw_stream()
 
 
 def _ptr(t):
@@ -234,7 +255,7 @@ def _ptr(t):
         raise ValueError("expected a CUDA tensor")
     if not t.is_contiguous():
         raise ValueError("expected a contiguous tensor")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def make_grid(g) -> eb_grid:
@@ -395,9 +416,11 @@ class EB:
         return out
 
     def apply(self, x, out=None, stream=None):
-        import torch
-        prec = {torch.float64: EB_F64, torch.float32: EB_F32, torch.bfloat16: EB_BF16}[x.dtype]
+        if _apply_prec is None:
+            _bind_torch()
+        prec = _apply_prec[x.dtype]
         if out is None:
+            import torch
             out = torch.zeros_like(x)
         _check(load().eb_apply(self._h, prec, _ptr(x), _ptr(out), _stream(stream)))
         return out

@@ -138,10 +138,11 @@ void launch_apply(const EBHandle& eb, const T* x, T* y, double sigma, cudaStream
   const A inv_h2 = (A)(1.0 / (eb.g.h * eb.g.h));
   const TileView tv = eb.tv();
   dim_dispatch(eb, [&](auto D) {
-    if (tv.pair_node)
-      k_apply<T, D.value | DIM_LIST><<<blocks_for(tv.npairs, APPLY_THREADS), APPLY_THREADS, 0, s>>>(
-          tv, eb.code, diag_of<T>(eb), x, y, (A)sigma, inv_h2);
-    else
+    if (tv.pair_node) {
+      const int th = list_threads(tv.npairs);
+      k_apply<T, D.value | DIM_LIST><<<blocks_for(tv.npairs, th), th, 0, s>>>(tv, eb.code, diag_of<T>(eb), x, y,
+                                                                              (A)sigma, inv_h2);
+    } else
       k_apply<T, D.value><<<tile_grid(eb), APPLY_THREADS, 0, s>>>(tv, eb.code, diag_of<T>(eb), x, y, (A)sigma,
                                                                   inv_h2);
   });
