@@ -128,13 +128,11 @@ __global__ void __launch_bounds__(128) k_l1_fwd(Image im, const float2* __restri
 // Implicit GEMM on the 5th-generation tensor cores (kernel k_conv32_tma below).
 // The B operand, the weights, sits in shared memory in the no-swizzle K-major
 // layout of "core matrices" (8 rows x 16 bytes stored contiguously):
-// [tap][channel group g][n][8 k] (SBO = 128 B between 8-row blocks of n,
-// LBO = 32 x 16 B between channel groups).  The A operand (activations) uses the
+// [dx][channel group g][dy 32 + n][8 k] (SBO = 128 B between 8-row blocks of n,
+// LBO = 96 x 16 B between channel groups).  The A operand (activations) uses the
 // 64-byte swizzled layout written by the tensor copies (tc_desc_sw64).
 constexpr int TC_PIX = TPX + 2;                  // pixels of a job's rows with their two halo pixels
-constexpr int TC_A = 3 * TC_PIX * NC * 2;        // a job's three rows: 24,960 bytes
-constexpr int TC_WTAP = 4 * NC * 16;             // 2048 per tap
-constexpr int TC_W = 9 * TC_WTAP;                // 18,432
+constexpr int TC_W = 9 * 4 * NC * 16;            // weights of a layer: 18,432 bytes
 constexpr uint32_t TC_SPIN = 1u << 22;           // bounded mbarrier polls (~0.1 s)
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -163,33 +161,40 @@ __device__ __forceinline__ constexpr uint32_t tc_idesc(int M, int N) {
 // ------------------------- 32 -> 32 convolution, TMA-fed warp-specialised pipeline
 // y = conv(x; wk) + bias (if bias), then ReLU (if relu), then 0 where
 // mask_ref <= 0 (if mask_ref: the ReLU derivative of a data gradient).
-// wk: bf16 [9][32 (n)][32 (k)].  A job is 128 pixels of one image row and all
-// 32 output channels: M = 128, N = 32, K = 9 taps x 32 channels = 18 MMAs of
-// 128 x 32 x 16 (bf16 in, f32 in TMEM).  One thread issues, per job, one 4D
-// tensor copy (cp.async.bulk.tensor) of the job's 3 rows x 130 pixels x 32
-// channels into a ring of CP_STAGES buffers, in the 64-byte swizzled K-major
-// layout (a pixel's 32 channels are one 64-byte row); the operand of tap
-// (dy, dx) and channel half kh starts at row dy * 130 + dx, byte 32 kh.  One
-// thread issues the 18 MMAs of each job into one of two TMEM accumulators;
-// four warps drain the accumulators (tcgen05.ld: warp w reads TMEM lanes
-// 32 w .. 32 w + 31, its 32 pixels) and run the epilogue while the next jobs
-// load and multiply.  The tensor map views the activations as (32 channels,
-// pixel, row in image, image), so the rows outside an image and the pixels
-// outside a row are filled with zeros by the copy.
-// Barriers: full[s] (copy -> MMA, transaction bytes), empty[s] (MMA commit ->
-// copy), tfull[a] (MMA commit -> epilogue), tempty[a] (4 epilogue warps ->
-// MMA).  Every wait is bounded; a wait that gives up raises a shared abort
-// flag that ends every role's loop, sets *err, and the CTA waits (bounded) for
-// its copies and MMAs in flight before freeing TMEM.
-constexpr int CP_STAGES = 2;
-constexpr int CP_STAGE = 25600;                        // TC_A rounded up to 1 KB (swizzle atoms stay aligned)
-constexpr int CP_W = CP_STAGES * CP_STAGE;             // weights after the stages
+// wk: bf16 [9][32 (n)][32 (k)].  A job is 128 pixels of rb <= 4 rows of an image
+// and all 32 output channels; its rb + 2 input rows x 130 pixels x 32 channels
+// arrive in one 4D tensor copy (cp.async.bulk.tensor) in the 64-byte swizzled
+// K-major layout (a pixel's 32 channels are one 64-byte row).  The MMAs are
+// input-row stationary: input row j, shifted by dx = 0, 1, 2 pixels (an offset
+// of 64 dx bytes) and split in two channel halves, times the weights of the tap
+// rows that lead from it into the job, N = 32 per output row: rows j + 1, j, j -
+// 1 with dy = 0, 1, 2, at increasing TMEM columns.  Four rows take 39 MMAs, where
+// one output row at a time takes 72; issuing one costs its thread some 190
+// cycles whatever N, so that count and not the tensor cores bounded the earlier
+// form: 172 us a layer at 16 x 512^2 pixels on average over forward and data
+// gradient (which also reads the masks), 127 us now, 5.3 TB/s.  An output row receives its taps in
+// (dy, dx, kh) order, the first without accumulating.
+// Four MMA warps take the jobs in turn, each with a stage and a TMEM region (128
+// columns) of its own; eight epilogue warps drain a region (warp w: TMEM lanes 32
+// (w % 4) .., rows (w / 4) rb / 2 ..), the ReLU masks of a data gradient loaded
+// while the MMAs run.  One CTA per SM.  The tensor map views the activations as
+// (32 channels, pixel, row in image, image), so the rows outside an image and the
+// pixels outside a row are filled with zeros by the copy.
+// Barriers, per stage: full (copy, transaction bytes), empty (MMA commit ->
+// copy), tfull (MMA commit -> epilogue), tempty (8 epilogue warps -> MMA).  Every
+// wait is bounded; a wait that gives up raises a shared abort flag that ends
+// every role's loop, sets *err, and the CTA waits (bounded) for its copies and
+// MMAs in flight before freeing TMEM.
+constexpr int CP_ROWS = 4;                             // rows of a job at most
+constexpr int CP_STAGES = 4;
+constexpr int CP_STAGE = 50176;                        // 6 x 130 x 64 bytes rounded up to 1 KB (swizzle atoms stay aligned)
+constexpr int CP_W = CP_STAGES * CP_STAGE;             // weights after the stages: [dx][channel group][dy 32 + n][8 k]
+constexpr int CP_WDX = 4 * 96 * 16;
 constexpr int CP_BAR = CP_W + TC_W;                    // barriers after the weights
-constexpr int CP_NBAR = 2 * CP_STAGES + 4;
+constexpr int CP_NBAR = 4 * CP_STAGES;
 constexpr int CP_SMEM = CP_BAR + 8 * CP_NBAR + 16;     // + TMEM slot and abort flag
-constexpr int CP_THREADS = 192;                        // warps 0-3 epilogue, 4 copies, 5 MMAs
-constexpr uint32_t CP_BOX_BYTES = 3 * TC_PIX * NC * 2;  // 24,960
-static_assert(CP_BOX_BYTES == TC_A, "box = staged operand");
+constexpr int CP_THREADS = 13 * 32;                    // warps 0-7 epilogue, 8 copies, 9-12 MMAs
+static_assert((CP_ROWS + 2) * TC_PIX * NC * 2 <= CP_STAGE && CP_STAGE % 1024 == 0 && CP_SMEM <= 227 * 1024, "conv stage");
 
 __device__ __forceinline__ bool cp_wait(uint32_t bar, uint32_t parity, volatile int* abort) {
   for (uint32_t it = 0; it < TC_SPIN; ++it) {
@@ -206,37 +211,36 @@ __device__ __forceinline__ bool cp_wait(uint32_t bar, uint32_t parity, volatile 
   return false;
 }
 
-__global__ void __launch_bounds__(CP_THREADS, 3) k_conv32_tma(const __grid_constant__ CUtensorMap xmap, Image im,
-                                                               const bf16* __restrict__ wk,
+__global__ void __launch_bounds__(CP_THREADS, 1) k_conv32_tma(const __grid_constant__ CUtensorMap xmap, Image im,
+                                                               int rb, const bf16* __restrict__ wk,
                                                                const float* __restrict__ bias, bf16* __restrict__ y,
                                                                int relu, const bf16* __restrict__ mask_ref,
                                                                int* __restrict__ err) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  unsigned char* sW = smem_raw + CP_W;
   const uint32_t base = smem_addr(smem_raw);
-  const uint32_t a0 = base, w0 = base + CP_W, bars = base + CP_BAR;
+  const uint32_t w0 = base + CP_W, bars = base + CP_BAR;
   auto full = [&](int st) { return bars + 8 * st; };
   auto empty = [&](int st) { return bars + 8 * (CP_STAGES + st); };
-  auto tfull = [&](int a) { return bars + 8 * (2 * CP_STAGES + a); };
-  auto tempty = [&](int a) { return bars + 8 * (2 * CP_STAGES + 2 + a); };
+  auto tfull = [&](int st) { return bars + 8 * (2 * CP_STAGES + st); };
+  auto tempty = [&](int st) { return bars + 8 * (3 * CP_STAGES + st); };
   uint32_t* tslot = reinterpret_cast<uint32_t*>(smem_raw + CP_BAR + 8 * CP_NBAR);
   volatile int* abort = reinterpret_cast<volatile int*>(smem_raw + CP_BAR + 8 * CP_NBAR + 8);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   for (int i = tid; i < 9 * NC * 4; i += CP_THREADS) {  // weights once per CTA
     const int g = i & 3, n = (i >> 2) % NC, d = (i >> 2) / NC;
-    *reinterpret_cast<int4*>(sW + d * TC_WTAP + g * (NC * 16) + n * 16) =
+    *reinterpret_cast<int4*>(smem_raw + CP_W + (d % 3) * CP_WDX + g * (96 * 16) + ((d / 3) * NC + n) * 16) =
         *reinterpret_cast<const int4*>(wk + (d * NC + n) * NC + g * 8);
   }
   if (tid == 0) {
     for (int b = 0; b < CP_NBAR; ++b) {
-      const uint32_t cnt = (b >= 2 * CP_STAGES + 2) ? 4u : 1u;  // tempty: one arrive per epilogue warp
+      const uint32_t cnt = b >= 3 * CP_STAGES ? 8u : 1u;  // tempty: one arrive per epilogue warp
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bars + 8 * b), "r"(cnt));
     }
     *abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
-  if (warp == 5) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 64;" ::"r"(smem_addr(tslot)));
+  if (warp == 9) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_addr(tslot)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   asm volatile("fence.proxy.async.shared::cta;");  // weights (generic stores) are read by the tensor cores
@@ -244,13 +248,14 @@ __global__ void __launch_bounds__(CP_THREADS, 3) k_conv32_tma(const __grid_const
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = *tslot;
-  const int segs = (im.W + TPX - 1) / TPX;
-  const int64_t jobs = (int64_t)segs * im.H;
+  const int segs = (im.W + TPX - 1) / TPX, chunks = (im.R + rb - 1) / rb;
+  const int64_t jobs = (int64_t)segs * chunks * (im.H / im.R);
   const int64_t njob = jobs > (int64_t)blockIdx.x ? (jobs - 1 - blockIdx.x) / gridDim.x + 1 : 0;  // this CTA's jobs
-  if (warp == 4) {
+  if (warp == 8) {
     // copies: stage s = k mod S, its u-th use waits for the MMAs of use u - 1
     if (lane == 0) {
       const uint64_t map = reinterpret_cast<uint64_t>(&xmap);
+      const uint32_t bytes = (uint32_t)((rb + 2) * TC_PIX * NC * 2);
       asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
       int64_t k = 0;
       for (; k < njob; ++k) {
@@ -258,14 +263,13 @@ __global__ void __launch_bounds__(CP_THREADS, 3) k_conv32_tma(const __grid_const
         const uint32_t u = (uint32_t)(k / CP_STAGES);
         if (u > 0 && !cp_wait(empty(st), (u - 1) & 1u, abort)) break;
         const int64_t job = blockIdx.x + k * gridDim.x;
-        const int r = (int)(job / segs), x0 = (int)(job % segs) * TPX;
-        const int img = r / im.R, rin = r - img * im.R;
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full(st)), "r"(CP_BOX_BYTES)
-                     : "memory");
+        const int x0 = (int)(job % segs) * TPX, r0 = (int)((job / segs) % chunks) * rb;
+        const int img = (int)(job / ((int64_t)segs * chunks));
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full(st)), "r"(bytes) : "memory");
         asm volatile(
             "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
-            "%5}], [%6];" ::"r"(a0 + st * CP_STAGE),
-            "l"(map), "r"(0), "r"(x0 - 1), "r"(rin - 1), "r"(img), "r"(full(st))
+            "%5}], [%6];" ::"r"(base + st * CP_STAGE),
+            "l"(map), "r"(0), "r"(x0 - 1), "r"(r0 - 1), "r"(img), "r"(full(st))
             : "memory");
       }
       // copies still in flight (an aborted run) land before the CTA ends
@@ -274,94 +278,134 @@ __global__ void __launch_bounds__(CP_THREADS, 3) k_conv32_tma(const __grid_const
         cp_wait(full((int)(q % CP_STAGES)), (uint32_t)(q / CP_STAGES) & 1u, &never);
       }
     }
-  } else if (warp == 5) {
+  } else if (warp > 8) {
     if (lane == 0) {
-      constexpr uint32_t idesc = tc_idesc(128, NC);
-      int64_t k = 0;
-      for (; k < njob; ++k) {
-        const int st = (int)(k % CP_STAGES);
-        const int a = (int)(k & 1);
-        if (!cp_wait(full(st), (uint32_t)(k / CP_STAGES) & 1u, abort)) break;
-        if (k >= 2 && !cp_wait(tempty(a), (uint32_t)((k >> 1) - 1) & 1u, abort)) break;
+      const int st = warp - 9;  // this warp's stage and TMEM region: jobs st, st + 4, ...
+      uint32_t u = 0;
+      for (int64_t k = st; k < njob; k += CP_STAGES, ++u) {
+        if (!cp_wait(full(st), u & 1u, abort)) break;
+        if (u > 0 && !cp_wait(tempty(st), (u - 1) & 1u, abort)) break;
         asm volatile("tcgen05.fence::after_thread_sync;");
-        const uint32_t sa = a0 + st * CP_STAGE;
-#pragma unroll 1
-        for (int q = 0; q < 18; ++q) {
-          const int d = q >> 1, kh = q & 1, dy = d / 3, dx = d % 3;
-          const uint64_t da = tc_desc_sw64(sa + (dy * TC_PIX + dx) * 64 + kh * 32);
-          const uint64_t db = tc_desc(w0 + d * TC_WTAP + (2 * kh) * (NC * 16), NC * 16, 128);
+        const uint32_t sa = base + st * CP_STAGE, region = tmem + (uint32_t)(128 * st);
+        auto mma = [&](uint32_t dst, uint64_t da, uint32_t sb, int n, uint32_t acc) {
+          const uint64_t db = tc_desc(sb, 96 * 16, 128);
           asm volatile(
               "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-              "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem + (uint32_t)(a * NC)),
-              "l"(da), "l"(db), "r"(idesc), "r"((uint32_t)(q > 0)));
+              "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(dst),
+              "l"(da), "l"(db), "r"(tc_idesc(128, n)), "r"(acc));
+        };
+#pragma unroll 1
+        for (int j = -1; j <= rb; ++j) {
+          // tap rows dl .. dh lead from input row j to the job's rows j + 1 - dy;
+          // row r accumulates at columns 32 (rb - 1 - r)
+          const int dl = j + 1 > rb - 1 ? j + 2 - rb : 0, dh = j + 1 < 2 ? j + 1 : 2;
+          const uint32_t dst = region + (uint32_t)(32 * (rb - 2 - j + dl));
+#pragma unroll 1
+          for (int q = 0; q < 6; ++q) {
+            const int dx = q >> 1, kh = q & 1;
+            const uint64_t da = tc_desc_sw64(sa + ((j + 1) * TC_PIX + dx) * 64 + kh * 32);
+            const uint32_t sb = w0 + dx * CP_WDX + (2 * kh) * (96 * 16) + dl * (NC * 16);
+            if (q == 0 && dl == 0) {  // row j + 1 starts here
+              mma(dst, da, sb, NC, 0u);
+              if (dh > 0) mma(dst + 32, da, sb + NC * 16, NC * dh, 1u);
+            } else {
+              mma(dst, da, sb, NC * (dh - dl + 1), 1u);
+            }
+          }
         }
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(empty(st))
                      : "memory");
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(tfull(a))
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(tfull(st))
                      : "memory");
       }
-      if (k > 0) {  // the last MMAs complete before TMEM is freed
+      if (u > 0) {  // the last MMAs complete before TMEM is freed
         volatile int never = 0;
-        cp_wait(tfull((int)((k - 1) & 1)), (uint32_t)(((k - 1) >> 1) & 1), &never);
+        cp_wait(tfull(st), (u - 1) & 1u, &never);
       }
     }
   } else {
-    // epilogue: warp w drains TMEM lanes 32 w .. 32 w + 31 (pixels x0 + 32 w + lane)
+    // epilogue: warp w drains TMEM lanes 32 (w % 4) .. (pixels x0 + 32 (w % 4) +
+    // lane) of rows (w / 4) half .. of each job
+    const int half = (rb + 1) >> 1, q0 = (warp >> 2) * half, q1 = min(q0 + half, rb);
     float bv[NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) bv[c] = bias ? bias[c] : 0.0f;
     for (int64_t k = 0; k < njob; ++k) {
-      const int a = (int)(k & 1);
+      const int st = (int)(k % CP_STAGES);
+      const int64_t job = blockIdx.x + k * gridDim.x;
+      const int gx = (int)(job % segs) * TPX + (warp & 3) * 32 + lane, r0 = (int)((job / segs) % chunks) * rb;
+      const int img = (int)(job / ((int64_t)segs * chunks));
+      const int64_t p0 = ((int64_t)img * im.R + r0) * im.W + gx;
+      uint4 mr[2][4];  // the masks of this warp's rows (at most two), on their way during the MMAs
+      if (mask_ref)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const bool on = q0 + h < q1 && r0 + q0 + h < im.R && gx < im.W;
+          const uint4* src = reinterpret_cast<const uint4*>(mask_ref + (on ? p0 + (int64_t)(q0 + h) * im.W : 0) * NC);
+#pragma unroll
+          for (int c = 0; c < 4; ++c) mr[h][c] = __ldg(src + c);
+        }
       // the warp leaves together or not at all (tcgen05.ld is warp-collective)
-      const bool okl = cp_wait(tfull(a), (uint32_t)(k >> 1) & 1u, abort);
+      const bool okl = cp_wait(tfull(st), (uint32_t)(k / CP_STAGES) & 1u, abort);
       if (!__all_sync(0xffffffffu, okl)) {
         *abort = 1;
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;");
-      uint32_t v[NC];
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,"
-          "%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-          : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-            "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-            "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-            "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-          : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(a * NC)));
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      asm volatile("tcgen05.fence::before_thread_sync;");
-      __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty(a)) : "memory");
-      const int64_t job = blockIdx.x + k * gridDim.x;
-      const int r = (int)(job / segs), x0 = (int)(job % segs) * TPX;
-      const int gx = x0 + warp * 32 + lane;
-      if (gx < im.W) {
-        const int64_t p = (int64_t)r * im.W + gx;
-        __align__(16) bf16 ov[NC];
-        __align__(16) bf16 mr[NC];
-        if (mask_ref) {
 #pragma unroll
-          for (int q = 0; q < 4; ++q)
-            reinterpret_cast<int4*>(mr)[q] = reinterpret_cast<const int4*>(mask_ref + p * NC)[q];
+      for (int h = 0; h < 2; ++h) {
+        const int r = q0 + h;
+        if (r >= q1) break;
+        uint32_t v[NC];
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,"
+            "%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+              "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
+              "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
+              "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+            : "r"(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(128 * st + 32 * (rb - 1 - r))));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (r + 1 == q1) {  // this warp's last read of the region
+          asm volatile("tcgen05.fence::before_thread_sync;");
+          __syncwarp();
+          if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty(st)) : "memory");
         }
+        if (gx < im.W && r0 + r < im.R) {
+          uint32_t o[NC / 2];
+          const uint32_t* m = reinterpret_cast<const uint32_t*>(mr[h]);
 #pragma unroll
-        for (int co = 0; co < NC; ++co) {
-          float f = __uint_as_float(v[co]) + bv[co];
-          if (relu) f = fmaxf(f, 0.0f);
-          if (mask_ref && !(__bfloat162float(mr[co]) > 0.0f)) f = 0.0f;
-          ov[co] = __float2bfloat16_rn(f);
+          for (int c = 0; c < NC; c += 2) {
+            float f0 = __uint_as_float(v[c]) + bv[c], f1 = __uint_as_float(v[c + 1]) + bv[c + 1];
+            if (relu) {
+              f0 = fmaxf(f0, 0.0f);
+              f1 = fmaxf(f1, 0.0f);
+            }
+            if (mask_ref) {
+              const uint32_t w = m[c / 2];
+              if (!(__uint_as_float(w << 16) > 0.0f)) f0 = 0.0f;
+              if (!(__uint_as_float(w & 0xFFFF0000u) > 0.0f)) f1 = 0.0f;
+            }
+            const __nv_bfloat162 hv = __floats2bfloat162_rn(f0, f1);
+            o[c / 2] = *reinterpret_cast<const uint32_t*>(&hv);
+          }
+          uint4* dst = reinterpret_cast<uint4*>(y + (p0 + (int64_t)r * im.W) * NC);
+#pragma unroll
+          for (int c = 0; c < 4; ++c) dst[c] = make_uint4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
         }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) reinterpret_cast<int4*>(y + p * NC)[q] = reinterpret_cast<const int4*>(ov)[q];
+      }
+      if (q0 >= q1) {  // rb = 1: the second half of the warps has no row
+        __syncwarp();
+        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty(st)) : "memory");
       }
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   if (tid == 0 && *abort) atomicExch(err, 1);
-  if (warp == 5) {
+  if (warp == 9) {
     asm volatile("tcgen05.fence::after_thread_sync;");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 64;" ::"r"(tmem));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
   }
 }
 
@@ -420,7 +464,7 @@ __global__ void k_l6_fwd(Image im, const bf16* __restrict__ y5, const float* __r
 //     columns; runs of adjacent slots take one MMA per (dx, kh), so a layer
 //     issues 6 MMAs per step (12 when the three slots wrap), a third of the
 //     18 of the output-stationary form.  The slot of row rho receives its taps
-//     in (dy, dx, kh) order, the order of k_conv32_tma's 18 MMAs, from zero.
+//     in (dy, dx, kh) order, as in k_conv32_tma, from zero.
 //   * epilogues of layers 2-4 (warps 0-3, one TMEM lane = one pixel per
 //     thread): read the finished slot of row rho and zero it for row rho + 4,
 //     bias, ReLU, bf16, 0 outside the image (the next layer's zero padding),
@@ -1770,9 +1814,9 @@ static void set_attrs() {
 
 // Tensor map of a BF16 NHWC activation stack: dimensions (32 channels, pixel,
 // row in image, image), strides 64 B, W * 64 B, R * W * 64 B; box (32, px,
-// rows, 1), k_conv32_tma's by default, written in the 64-byte swizzled layout;
+// rows, 1) written in the 64-byte swizzled layout;
 // out-of-range elements read as zero.
-static CUtensorMap conv_map(const bf16* x, const Image& im, int px = TC_PIX, int rows = 3) {
+static CUtensorMap conv_map(const bf16* x, const Image& im, int px, int rows) {
   EB_REQUIRE(((uintptr_t)x & 15) == 0, EB_ERR_INVALID, "conv: activations not 16-byte aligned");
   EB_REQUIRE(im.R > 0 && im.H % im.R == 0, EB_ERR_INVALID, "conv: rows are not whole images");
   CUtensorMap m;
@@ -1788,13 +1832,15 @@ static CUtensorMap conv_map(const bf16* x, const Image& im, int px = TC_PIX, int
   return m;
 }
 
-// y = conv(x; wk) (+ bias, ReLU, mask) through k_conv32_tma
+// y = conv(x; wk) (+ bias, ReLU, mask) through k_conv32_tma: jobs of four rows,
+// or of two or one where four would not give every SM two of them
 static void conv32(const Image& im, const bf16* x, const bf16* wk, const float* bias, bf16* y, int relu,
                    const bf16* mask_ref, int* err, cudaStream_t s) {
-  const CUtensorMap m = conv_map(x, im);
-  const int64_t jobs = (int64_t)((im.W + TPX - 1) / TPX) * im.H;
-  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(jobs, (int64_t)num_sms() * 3));
-  k_conv32_tma<<<grid, CP_THREADS, CP_SMEM, s>>>(m, im, wk, bias, y, relu, mask_ref, err);
+  auto jobs = [&](int rb) { return (int64_t)((im.W + TPX - 1) / TPX) * ((im.R + rb - 1) / rb) * (im.H / im.R); };
+  const int rb = jobs(4) >= 2 * num_sms() ? 4 : (jobs(2) >= 2 * num_sms() ? 2 : 1);
+  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(jobs(rb), num_sms()));
+  k_conv32_tma<<<grid, CP_THREADS, CP_SMEM, s>>>(conv_map(x, im, TC_PIX, rb + 2), im, rb, wk, bias, y, relu, mask_ref,
+                                                 err);
 }
 
 static void ensure_act(NN& N, int64_t px, cudaStream_t s) {
