@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(TILE_NODES) k_g_cheb_step(TileView tv, const u
     const A res1 = inv_diag_t<A>(k1, diag, node + 1, ot) * (bv.y - (core.y * ot.inv_h2 + ot.sigma * xc.y));
     const A d0 = (k0 & CODE_CP) ? c1 * dv.x + c2 * res0 : (A)0;
     const A d1 = (k1 & CODE_CP) ? c1 * dv.y + c2 * res1 : (A)0;
-    st2o(d + node, d0, d1);
+    if constexpr (DOT == 0) st2o(d + node, d0, d1);  // the launch that forms z is a cycle's last: d ends there
     const A z0 = (k0 & CODE_CP) ? xc.x + d0 : (A)0, z1 = (k1 & CODE_CP) ? xc.y + d1 : (A)0;
     st2(xo + node, z0, z1);
     if constexpr (DOT == 1) {
@@ -376,6 +376,113 @@ __global__ void __launch_bounds__(TILE_NODES) k_g_cheb_step(TileView tv, const u
     __shared__ DF dsm[32];
     const DF a = df_block_sum_df(srz_df, dsm);
     if (threadIdx.x == 0) df_part_store(part, blockIdx.x, a);
+  }
+}
+
+// The batched DF iteration's x/r update (k_b_update_xr_df of the PCG: x += alpha
+// p, r -= alpha q in DF, per-tile DF partials r.r and r.zold as pairs, tiles of
+// converged geometries skipped) with the V-cycle's first level-0 step on the
+// new r's FP32 high part while it is in registers: saves a pass over r (64
+// stars: 65 + 27 us as two launches)
+template <class V>
+__global__ void __launch_bounds__(PAIR_THREADS) k_b_update_first_df(TileView tv, BatchUpdate u,
+                                                                    const uint8_t* __restrict__ code,
+                                                                    const typename DiagOf<V>::type* __restrict__ diag,
+                                                                    GOp<float> o, V* __restrict__ b_out,
+                                                                    V* __restrict__ x0, V* __restrict__ d,
+                                                                    float inv_theta) {
+  __shared__ DF dsm[PAIR_THREADS / 32];
+  __shared__ DF s_a;
+  double* const x = u.sc->x;
+  for (int64_t tt = blockIdx.x; tt < tv.ntiles; tt += gridDim.x) {
+    const PcgScalars& S = u.sc[u.tile_geo[tt]];
+    if (S.done) continue;
+    __syncthreads();  // s_a of the previous tile is read
+    if (threadIdx.x == 0) s_a = df_from_double(S.alpha);
+    __syncthreads();
+    const DF a = s_a;
+    int32_t node;
+    DF srr{0.0f, 0.0f}, srzo{0.0f, 0.0f};
+    if (tile_pair<2>(tv, tt, threadIdx.x, node)) {
+      DF r0, r1, q0, q1, p0, p1, xa, xb;
+      df_ld2_rw(u.r, node, r0, r1);
+      df_ld2(u.q, node, q0, q1);
+      df_ld2(u.p, node, p0, p1);
+      df_ld2_rw(x, node, xa, xb);
+      const float2 zv = __ldg(reinterpret_cast<const float2*>(u.z + node));
+      uint32_t c0, c1;
+      ld_codes(code, node, c0, c1);
+      r0 = df_sub(r0, df_mul(a, q0));
+      r1 = df_sub(r1, df_mul(a, q1));
+      df_st2(x, node, df_add_fast(xa, df_mul(a, p0)), df_add_fast(xb, df_mul(a, p1)));
+      df_st2(u.r, node, r0, r1);
+      df_acc_prod(srr, r0, r0);
+      df_acc_prod(srr, r1, r1);
+      df_acc_prod_f(srzo, r0, zv.x);
+      df_acc_prod_f(srzo, r1, zv.y);
+      const GOp<float> ot = tile_op(tv, tt, o);
+      const float b0 = (c0 & CODE_CP) ? r0.hi : 0.0f, b1 = (c1 & CODE_CP) ? r1.hi : 0.0f;
+      st2o(b_out + node, b0, b1);
+      const float v0 = (c0 & CODE_CP) ? inv_diag_t<float>(c0, diag, node, ot) * b0 * inv_theta : 0.0f;
+      const float v1 = (c1 & CODE_CP) ? inv_diag_t<float>(c1, diag, node + 1, ot) * b1 * inv_theta : 0.0f;
+      st2o(x0 + node, v0, v1);
+      st2o(d + node, v0, v1);
+    }
+    const DF t = df_block_sum_df(srr, dsm);
+    const DF w = df_block_sum_df(srzo, dsm);
+    if (threadIdx.x == 0) {
+      df_part_store(u.part, 2 * tt, t);
+      df_part_store(u.part, 2 * tt + 1, w);
+    }
+  }
+}
+
+// The last level-0 step of a batched V-cycle for the DF iteration: z in FP32 on
+// every node of the tiles and, per tile, the DF partial r.z (pairs (r.z, 0));
+// k_g_cheb_step's arithmetic.  Two tiles per CTA and pass, each reduced by its
+// 128 threads (a named barrier each; the slots alternate, so one barrier per
+// tile).  Saves the dot's own pass over r and z (64 stars: 25 us).
+template <class V>
+__global__ void __launch_bounds__(TILE_NODES) k_g_cheb_last_df(TileView tv, const uint8_t* __restrict__ code,
+                                                               const typename DiagOf<V>::type* __restrict__ diag,
+                                                               GOp<float> o, const V* __restrict__ b,
+                                                               const V* __restrict__ x, float* __restrict__ z,
+                                                               const V* __restrict__ d, float c1, float c2,
+                                                               const double* __restrict__ r, double* __restrict__ part) {
+  __shared__ DF dsm[2][2][4];
+  const int half = threadIdx.x >> 7, t = threadIdx.x & 127;
+  int it = 0;
+  for (int64_t tt = 2 * (int64_t)blockIdx.x + half; tt < tv.ntiles; tt += 2 * (int64_t)gridDim.x, ++it) {
+    int32_t node;
+    DF s{0.0f, 0.0f};
+    if (tile_pair<2>(tv, tt, t, node)) {
+      const GOp<float> ot = tile_op(tv, tt, o);
+      uint32_t k0, k1;
+      ld_codes(code, node, k0, k1);
+      Two<float> xc, core;
+      stencil_tv<2, LdRO>(tv, x, node, k0, k1, diag, xc, core);
+      const Two<float> bv = LdRO::ld2(b + node);
+      Two<float> dv{0, 0};
+      if (c1 != 0.0f) dv = LdRO::ld2(d + node);
+      DF ra, rb;
+      df_ld2(r, node, ra, rb);
+      const float res0 = inv_diag_t<float>(k0, diag, node, ot) * (bv.x - (core.x * ot.inv_h2 + ot.sigma * xc.x));
+      const float res1 = inv_diag_t<float>(k1, diag, node + 1, ot) * (bv.y - (core.y * ot.inv_h2 + ot.sigma * xc.y));
+      const float z0 = (k0 & CODE_CP) ? xc.x + (c1 * dv.x + c2 * res0) : 0.0f;
+      const float z1 = (k1 & CODE_CP) ? xc.y + (c1 * dv.y + c2 * res1) : 0.0f;
+      st2(z + node, z0, z1);
+      df_acc_prod_f(s, ra, z0);
+      df_acc_prod_f(s, rb, z1);
+    }
+    for (int w = 16; w > 0; w >>= 1)
+      s = df_add(s, DF{__shfl_xor_sync(0xffffffffu, s.hi, w), __shfl_xor_sync(0xffffffffu, s.lo, w)});
+    if ((t & 31) == 0) dsm[half][it & 1][t >> 5] = s;
+    asm volatile("bar.sync %0, 128;" ::"r"(1 + half) : "memory");
+    if (t == 0) {
+      const DF* q = dsm[half][it & 1];
+      df_part_store(part, 2 * tt, df_add(df_add(df_add(q[0], q[1]), q[2]), q[3]));
+      df_part_store(part, 2 * tt + 1, DF{0.0f, 0.0f});
+    }
   }
 }
 
@@ -1292,7 +1399,11 @@ static int vcycle_grid(Solver& S, const double* r, double* z, cudaStream_t s, co
       k_g_cheb_step<DIM, V, float, 2><<<gd, th, 0, s>>>(tv, eb.code, diag, o, b, x,
                                                                 reinterpret_cast<float*>(z), g.d, (A)cc.c1[k],
                                                                 (A)cc.c2[k], dot->r, dot->part);
-    else if (k == cc.deg - 1 && rdf)  // z in FP32 on every node of the active tiles, 0 off the CPs
+    else if (k == cc.deg - 1 && rdf && dot->tile_part) {  // batched: with the per-tile r'z partials
+      if constexpr (!std::is_same<V, double>::value && dim_of(DIM) == 2 && (DIM & (DIM_VB | DIM_LIST)) == 0)
+        k_g_cheb_last_df<V><<<gb, TILE_NODES, 0, s>>>(tv, eb.code, diag, o, b, x, reinterpret_cast<float*>(z), g.d,
+                                                      (A)cc.c1[k], (A)cc.c2[k], dot->r, dot->tile_part);
+    } else if (k == cc.deg - 1 && rdf)  // z in FP32 on every node of the active tiles, 0 off the CPs
       k_g_cheb_step<(DIM & ~DIM_LIST), V, float><<<gb, TILE_NODES, 0, s>>>(
           tiles_only(tv), eb.code, diag, o, b, x, reinterpret_cast<float*>(z), g.d, (A)cc.c1[k], (A)cc.c2[k]);
     else if (k == cc.deg - 1 && dot)
@@ -1351,6 +1462,21 @@ static void update_first(Solver& S, const PcgUpdate& u, cudaStream_t s) {
   }
   k_update_first<DIM, V><<<(unsigned)u.nblk, S.iter_threads(), 0, s>>>(eb.pairs(), u, eb.code, diag_of<V>(eb), o, bcopy,
                                                                  g.x, g.d, DivBy{cc.theta, 1.0 / cc.theta});
+}
+
+template <class V>
+static void batch_update_first(Solver& S, const BatchUpdate& u, unsigned grid, cudaStream_t s) {
+  const EBHandle& eb = *S.eb;
+  const ChebCoef cc = cheb_coef(S.H->L[0].rho, S.opts.cheb_degree);
+  VecSet<V>& g = LevelView<V>::grid(*S.H);
+  k_b_update_first_df<V><<<grid, PAIR_THREADS, 0, s>>>(eb.tv(), u, eb.code, diag_of<V>(eb), grid_op<float>(S), g.b, g.x,
+                                                       g.d, (float)(1.0 / cc.theta));
+}
+
+void amg_batch_update_first(Solver& S, const BatchUpdate& u, unsigned grid, cudaStream_t s) {
+  if (S.opts.vcycle_prec == EB_F32) batch_update_first<float>(S, u, grid, s);
+  else batch_update_first<__nv_bfloat16>(S, u, grid, s);
+  EB_CUDA(cudaGetLastError());
 }
 
 int amg_levels(const Solver& S) { return S.H ? (int)S.H->L.size() : 0; }

@@ -36,6 +36,10 @@ constexpr int BT = PAIR_THREADS;  // one tile per CTA of 128 threads
 
 struct GeoConst {
   double h2, dt, theta;
+  double inv_dt, s, w;  // 1 / dt, h2 / theta, (1 - theta) / theta: no FP64 division per node
+  static GeoConst make(double h2, double dt, double theta) {
+    return GeoConst{h2, dt, theta, 1.0 / dt, h2 / theta, (1.0 - theta) / theta};
+  }
 };
 
 struct Batch {
@@ -181,7 +185,7 @@ static void build_batch(Batch& B, const eb_grid* grids, const eb_levelset* lss, 
   EB_CUDA(cudaMemcpyAsync(B.cut_off_cp + ncp, &ncut32, 4, cudaMemcpyHostToDevice, s));
   B.gconst = dalloc<GeoConst>(count, s);
   B.hconst.resize(count);
-  for (int g = 0; g < count; ++g) B.hconst[g] = GeoConst{grids[g].h * grids[g].h, 1.0, 1.0};
+  for (int g = 0; g < count; ++g) B.hconst[g] = GeoConst::make(grids[g].h * grids[g].h, 1.0, 1.0);
   EB_CUDA(cudaMemcpyAsync(B.gconst, B.hconst.data(), sizeof(GeoConst) * count, cudaMemcpyHostToDevice, s));
   B.sc = dalloc<PcgScalars>(count, s);
   EB_CUDA(cudaMallocHost((void**)&B.sc_host, sizeof(PcgScalars) * count));
@@ -295,17 +299,8 @@ __global__ void __launch_bounds__(BT) k_b_rhs(TileView tv, const int32_t* tile_g
 }
 
 // ------------------------------------------------------------ batched PCG
-__device__ __forceinline__ double tile_sum(double v, double* sm) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) sm[w] = v;
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x == 0)
-    for (int i = 0; i < BT / 32; ++i) s += sm[i];
-  return s;
-}
+// sum over the tile's CTA (block_sum: one warp adds; sm: BT doubles)
+__device__ __forceinline__ double tile_sum(double v, double* sm) { return block_sum(v, sm); }
 
 // unit-spacing operator with the tile's shift: (sigma' + D) x - sum of CP neighbours
 __device__ __forceinline__ void b_op(const TileView& tv, int64_t tt, const double* x, int32_t node, uint32_t c0,
@@ -320,7 +315,7 @@ __device__ __forceinline__ void b_op(const TileView& tv, int64_t tt, const doubl
 // r = b - B x; per-tile partials (b.b, r.r)
 __global__ void __launch_bounds__(BT) k_b_resid(TileView tv, const uint8_t* code, const double* diag, const double* b,
                                                 const double* x, double* r, double* part) {
-  __shared__ double sm[BT / 32];
+  __shared__ double sm[BT];
   for (int64_t tt = blockIdx.x; tt < tv.ntiles; tt += gridDim.x) {
     int32_t node;
     double sbb = 0.0, srr = 0.0;
@@ -355,7 +350,7 @@ __global__ void __launch_bounds__(BT) k_b_resid(TileView tv, const uint8_t* code
 __global__ void __launch_bounds__(BT) k_b_xpby_apply(TileView tv, const int32_t* tile_geo, const PcgScalars* sc,
                                                      const uint8_t* code, const double* diag, const double* z,
                                                      double* p, double* q, int first, double* part) {
-  __shared__ double sm[BT / 32];
+  __shared__ double sm[BT];
   for (int64_t tt = blockIdx.x; tt < tv.ntiles; tt += gridDim.x) {
     const PcgScalars& S = sc[tile_geo[tt]];
     if (S.done) continue;
@@ -392,7 +387,7 @@ __global__ void __launch_bounds__(BT) k_b_xpby_apply(TileView tv, const int32_t*
 __global__ void __launch_bounds__(BT) k_b_update_xr(TileView tv, const int32_t* tile_geo, const PcgScalars* sc,
                                                     double* r, const double* p, const double* q,
                                                     const double* z, double* part) {
-  __shared__ double sm[BT / 32];
+  __shared__ double sm[BT];
   double* const x = sc->x;
   for (int64_t tt = blockIdx.x; tt < tv.ntiles; tt += gridDim.x) {
     const PcgScalars& S = sc[tile_geo[tt]];
@@ -428,7 +423,7 @@ __global__ void __launch_bounds__(BT) k_b_update_xr(TileView tv, const int32_t* 
 // FIN_RZ0 / FIN_BETA)
 __global__ void __launch_bounds__(BT) k_b_dot(TileView tv, const int32_t* tile_geo, const PcgScalars* sc,
                                               const double* r, const double* z, double* part) {
-  __shared__ double sm[BT / 32];
+  __shared__ double sm[BT];
   for (int64_t tt = blockIdx.x; tt < tv.ntiles; tt += gridDim.x) {
     if (sc[tile_geo[tt]].done) continue;
     int32_t node;
@@ -470,11 +465,11 @@ __global__ void __launch_bounds__(BT) k_b_heat_rhs(TileView tv, const int32_t* t
     Two<double> uc, core;
     stencil_pair<2, LdRO>(u, node, tv.nn, c0, c1, diag, tv.sy, tv.sz, uc, core);
     const Two<double> v1 = LdRO::ld2(b1 + node);
-    const double s = c.h2 / c.theta;
-    double r0 = s * (uc.x / c.dt + c.theta * v1.x), r1 = s * (uc.y / c.dt + c.theta * v1.y);
+    const double s = c.s;
+    double r0 = s * (uc.x * c.inv_dt + c.theta * v1.x), r1 = s * (uc.y * c.inv_dt + c.theta * v1.y);
     if (c.theta < 1.0) {
       const Two<double> v0 = LdRO::ld2(b0 + node);
-      const double w = (1.0 - c.theta) / c.theta;
+      const double w = c.w;
       r0 += s * (1.0 - c.theta) * v0.x - w * core.x;
       r1 += s * (1.0 - c.theta) * v0.y - w * core.y;
     }
@@ -488,77 +483,6 @@ __global__ void __launch_bounds__(BT) k_b_heat_rhs(TileView tv, const int32_t* t
 // (in the slots of the doubles), as the single-grid DF iteration: every vector
 // operation on the FP32 pipe with error-free transformations.  A tile's
 // scalars (alpha or beta, the shift sigma') are split into DF once per tile.
-
-// x += alpha p, r -= alpha q in DF; per-tile DF partials r.r and, with z
-// (flexible CG), r.zold as pairs, else r.r alone (k_b_update_xr's layout)
-__global__ void __launch_bounds__(BT) k_b_update_xr_df(TileView tv, const int32_t* tile_geo, const PcgScalars* sc,
-                                                       double* r, const double* p, const double* q,
-                                                       const float* z, double* part) {
-  __shared__ DF dsm[BT / 32];
-  __shared__ DF s_a;
-  double* const x = sc->x;
-  for (int64_t tt = blockIdx.x; tt < tv.ntiles; tt += gridDim.x) {
-    const PcgScalars& S = sc[tile_geo[tt]];
-    if (S.done) continue;
-    __syncthreads();  // s_a of the previous tile is read
-    if (threadIdx.x == 0) s_a = df_from_double(S.alpha);
-    __syncthreads();
-    const DF a = s_a;
-    int32_t node;
-    DF srr{0.0f, 0.0f}, srzo{0.0f, 0.0f};
-    if (tile_pair<2>(tv, tt, threadIdx.x, node)) {
-      DF r0, r1, q0, q1, p0, p1, xa, xb;
-      df_ld2_rw(r, node, r0, r1);
-      df_ld2(q, node, q0, q1);
-      df_ld2(p, node, p0, p1);
-      df_ld2_rw(x, node, xa, xb);
-      r0 = df_sub(r0, df_mul(a, q0));
-      r1 = df_sub(r1, df_mul(a, q1));
-      df_st2(x, node, df_add_fast(xa, df_mul(a, p0)), df_add_fast(xb, df_mul(a, p1)));
-      df_st2(r, node, r0, r1);
-      df_acc_prod(srr, r0, r0);
-      df_acc_prod(srr, r1, r1);
-      if (z) {
-        const float2 zv = __ldg(reinterpret_cast<const float2*>(z + node));
-        df_acc_prod_f(srzo, r0, zv.x);
-        df_acc_prod_f(srzo, r1, zv.y);
-      }
-    }
-    const DF t = df_block_sum_df(srr, dsm);
-    if (z) {
-      const DF u = df_block_sum_df(srzo, dsm);
-      if (threadIdx.x == 0) {
-        df_part_store(part, 2 * tt, t);
-        df_part_store(part, 2 * tt + 1, u);
-      }
-    } else if (threadIdx.x == 0) {
-      df_part_store(part, tt, t);
-    }
-  }
-}
-
-// per-tile DF partials r.z (pairs (r.z, 0)) for r in DF and the FP32 z
-__global__ void __launch_bounds__(BT) k_b_dot_df(TileView tv, const int32_t* tile_geo, const PcgScalars* sc,
-                                                 const double* r, const float* z, double* part) {
-  __shared__ DF dsm[BT / 32];
-  for (int64_t tt = blockIdx.x; tt < tv.ntiles; tt += gridDim.x) {
-    if (sc[tile_geo[tt]].done) continue;
-    int32_t node;
-    DF a{0.0f, 0.0f};
-    if (tile_pair<2>(tv, tt, threadIdx.x, node)) {
-      DF r0, r1;
-      df_ld2(r, node, r0, r1);
-      const float2 zv = __ldg(reinterpret_cast<const float2*>(z + node));
-      df_acc_prod_f(a, r0, zv.x);
-      df_acc_prod_f(a, r1, zv.y);
-    }
-    const DF u = df_block_sum_df(a, dsm);
-    if (threadIdx.x == 0) {
-      df_part_store(part, 2 * tt, u);
-      df_part_store(part, 2 * tt + 1, DF{0.0f, 0.0f});
-    }
-  }
-}
 
 // p = z + beta p, q = B z + beta q in DF with the per-tile DF partials p.q;
 // B z = (sigma' + D_k) z_k - sum of the CP-neighbour values on the FP32 z (the
@@ -785,23 +709,22 @@ static void b_finalize(Batch& B, int op, cudaStream_t s) {
 
 // z = M^-1 r for all geometries at once (block-diagonal V-cycle), then the
 // per-tile dot partials for beta
-static void b_precondition(Batch& B, const double* r, double* z, cudaStream_t s) {
+static void b_precondition(Batch& B, const double* r, double* z, cudaStream_t s, bool first_done = false) {
   Solver& S = *B.S;
   const int64_t n0 = S.nlaunch;
   if (B.df) {  // r in DF, z in FP32
     VcycleDot in;
     in.r = r;
     in.df = true;
-    amg_vcycle_grid(S, r, z, s, &in);
+    in.tile_part = B.part;
+    amg_vcycle_grid(S, r, z, s, &in, first_done);
   } else {
     amg_vcycle_grid(S, r, z, s);
   }
   B.nlaunch += S.nlaunch - n0;
+  if (B.df) return;  // the V-cycle's last launch formed the partials
   ++B.nlaunch;
-  if (B.df)
-    k_b_dot_df<<<bgrid(B), BT, 0, s>>>(B.view.tv(), B.tile_geo, B.sc, r, reinterpret_cast<const float*>(z), B.part);
-  else
-    k_b_dot<<<bgrid(B), BT, 0, s>>>(B.view.tv(), B.tile_geo, B.sc, r, z, B.part);
+  k_b_dot<<<bgrid(B), BT, 0, s>>>(B.view.tv(), B.tile_geo, B.sc, r, z, B.part);
 }
 
 static void b_xpby_apply(Batch& B, int first, cudaStream_t s) {
@@ -824,13 +747,21 @@ static void b_iteration(Batch& B, bool flex, cudaStream_t s) {
   const unsigned gb = bgrid(B);
   ++B.nlaunch;
   b_finalize(B, FIN_ALPHA, s);
-  if (B.df)
-    k_b_update_xr_df<<<gb, BT, 0, s>>>(tv, B.tile_geo, B.sc, S.r, S.p, S.q,
-                                       flex ? reinterpret_cast<const float*>(S.z) : nullptr, B.part);
-  else
+  if (B.df) {  // DF: always flexible (a reduced-precision V-cycle)
+    BatchUpdate u;
+    u.tile_geo = B.tile_geo;
+    u.sc = B.sc;
+    u.r = S.r;
+    u.p = S.p;
+    u.q = S.q;
+    u.z = reinterpret_cast<const float*>(S.z);
+    u.part = B.part;
+    amg_batch_update_first(S, u, gb, s);
+  } else {
     k_b_update_xr<<<gb, BT, 0, s>>>(tv, B.tile_geo, B.sc, S.r, S.p, S.q, flex ? S.z : nullptr, B.part);
+  }
   b_finalize(B, flex ? FIN_RRF : FIN_RR, s);
-  b_precondition(B, S.r, S.z, s);
+  b_precondition(B, S.r, S.z, s, B.df);
   b_finalize(B, flex ? FIN_BETAF : FIN_BETA, s);
   b_xpby_apply(B, 0, s);
 }
@@ -1191,7 +1122,7 @@ int batch_heat_setup(batch_handle* b, const double* dt, double theta, const amg_
       EB_REQUIRE(dt[g] > 0.0 && (std::isfinite(dt[g]) || (std::isinf(dt[g]) && theta == 1.0)), EB_ERR_INVALID,
                  "batch_heat_setup: dt must be > 0 (+infinity only with theta = 1)");
       const double h = B.geo[g]->h.g.h;
-      B.hconst[g] = GeoConst{h * h, dt[g], theta};
+      B.hconst[g] = GeoConst::make(h * h, dt[g], theta);
     }
     EB_CUDA(cudaMemcpyAsync(B.gconst, B.hconst.data(), sizeof(GeoConst) * ng, cudaMemcpyHostToDevice, stream));
     k_tile_shift<<<blocks_for(B.view.num_tiles, 256), 256, 0, stream>>>(B.view.num_tiles, B.tile_geo, B.gconst,

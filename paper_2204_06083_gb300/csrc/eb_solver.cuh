@@ -275,6 +275,18 @@ struct PcgUpdate {
 };
 int amg_update_first(Solver& S, const PcgUpdate& u, cudaStream_t s);
 
+// The batched DF iteration's x/r update with the V-cycle's first level-0 step
+// (a hierarchy of two or more levels with FP32 or BF16 storage); x is sc[0].x
+struct BatchUpdate {
+  const int32_t* tile_geo = nullptr;
+  const PcgScalars* sc = nullptr;
+  double* r = nullptr;
+  const double *p = nullptr, *q = nullptr;
+  const float* z = nullptr;
+  double* part = nullptr;  // per-tile pairs (r.r, r.zold)
+};
+void amg_batch_update_first(Solver& S, const BatchUpdate& u, unsigned grid, cudaStream_t s);
+
 // z = V r.  With dot, the last level-0 smoothing launch also writes per-CTA
 // partials of r.z to dot->part; returns their count, or 0 if no launch wrote
 // them (single-level hierarchy), in which case the caller computes the dot
@@ -285,6 +297,7 @@ struct VcycleDot {
   // the DF outer iteration: r holds double-float pairs, z is written in FP32
   // (part null: no partials, z on every node of the active tiles)
   bool df = false;
+  double* tile_part = nullptr;  // batched DF iteration: per-tile pairs (r.z, 0)
 };
 // first_done: amg_update_first already did the first level-0 step for this r.
 int amg_vcycle_grid(Solver& S, const double* r, double* z, cudaStream_t s, const VcycleDot* dot = nullptr,
