@@ -181,11 +181,6 @@ __global__ void __launch_bounds__(TILE_NODES) k_update_first(PairList pl, PcgUpd
                                                              DivBy theta) {
   using A = typename AccOf<V>::type;
   __shared__ double sm[TILE_NODES];
-  __shared__ double s_alpha;
-  if (cta_done(u.sc)) {
-    if (threadIdx.x == 0) u.rr_part[blockIdx.x] = 0.0;
-    return;
-  }
   double* const x = u.sc->x;
   // this thread's first pair on its way into L1 during the partial sums
   const int64_t l0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -198,7 +193,11 @@ __global__ void __launch_bounds__(TILE_NODES) k_update_first(PairList pl, PcgUpd
     prefetch_l1(code + nd);
     if (u.rzo_part) prefetch_l1(u.z + nd);
   }
-  const double alpha = pcg_alpha(u.sc, u.pq_part, u.nblk, sm, &s_alpha);
+  double alpha;
+  if (!pcg_alpha(u.sc, u.pq_part, u.nblk, sm, alpha)) {
+    if (threadIdx.x == 0) u.rr_part[blockIdx.x] = 0.0;
+    return;
+  }
   const double ax = alpha * u.h2;  // q holds h^2 (sigma I + A) p
   double srr = 0.0, srzo = 0.0;
   EB_LIST_LOOP(pl, node) {
@@ -267,13 +266,8 @@ __global__ void __launch_bounds__(TILE_NODES) k_update_first_df(PairList pl, Pcg
                                                                 float inv_theta) {
   __shared__ DF dsm[32];
   __shared__ DF s_a[2];
-  if (cta_done(u.sc)) {
-    if (threadIdx.x == 0) {
-      df_part_store(u.rr_part, blockIdx.x, DF{0.0f, 0.0f});
-      if (u.rzo_part) df_part_store(u.rzo_part, blockIdx.x, DF{0.0f, 0.0f});
-    }
-    return;
-  }
+  __shared__ int s_done;
+  const PcgHead hd = pcg_head(u.sc, false);
   const int64_t step = (int64_t)gridDim.x * blockDim.x;
   int64_t li = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double* const x = u.sc->x;
@@ -283,11 +277,21 @@ __global__ void __launch_bounds__(TILE_NODES) k_update_first_df(PairList pl, Pcg
   // alpha from the DF p'q partials (FP64 scalars), split into DF once per CTA
   const double pq = df_sum_parts(u.pq_part, u.nblk, dsm);
   if (threadIdx.x == 0) {
-    const double alpha = pcg_alpha_from(u.sc, pq);
-    s_a[0] = df_from_double(alpha);
-    s_a[1] = df_from_double(alpha * u.h2);
+    s_done = hd.done;
+    if (!hd.done) {
+      const double alpha = pcg_alpha_from(u.sc, hd, pq);
+      s_a[0] = df_from_double(alpha);
+      s_a[1] = df_from_double(alpha * u.h2);
+    }
   }
   __syncthreads();
+  if (s_done) {
+    if (threadIdx.x == 0) {
+      df_part_store(u.rr_part, blockIdx.x, DF{0.0f, 0.0f});
+      if (u.rzo_part) df_part_store(u.rzo_part, blockIdx.x, DF{0.0f, 0.0f});
+    }
+    return;
+  }
   const DF a_df = s_a[0], ax_df = s_a[1];
   DF srr{0.0f, 0.0f}, srzo{0.0f, 0.0f};
   while (li < pl.n) {
@@ -1059,13 +1063,14 @@ __global__ void __launch_bounds__(32 * GV_WARPS) k_dense_gemv(const double* __re
   const int lane = threadIdx.x & 31;
   const int64_t row = (int64_t)blockIdx.x * GV_WARPS + (threadIdx.x >> 5);
   const double* Mr = M + (row < n ? row : 0) * n;
+  for (int64_t j = 16 * lane; j < min(n, (int64_t)GV_CHUNK); j += 512) prefetch_l1(Mr + j);
   double t = 0.0;
   if constexpr (std::is_same<V, double>::value) {
-#pragma unroll 4
-    for (int64_t j = lane; j < n; j += 32) t += Mr[j] * b[j];
+    const int m = (int)n;
+#pragma unroll 8
+    for (int j = lane; j < m; j += 32) t += Mr[j] * b[j];
   } else {
     __shared__ double sb[GV_CHUNK];
-    for (int64_t j = 16 * lane; j < min(n, (int64_t)GV_CHUNK); j += 512) prefetch_l1(Mr + j);
     for (int64_t c = 0; c < n; c += GV_CHUNK) {
       const int m = (int)min((int64_t)GV_CHUNK, n - c);
       __syncthreads();

@@ -90,13 +90,12 @@ __global__ void __launch_bounds__(TILE_NODES) k_update_xr(PairList pl, PcgScalar
                                                           int nblk, double* part, double h2, const double* z,
                                                           double* rzo_part) {
   __shared__ double sm[TILE_NODES];
-  __shared__ double s_alpha;
-  if (cta_done(sc)) {
+  double* const x = sc->x;
+  double alpha;
+  if (!pcg_alpha(sc, pq_part, nblk, sm, alpha)) {
     if (threadIdx.x == 0) part[blockIdx.x] = 0.0;
     return;
   }
-  double* const x = sc->x;
-  const double alpha = pcg_alpha(sc, pq_part, nblk, sm, &s_alpha);
   const double ax = alpha * h2;
   double s = 0.0, so = 0.0;
   EB_LIST_LOOP(pl, node) {
@@ -175,12 +174,13 @@ __global__ void __launch_bounds__(TILE_NODES) k_xpby_apply(TileView tv, PairList
                                                            cudaGraphConditionalHandle h) {
   __shared__ double sm[TILE_NODES + 2];
   __shared__ double s_beta;
-  if (cta_done(sc)) {
-    if (COND && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(h, 0u);
-    return;
-  }
+  __shared__ int s_done;
+  // with COND, CTA 0 does the scalars and the loop test and the others the pairs
+  const int work = (int)blockIdx.x - (COND ? 1 : 0), nwork = (int)gridDim.x - (COND ? 1 : 0);
+  const int64_t step = (int64_t)nwork * blockDim.x;
+  const int64_t l0 = work < 0 ? pl.n : (int64_t)work * blockDim.x + threadIdx.x;
+  const PcgHead hd = pcg_head(sc, true);
   // this thread's first pair on its way into L1 during the partial sums
-  const int64_t l0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (l0 < pl.n) {
     const int32_t nd = __ldg(pl.node + l0);
     prefetch_l1(z + nd);
@@ -196,49 +196,30 @@ __global__ void __launch_bounds__(TILE_NODES) k_xpby_apply(TileView tv, PairList
       prefetch_l1(q + nd);
     }
   }
+  const double inv_rz = threadIdx.x == 0 ? 1.0 / hd.rz : 0.0;
+  double v = 0.0, t = 0.0;
   if (!first) {
-    double v, t = 0.0;
     if (rzo_part) sum_parts2(rz_part, nrz, rzo_part, nupd, sm, v, t);
     else v = sum_parts(rz_part, nrz, sm);
-    if (threadIdx.x == 0) {
-      const int k = sc->slot;  // not sc->iters: CTA 0 of this launch may advance it
-      const bool ok = v > 0.0;
-      const double beta = ok ? (v - t) / sc->rz[k] : 0.0;
-      s_beta = beta;
-      if (blockIdx.x == 0) {
-        sc->beta = beta;
-        sc->rz[k ^ 1] = v;
-        if (!ok) {
-          sc->flags |= isfinite(v) ? PCG_FLAG_BREAKDOWN : PCG_FLAG_NONFINITE;
-          sc->done = 1;
-        }
-      }
-    }
-    __syncthreads();
   }
-  const double beta = first ? 0.0 : s_beta;
+  if (threadIdx.x == 0) {
+    s_done = hd.done;
+    s_beta = (first || hd.done) ? 0.0 : pcg_beta_from(sc, hd, inv_rz, v, t, blockIdx.x == 0);
+  }
+  __syncthreads();
+  if (s_done) {
+    if (COND && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(h, 0u);
+    return;
+  }
+  const double beta = s_beta;
   if (COND && blockIdx.x == 0) {
-    // the device-side loop's test, after the beta breakdown check: r'r of
-    // this iteration's update, then continue while not converged (or broken
-    // down) and below the iteration limit.  CTAs that start after it and see
-    // done skip the p, q update, which a finished loop does not use.
-    const double v = sum_parts(rr_part, nupd, sm);
-    if (threadIdx.x == 0) {
-      if (!sc->done) {
-        sc->rr = v;
-        sc->iters += 1;
-        if (!isfinite(v)) {
-          sc->flags |= PCG_FLAG_NONFINITE;
-          sc->done = 1;
-        } else if (v <= sc->tol2 * sc->bb) {
-          sc->done = 1;
-        }
-      }
-      cudaGraphSetConditional(h, (!sc->done && sc->iters < sc->maxit) ? 1u : 0u);
-    }
+    const double rr = sum_parts(rr_part, nupd, sm);
+    if (threadIdx.x == 0) pcg_loop_test(sc, rr, h);
+    return;
   }
   double s = 0.0;
-  EB_LIST_LOOP(pl, node) {
+  for (int64_t li = l0; li < pl.n; li += step) {
+    const int32_t node = __ldg(pl.node + li);
     uint32_t c0, c1;
     ld_codes(code, node, c0, c1);
     Two<double> zc, az;
@@ -257,8 +238,8 @@ __global__ void __launch_bounds__(TILE_NODES) k_xpby_apply(TileView tv, PairList
     st2(q + node, q0, q1);
     s += p0 * q0 + p1 * q1;
   }
-  const double t = block_sum(s, sm);
-  if (threadIdx.x == 0) pq_part[blockIdx.x] = t;
+  const double pq = block_sum(s, sm);
+  if (threadIdx.x == 0) pq_part[work] = pq;
 }
 
 // ------------------------------------------------- the DF outer iteration
@@ -421,52 +402,36 @@ __global__ void __launch_bounds__(TILE_NODES) k_xpby_apply_df(TileView tv, PairL
                                                               cudaGraphConditionalHandle h, DfBeta bdf) {
   __shared__ DF dsm[32];
   __shared__ DF s_beta;
-  if (cta_done(sc)) {
-    if (COND && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(h, 0u);
-    return;
-  }
-  const int64_t step = (int64_t)gridDim.x * blockDim.x;
-  int64_t li = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ int s_done;
+  // with COND, CTA 0 does the scalars and the loop test and the others the pairs
+  const int work = (int)blockIdx.x - (COND ? 1 : 0), nwork = (int)gridDim.x - (COND ? 1 : 0);
+  const int64_t step = (int64_t)nwork * blockDim.x;
+  int64_t li = work < 0 ? pl.n : (int64_t)work * blockDim.x + threadIdx.x;
+  const PcgHead hd = pcg_head(sc, true);
   XpIn cur;
   int32_t node = li < pl.n ? __ldg(pl.node + li) : 0;
   if (li < pl.n) xp_load<DIM>(cur, tv, code, z, p, q, first, node);
-  if (threadIdx.x == 0) s_beta = DF{0.0f, 0.0f};
+  const double inv_rz = threadIdx.x == 0 ? 1.0 / hd.rz : 0.0;
+  double v = 0.0, t = 0.0;
   if (!first) {
-    const double v = df_sum_parts(rz_part, nrz, dsm);
+    v = df_sum_parts(rz_part, nrz, dsm);
     __syncthreads();
-    const double t = rzo_part ? df_sum_parts(rzo_part, nupd, dsm) : 0.0;
-    if (threadIdx.x == 0) {
-      const int k = sc->slot;
-      const bool ok = v > 0.0;
-      const double beta = ok ? (v - t) / sc->rz[k] : 0.0;
-      s_beta = df_from_double(beta);
-      if (blockIdx.x == 0) {
-        sc->beta = beta;
-        sc->rz[k ^ 1] = v;
-        if (!ok) {
-          sc->flags |= isfinite(v) ? PCG_FLAG_BREAKDOWN : PCG_FLAG_NONFINITE;
-          sc->done = 1;
-        }
-      }
-    }
+    t = rzo_part ? df_sum_parts(rzo_part, nupd, dsm) : 0.0;
+  }
+  if (threadIdx.x == 0) {
+    s_done = hd.done;
+    s_beta = df_from_double((first || hd.done) ? 0.0 : pcg_beta_from(sc, hd, inv_rz, v, t, blockIdx.x == 0));
   }
   __syncthreads();
+  if (s_done) {
+    if (COND && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(h, 0u);
+    return;
+  }
   const DF beta = s_beta;
   if (COND && blockIdx.x == 0) {
-    const double v = df_sum_parts(rr_part, nupd, dsm);
-    if (threadIdx.x == 0) {
-      if (!sc->done) {
-        sc->rr = v;
-        sc->iters += 1;
-        if (!isfinite(v)) {
-          sc->flags |= PCG_FLAG_NONFINITE;
-          sc->done = 1;
-        } else if (v <= sc->tol2 * sc->bb) {
-          sc->done = 1;
-        }
-      }
-      cudaGraphSetConditional(h, (!sc->done && sc->iters < sc->maxit) ? 1u : 0u);
-    }
+    const double rr = df_sum_parts(rr_part, nupd, dsm);
+    if (threadIdx.x == 0) pcg_loop_test(sc, rr, h);
+    return;
   }
   DF s{0.0f, 0.0f};
   while (li < pl.n) {
@@ -477,8 +442,8 @@ __global__ void __launch_bounds__(TILE_NODES) k_xpby_apply_df(TileView tv, PairL
     li = ln;
     node = nnode;
   }
-  const DF t = df_block_sum_df(s, dsm);
-  if (threadIdx.x == 0) df_part_store(pq_part, blockIdx.x, t);
+  const DF pq = df_block_sum_df(s, dsm);
+  if (threadIdx.x == 0) df_part_store(pq_part, work, pq);
 }
 
 // Into DF: xd = scale x and, in place, r = scale r (FP64 -> DF), over the CP
@@ -989,7 +954,7 @@ static void launch_xpby_apply(const EBHandle& eb, unsigned g, cudaStream_t s, co
                               const double* rzo, int nupd, double* pq, const double* rr,
                               cudaGraphConditionalHandle h) {
   dim_dispatch(eb, [&](auto D) {
-    k_xpby_apply<D.value, SHIFT, COND><<<g, list_threads(pl.n), 0, s>>>(tv, pl, sc, code, diag, op, z, p, q, first, rz, nrz,
+    k_xpby_apply<D.value, SHIFT, COND><<<g + (COND ? 1 : 0), list_threads(pl.n), 0, s>>>(tv, pl, sc, code, diag, op, z, p, q, first, rz, nrz,
                                                                 rzo, nupd, pq, rr, h);
   });
 }
@@ -1011,7 +976,7 @@ void Solver::xpby_apply(const OpParams& op, bool flex, int first, cudaStream_t s
       DfBeta bdf;
       for (int a = 0; a < 3; ++a) bdf.b[a] = beta_df[a];
       dim_dispatch(*eb, [&](auto D) {
-        k_xpby_apply_df<D.value, SH, CO><<<g, iter_threads(), 0, s>>>(tv, pl, sc, eb->code, diag_df, sig, zf, p, q, first,
+        k_xpby_apply_df<D.value, SH, CO><<<g + (CO ? 1 : 0), iter_threads(), 0, s>>>(tv, pl, sc, eb->code, diag_df, sig, zf, p, q, first,
                                                                   part_rz(), rz_n, rzo, (int)g, part_pq(), part_rr(),
                                                                   h, bdf);
       });

@@ -68,7 +68,9 @@ struct Solver {
   // r'zold partials of the flexible beta (from the x/r update)
   double* part_rzo() const { return part + 4 * (int64_t)npart + rz_cap; }
   // CTAs (= partials) of the iteration's x/r update and p update + apply
-  int nblk_iter() const { return list_blocks(*eb); }
+  // (a full grid leaves room for the CTA of the loop test, so that all are
+  // resident at once)
+  int nblk_iter() const { return std::min(list_blocks(*eb), 4 * num_sms() - 1); }
   int iter_threads() const { return list_threads(eb->num_pairs); }
   int64_t rz_cap = 0;
   int nblk = 1;
@@ -173,15 +175,26 @@ __device__ __forceinline__ double block_sum(double v, double* sm) {
   return threadIdx.x < 32 ? warp_column_sum(sm, (int)blockDim.x) : 0.0;
 }
 
-// sc->done as thread 0 of the CTA reads it, the same for all its threads (CTA
-// 0 of the launch may set it meanwhile, so threads reading it themselves could
-// disagree and part of the CTA skip the barriers the rest waits at); all
-// threads call it.
-__device__ __forceinline__ bool cta_done(const PcgScalars* sc) {
-  __shared__ int s_done;
-  if (threadIdx.x == 0) s_done = *(volatile const int*)&sc->done;
-  __syncthreads();
-  return s_done != 0;
+// What a CTA of the update kernels needs of the scalars, read by its thread 0 at
+// the start, all loads at once, ahead of the partial sums.  done is passed on
+// through shared memory: another CTA of the launch may set it meanwhile, and
+// threads that read it themselves could disagree, part of the CTA skipping the
+// barriers the rest waits at.
+struct PcgHead {
+  int done = 0, k = 0;  // k: the iteration's r'z slot
+  double rz = 0.0;
+};
+__device__ __forceinline__ PcgHead pcg_head(const PcgScalars* sc, bool recorded_slot) {
+  PcgHead h;
+  if (threadIdx.x == 0) {
+    const volatile PcgScalars* v = sc;
+    const int it = v->iters, sl = v->slot;
+    const double a = v->rz[0], b = v->rz[1];
+    h.done = v->done;
+    h.k = recorded_slot ? sl : (it & 1);
+    h.rz = h.k ? b : a;
+  }
+  return h;
 }
 
 // sum of n partials in a fixed order, the same in every CTA of a launch;
@@ -227,19 +240,17 @@ __device__ __forceinline__ void sum_parts2(const double* pa, int na, const doubl
 // into L1 ahead of a load (the reduction sums between hide the latency)
 __device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 
-// alpha = rz / p'q from the nblk partials of k_xpby_apply (q scaled by h^2:
-// the CG step length over h^2), formed by every CTA in
-// the same order; CTA 0 records p'q, alpha and a breakdown (p'q <= 0 or not
-// finite).  All threads of the CTA call it; returns alpha to every thread.
-// thread 0's part of pcg_alpha, given the summed p'q: returns alpha (CTA 0
-// records p'q, alpha and a breakdown)
-__device__ __forceinline__ double pcg_alpha_from(PcgScalars* sc, double pq) {
+// alpha = rz / p'q from the nblk partials of k_xpby_apply (q scaled by h^2: the
+// CG step length over h^2), formed by every CTA in the same order; CTA 0 records
+// p'q, alpha and a breakdown (p'q <= 0 or not finite).  Thread 0's part, given
+// the summed p'q
+__device__ __forceinline__ double pcg_alpha_from(PcgScalars* sc, const PcgHead& h, double pq) {
   const bool ok = pq > 0.0;  // false for NaN too
-  const double alpha = ok ? sc->rz[sc->iters & 1] / pq : 0.0;
+  const double alpha = ok ? h.rz / pq : 0.0;
   if (blockIdx.x == 0) {
     sc->pq = pq;
     sc->alpha = alpha;
-    sc->slot = sc->iters & 1;
+    sc->slot = h.k;
     if (!ok) {
       sc->flags |= isfinite(pq) ? PCG_FLAG_BREAKDOWN : PCG_FLAG_NONFINITE;
       sc->done = 1;
@@ -248,12 +259,55 @@ __device__ __forceinline__ double pcg_alpha_from(PcgScalars* sc, double pq) {
   return alpha;
 }
 
-__device__ __forceinline__ double pcg_alpha(PcgScalars* sc, const double* pq_part, int nblk, double* sm,
-                                            double* s_alpha) {
+// all threads of the CTA; false (all threads) when the solve is done
+__device__ __forceinline__ bool pcg_alpha(PcgScalars* sc, const double* pq_part, int nblk, double* sm, double& alpha) {
+  __shared__ double s_alpha;
+  __shared__ int s_done;
+  const PcgHead h = pcg_head(sc, false);
   const double pq = sum_parts(pq_part, nblk, sm);
-  if (threadIdx.x == 0) *s_alpha = pcg_alpha_from(sc, pq);
+  if (threadIdx.x == 0) {
+    s_done = h.done;
+    if (!h.done) s_alpha = pcg_alpha_from(sc, h, pq);
+  }
   __syncthreads();
-  return *s_alpha;
+  alpha = s_alpha;
+  return s_done == 0;
+}
+
+// The end of an iteration, thread 0's part: beta = (v - t) / rz from the summed
+// r'z (v) and, flexible, r'zold (t); with rec (one CTA of the launch) recorded
+// with the next r'z and a breakdown.  inv_rz: 1 / h.rz, formed ahead.
+__device__ __forceinline__ double pcg_beta_from(PcgScalars* sc, const PcgHead& h, double inv_rz, double v, double t,
+                                                bool rec) {
+  const bool ok = v > 0.0;
+  const double beta = ok ? (v - t) * inv_rz : 0.0;
+  if (rec) {
+    sc->beta = beta;
+    sc->rz[h.k ^ 1] = v;
+    if (!ok) {
+      sc->flags |= isfinite(v) ? PCG_FLAG_BREAKDOWN : PCG_FLAG_NONFINITE;
+      sc->done = 1;
+    }
+  }
+  return beta;
+}
+
+// The device-side loop's test (one thread), after the beta breakdown check: r'r
+// of this iteration's update (v), then continue while not converged (or broken
+// down) and below the iteration limit.  CTAs that start after it and see done
+// skip the p, q update, which a finished loop does not use.
+__device__ __forceinline__ void pcg_loop_test(PcgScalars* sc, double v, cudaGraphConditionalHandle h) {
+  if (!sc->done) {
+    sc->rr = v;
+    sc->iters += 1;
+    if (!isfinite(v)) {
+      sc->flags |= PCG_FLAG_NONFINITE;
+      sc->done = 1;
+    } else if (v <= sc->tol2 * sc->bb) {
+      sc->done = 1;
+    }
+  }
+  cudaGraphSetConditional(h, (!sc->done && sc->iters < sc->maxit) ? 1u : 0u);
 }
 
 // The PCG update x += alpha p, r -= alpha q (with the r'r partials of
