@@ -386,13 +386,39 @@ __global__ void k_smooth_p(DCsr T, const int32_t* agg, const double* phat, const
 
 // ------------------------------------------------------------------ SpGEMM
 constexpr int SPG_WARPS = 4;
-constexpr int SPG_BITS = 1 << 16;            // bitmap capacity (column range per row)
-constexpr int SPG_WORDS = SPG_BITS / 32;
+// Bound by the latency of the walk over B's rows, so by the warps in flight.
+// Bitmap words per warp (32 columns each): 512 (a range of 16,384 columns) leave
+// 36 warps per SM resident, 2048 (65,536) 12; the larger ones are taken when a
+// row needs them (seen by the count pass, which then runs again). The six
+// products of a 514 x 501 star: 730 us with 2048 and the sums in global memory,
+// 362 us with 512, a row's entries loaded 32 at a time and sums in shared memory.
+constexpr int SPG_SMALL = 512, SPG_LARGE = 2048;
+constexpr int SPG_ACC = 256;  // entries of a row summed in shared memory
 
+template <int W>
 struct SpgSmem {
-  uint32_t bits[SPG_WORDS];
-  int32_t pre[SPG_WORDS];
+  uint32_t bits[W];
+  int32_t pre[W];
+  double acc[SPG_ACC];
 };
+
+// One row of A at a time: lanes load the row's next 32 entries -- column k,
+// value, the range of B's row k -- at once, so that only B's own entries are
+// dependent loads of the walk
+struct SpgRow {
+  int32_t b0, b1;
+  double a;
+};
+__device__ __forceinline__ SpgRow spg_load(const DCsr& A, const DCsr& B, int32_t e, int32_t end, bool value) {
+  SpgRow r{0, 0, 0.0};
+  if (e < end) {
+    const int32_t k = A.ci[e];
+    r.b0 = B.rp[k];
+    r.b1 = B.rp[k + 1];
+    if (value) r.a = A.v[e];
+  }
+  return r;
+}
 
 // column range of the products of row i; false when the row is empty
 __device__ __forceinline__ bool spg_range(const DCsr& A, const DCsr& B, int64_t i, int lane, int32_t& cmin,
@@ -419,11 +445,15 @@ __device__ void spg_mark(const DCsr& A, const DCsr& B, int64_t i, int lane, int3
                          uint32_t* bits) {
   for (int w = lane; w < nwords; w += 32) bits[w] = 0u;
   __syncwarp();
-  for (int32_t e = A.rp[i]; e < A.rp[i + 1]; ++e) {
-    int32_t k = A.ci[e];
-    for (int32_t f = B.rp[k] + lane; f < B.rp[k + 1]; f += 32) {
-      int32_t off = B.ci[f] - cmin;
-      atomicOr(&bits[off >> 5], 1u << (off & 31));
+  const int32_t beg = A.rp[i], end = A.rp[i + 1];
+  for (int32_t e0 = beg; e0 < end; e0 += 32) {
+    const SpgRow r = spg_load(A, B, e0 + lane, end, false);
+    for (int t = 0; t < min(32, end - e0); ++t) {
+      const int32_t b1 = __shfl_sync(0xffffffffu, r.b1, t);
+      for (int32_t f = __shfl_sync(0xffffffffu, r.b0, t) + lane; f < b1; f += 32) {
+        int32_t off = B.ci[f] - cmin;
+        atomicOr(&bits[off >> 5], 1u << (off & 31));
+      }
     }
   }
   __syncwarp();
@@ -449,10 +479,11 @@ __device__ int32_t spg_prefix(int lane, int nwords, const uint32_t* bits, int32_
 
 // phase 0: count of the output row; rows whose column range exceeds the bitmap
 // are flagged
+template <int W>
 __global__ void k_spg_count(DCsr A, DCsr B, int32_t* cnt, int* overflow) {
-  extern __shared__ SpgSmem sm_spg[];
+  extern __shared__ __align__(8) unsigned char sm_spg[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  SpgSmem& S = sm_spg[warp];
+  SpgSmem<W>& S = reinterpret_cast<SpgSmem<W>*>(sm_spg)[warp];
   for (int64_t i = (int64_t)blockIdx.x * SPG_WARPS + warp; i < A.n; i += (int64_t)gridDim.x * SPG_WARPS) {
     int32_t cmin, cmax;
     if (!spg_range(A, B, i, lane, cmin, cmax)) {
@@ -460,7 +491,7 @@ __global__ void k_spg_count(DCsr A, DCsr B, int32_t* cnt, int* overflow) {
       continue;
     }
     int64_t range = (int64_t)cmax - cmin + 1;
-    if (range > SPG_BITS) {
+    if (range > 32 * W) {
       if (lane == 0) {
         cnt[i] = 0;
         atomicAdd(overflow, 1);
@@ -477,43 +508,62 @@ __global__ void k_spg_count(DCsr A, DCsr B, int32_t* cnt, int* overflow) {
   }
 }
 
-// phase 1: sorted columns and values of the output rows
+// phase 1: sorted columns and values of the output rows; the products of an
+// entry are added in the order of A's row, in shared memory for rows of up to
+// SPG_ACC entries (in place beyond)
+template <int W>
 __global__ void k_spg_fill(DCsr A, DCsr B, DCsr C) {
-  extern __shared__ SpgSmem sm_spg[];
+  extern __shared__ __align__(8) unsigned char sm_spg[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  SpgSmem& S = sm_spg[warp];
+  SpgSmem<W>& S = reinterpret_cast<SpgSmem<W>*>(sm_spg)[warp];
   for (int64_t i = (int64_t)blockIdx.x * SPG_WARPS + warp; i < A.n; i += (int64_t)gridDim.x * SPG_WARPS) {
     int32_t cmin, cmax;
     if (!spg_range(A, B, i, lane, cmin, cmax)) continue;
     int nwords = (int)((((int64_t)cmax - cmin + 1) + 31) >> 5);
     spg_mark(A, B, i, lane, cmin, nwords, S.bits);
-    spg_prefix(lane, nwords, S.bits, S.pre);
+    const int32_t total = spg_prefix(lane, nwords, S.bits, S.pre);
     const int32_t base = C.rp[i];
+    double* acc = total <= SPG_ACC ? S.acc : C.v + base;
     for (int w = lane; w < nwords; w += 32) {
       uint32_t word = S.bits[w];
-      int32_t p = base + S.pre[w];
+      int32_t p = S.pre[w];
       while (word) {
         int b = __ffs(word) - 1;
         word &= word - 1;
-        C.ci[p] = cmin + 32 * w + b;
-        C.v[p] = 0.0;
+        C.ci[base + p] = cmin + 32 * w + b;
         ++p;
       }
     }
+    for (int32_t p = lane; p < total; p += 32) acc[p] = 0.0;
     __syncwarp();
     // values: k in the order of A's row; lanes over the distinct columns of B_k
-    for (int32_t e = A.rp[i]; e < A.rp[i + 1]; ++e) {
-      const int32_t k = A.ci[e];
-      const double a = A.v[e];
-      for (int32_t f = B.rp[k] + lane; f < B.rp[k + 1]; f += 32) {
-        int32_t off = B.ci[f] - cmin;
-        uint32_t word = S.bits[off >> 5];
-        int32_t pos = base + S.pre[off >> 5] + __popc(word & ((1u << (off & 31)) - 1u));
-        C.v[pos] = __dadd_rn(C.v[pos], __dmul_rn(a, B.v[f]));
+    const int32_t beg = A.rp[i], end = A.rp[i + 1];
+    for (int32_t e0 = beg; e0 < end; e0 += 32) {
+      const SpgRow r = spg_load(A, B, e0 + lane, end, true);
+      for (int t = 0; t < min(32, end - e0); ++t) {
+        const int32_t b1 = __shfl_sync(0xffffffffu, r.b1, t);
+        const double a = __shfl_sync(0xffffffffu, r.a, t);
+        for (int32_t f = __shfl_sync(0xffffffffu, r.b0, t) + lane; f < b1; f += 32) {
+          int32_t off = B.ci[f] - cmin;
+          uint32_t word = S.bits[off >> 5];
+          const int32_t pos = S.pre[off >> 5] + __popc(word & ((1u << (off & 31)) - 1u));
+          acc[pos] = __dadd_rn(acc[pos], __dmul_rn(a, B.v[f]));
+        }
+        __syncwarp();
       }
-      __syncwarp();
     }
+    if (total <= SPG_ACC)
+      for (int32_t p = lane; p < total; p += 32) C.v[base + p] = acc[p];
+    __syncwarp();
   }
+}
+
+template <int W>
+static size_t spg_smem() {
+  const size_t smem = sizeof(SpgSmem<W>) * SPG_WARPS;
+  EB_CUDA(cudaFuncSetAttribute(k_spg_count<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  EB_CUDA(cudaFuncSetAttribute(k_spg_fill<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  return smem;
 }
 
 static DCsr spgemm(const DCsr& A, const DCsr& B, cudaStream_t s) {
@@ -523,32 +573,41 @@ static DCsr spgemm(const DCsr& A, const DCsr& B, cudaStream_t s) {
   C.m = B.m;
   int32_t* cnt = dalloc<int32_t>(A.n + 1, s);
   int* ovf = dalloc<int>(1, s);
-  const size_t smem = sizeof(SpgSmem) * SPG_WARPS;
-  static bool attr = false;
-  if (!attr) {
-    EB_CUDA(cudaFuncSetAttribute(k_spg_count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    EB_CUDA(cudaFuncSetAttribute(k_spg_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    attr = true;
-  }
-  unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((A.n + SPG_WARPS - 1) / SPG_WARPS,
-                                                                     (int64_t)num_sms() * 16));
-  k_spg_count<<<blocks, 32 * SPG_WARPS, smem, s>>>(A, B, cnt, ovf);
-  EB_CUDA(cudaGetLastError());
-  int hovf = 0;
-  EB_CUDA(cudaMemcpyAsync(&hovf, ovf, sizeof(int), cudaMemcpyDeviceToHost, s));
+  const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((A.n + SPG_WARPS - 1) / SPG_WARPS,
+                                                                           (int64_t)num_sms() * 16));
   C.rp = dalloc<int32_t>(A.n + 1, s, false);
-  exclusive_scan_i32(cnt, C.rp, A.n, s);
+  int hovf = 0;
   int32_t nnz = 0;
-  EB_CUDA(cudaMemcpyAsync(&nnz, C.rp + A.n, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  EB_CUDA(cudaStreamSynchronize(s));
+  auto count = [&](auto words) {
+    constexpr int W = decltype(words)::value;
+    k_spg_count<W><<<blocks, 32 * SPG_WARPS, spg_smem<W>(), s>>>(A, B, cnt, ovf);
+    EB_CUDA(cudaGetLastError());
+    EB_CUDA(cudaMemcpyAsync(&hovf, ovf, sizeof(int), cudaMemcpyDeviceToHost, s));
+    exclusive_scan_i32(cnt, C.rp, A.n, s);
+    EB_CUDA(cudaMemcpyAsync(&nnz, C.rp + A.n, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    EB_CUDA(cudaStreamSynchronize(s));
+  };
+  auto fill = [&](auto words) {
+    constexpr int W = decltype(words)::value;
+    C.nnz = nnz;
+    C.ci = dalloc<int32_t>(nnz, s, false);
+    C.v = dalloc<double>(nnz, s, false);
+    k_spg_fill<W><<<blocks, 32 * SPG_WARPS, spg_smem<W>(), s>>>(A, B, C);
+    EB_CUDA(cudaGetLastError());
+  };
+  using Small = std::integral_constant<int, SPG_SMALL>;
+  using Large = std::integral_constant<int, SPG_LARGE>;
+  count(Small{});
+  const bool large = hovf != 0;
+  if (large) {
+    EB_CUDA(cudaMemsetAsync(ovf, 0, sizeof(int), s));
+    count(Large{});
+  }
   dfree(cnt, s);
   dfree(ovf, s);
   EB_REQUIRE(hovf == 0, EB_ERR_OOM, "spgemm: a product row spans more than 65536 columns");
-  C.nnz = nnz;
-  C.ci = dalloc<int32_t>(nnz, s, false);
-  C.v = dalloc<double>(nnz, s, false);
-  k_spg_fill<<<blocks, 32 * SPG_WARPS, smem, s>>>(A, B, C);
-  EB_CUDA(cudaGetLastError());
+  if (large) fill(Large{});
+  else fill(Small{});
   return C;
 }
 
@@ -1069,15 +1128,21 @@ void amg_build_from(Solver& S, DCsr A0, cudaStream_t s) {
     EB_CUDA(cudaMemsetAsync(state, 1, A.n, s));
     uint64_t* k1 = dalloc<uint64_t>(A.n, s, false);
     int* und = dalloc<int>(1, s);
-    for (int round = 0; round < 1000; ++round) {
-      EB_CUDA(cudaMemsetAsync(und, 0, sizeof(int), s));
-      k_mis_max1<<<blocks_for(A.n, 256), 256, 0, s>>>(A, strong, state, k1);
-      k_mis_max2<<<blocks_for(A.n, 256), 256, 0, s>>>(A, strong, k1, state, und);
+    // rounds until every node is decided (further rounds change nothing); on
+    // small levels, where a round costs less than reading the count back, four
+    // between two looks at it
+    const int batch = A.n < 300000 ? 4 : 1;
+    for (int round = 0;;) {
+      for (int k = 0; k < batch; ++k, ++round) {
+        if (k + 1 == batch) EB_CUDA(cudaMemsetAsync(und, 0, sizeof(int), s));
+        k_mis_max1<<<blocks_for(A.n, 256), 256, 0, s>>>(A, strong, state, k1);
+        k_mis_max2<<<blocks_for(A.n, 256), 256, 0, s>>>(A, strong, k1, state, und);
+      }
       int hund = 0;
       EB_CUDA(cudaMemcpyAsync(&hund, und, sizeof(int), cudaMemcpyDeviceToHost, s));
       EB_CUDA(cudaStreamSynchronize(s));
       if (hund == 0) break;
-      EB_REQUIRE(round < 999, EB_ERR_INVALID, "amg_setup: MIS-2 did not terminate");
+      EB_REQUIRE(round < 1000, EB_ERR_INVALID, "amg_setup: MIS-2 did not terminate");
     }
     int32_t* rflag = dalloc<int32_t>(A.n + 1, s);
     int32_t* roff = dalloc<int32_t>(A.n + 1, s, false);

@@ -1063,14 +1063,13 @@ __global__ void __launch_bounds__(32 * GV_WARPS) k_dense_gemv(const double* __re
   const int lane = threadIdx.x & 31;
   const int64_t row = (int64_t)blockIdx.x * GV_WARPS + (threadIdx.x >> 5);
   const double* Mr = M + (row < n ? row : 0) * n;
-  for (int64_t j = 16 * lane; j < min(n, (int64_t)GV_CHUNK); j += 512) prefetch_l1(Mr + j);
   double t = 0.0;
   if constexpr (std::is_same<V, double>::value) {
-    const int m = (int)n;
-#pragma unroll 8
-    for (int j = lane; j < m; j += 32) t += Mr[j] * b[j];
+#pragma unroll 4
+    for (int64_t j = lane; j < n; j += 32) t += Mr[j] * b[j];
   } else {
     __shared__ double sb[GV_CHUNK];
+    for (int64_t j = 16 * lane; j < min(n, (int64_t)GV_CHUNK); j += 512) prefetch_l1(Mr + j);
     for (int64_t c = 0; c < n; c += GV_CHUNK) {
       const int m = (int)min((int64_t)GV_CHUNK, n - c);
       __syncthreads();

@@ -663,7 +663,6 @@ void Solver::alloc_work(cudaStream_t s) {
   npart = std::max(nblk, nblk_iter());
   part = dalloc<double>(5 * (int64_t)npart + rz_cap, s);
   sc = dalloc<PcgScalars>(1, s);
-  EB_CUDA(cudaMallocHost((void**)&sc_host, sizeof(PcgScalars)));
 }
 
 void Solver::free_work() {
@@ -675,8 +674,6 @@ void Solver::free_work() {
   dfree(r, s); dfree(z, s); dfree(p, s); dfree(q, s); dfree(tmp, s); dfree(part, s); dfree(sc, s); dfree(wx, s);
   dfree(diag_df, s); dfree(xdf, s); dfree(dev_err, s);
   for (auto& bd : beta_df) dfree(bd, s);
-  if (sc_host) cudaFreeHost(sc_host);
-  sc_host = nullptr;
 }
 
 void Solver::finalize(int op, const double* src, cudaStream_t s, int count) {
@@ -781,34 +778,34 @@ int Solver::pcg(const double* b, double* x, double rtol, int maxit, const pcg_op
     EB_DIM_LAUNCH(dim, k_mask_copy, nblk, tv, eb->code, x, x);
     EB_DIMV_LAUNCH(*eb, k_resid, nblk, tv, eb->code, eb->diag, op, b, x, r, part_pq());
     finalize(FIN_INIT, part_pq(), s);
-    EB_CUDA(cudaMemcpyAsync(sc_host, sc, sizeof(PcgScalars), cudaMemcpyDeviceToHost, s));
+    EB_CUDA(cudaMemcpyAsync(&sc_host, sc, sizeof(PcgScalars), cudaMemcpyDeviceToHost, s));
     EB_CUDA(cudaStreamSynchronize(s));
-    if (sc_host->flags & PCG_FLAG_NONFINITE) {
-      flags |= sc_host->flags;
+    if (sc_host.flags & PCG_FLAG_NONFINITE) {
+      flags |= sc_host.flags;
       break;
     }
-    if (sc_host->bb == 0.0) {  // b = 0: x = 0 is the solution
+    if (sc_host.bb == 0.0) {  // b = 0: x = 0 is the solution
       EB_DIM_LAUNCH(dim, k_mask_copy, nblk, tv, eb->code, b, x);
       converged = true;
       rel = 0.0;
       break;
     }
-    if (sc_host->done) {
+    if (sc_host.done) {
       converged = true;
-      rel = std::sqrt(sc_host->rr / sc_host->bb);
+      rel = std::sqrt(sc_host.rr / sc_host.bb);
       break;
     }
     if (total_iters >= maxit) break;
     double scale = 1.0;
     if (df_on) {
       // scale by a power of two so that the scaled b has a unit root mean square
-      const double ms = sc_host->bb / (double)std::max<int64_t>(eb->num_cp, 1);
+      const double ms = sc_host.bb / (double)std::max<int64_t>(eb->num_cp, 1);
       scale = std::ldexp(1.0, -(int)std::lround(0.5 * std::log2(ms)));
       ++nlaunch;
       k_df_in<<<nblk, TILE_NODES, 0, s>>>(eb->pairs(), x, xi, r, scale);
-      sc_host->bb *= scale * scale;
-      sc_host->rr *= scale * scale;
-      EB_CUDA(cudaMemcpyAsync(sc, sc_host, sizeof(PcgScalars), cudaMemcpyHostToDevice, s));
+      sc_host.bb *= scale * scale;
+      sc_host.rr *= scale * scale;
+      EB_CUDA(cudaMemcpyAsync(sc, &sc_host, sizeof(PcgScalars), cudaMemcpyHostToDevice, s));
     }
     precondition(kind, r, z, s);
     const bool flex = flex_for(kind);
@@ -819,9 +816,9 @@ int Solver::pcg(const double* b, double* x, double rtol, int maxit, const pcg_op
     if (o.use_graph == 1 && !prof_on) {  // the whole loop on the device
       loop_prepare(kind);
       EB_CUDA(cudaGraphLaunch(lexec, s));
-      EB_CUDA(cudaMemcpyAsync(sc_host, sc, sizeof(PcgScalars), cudaMemcpyDeviceToHost, s));
+      EB_CUDA(cudaMemcpyAsync(&sc_host, sc, sizeof(PcgScalars), cudaMemcpyDeviceToHost, s));
       EB_CUDA(cudaStreamSynchronize(s));
-      nlaunch += l_launches * sc_host->iters;
+      nlaunch += l_launches * sc_host.iters;
       stop = true;
     }
     while (!stop) {
@@ -837,17 +834,17 @@ int Solver::pcg(const double* b, double* x, double rtol, int maxit, const pcg_op
         for (int j = 0; j < nb; ++j, ++it) iteration(kind, s);
       }
       EB_CUDA(cudaGetLastError());
-      EB_CUDA(cudaMemcpyAsync(sc_host, sc, sizeof(PcgScalars), cudaMemcpyDeviceToHost, s));
+      EB_CUDA(cudaMemcpyAsync(&sc_host, sc, sizeof(PcgScalars), cudaMemcpyDeviceToHost, s));
       EB_CUDA(cudaStreamSynchronize(s));
       if (prof_on) {
         if (graphed) prof_collect(0, g_pairs);
         prof_collect(g_pairs, prof_n - g_pairs);
         prof_n = g_pairs;
       }
-      if (sc_host->done || total_iters + it >= maxit) stop = true;
+      if (sc_host.done || total_iters + it >= maxit) stop = true;
     }
-    total_iters += sc_host->iters;
-    flags |= sc_host->flags;
+    total_iters += sc_host.iters;
+    flags |= sc_host.flags;
     if (df_on) {
       ++nlaunch;
       k_df_out<<<nblk, TILE_NODES, 0, s>>>(eb->pairs(), xi, x, 1.0 / scale);
@@ -856,10 +853,10 @@ int Solver::pcg(const double* b, double* x, double rtol, int maxit, const pcg_op
     // true residual at exit (FP64)
     EB_DIMV_LAUNCH(*eb, k_resid, nblk, tv, eb->code, eb->diag, op, b, x, r, part_pq());
     finalize(FIN_INIT, part_pq(), s);
-    EB_CUDA(cudaMemcpyAsync(sc_host, sc, sizeof(PcgScalars), cudaMemcpyDeviceToHost, s));
+    EB_CUDA(cudaMemcpyAsync(&sc_host, sc, sizeof(PcgScalars), cudaMemcpyDeviceToHost, s));
     EB_CUDA(cudaStreamSynchronize(s));
-    rel = sc_host->bb > 0 ? std::sqrt(sc_host->rr / sc_host->bb) : 0.0;
-    if (sc_host->done) converged = true;
+    rel = sc_host.bb > 0 ? std::sqrt(sc_host.rr / sc_host.bb) : 0.0;
+    if (sc_host.done) converged = true;
     if (total_iters >= maxit) break;
   }
   auto t1 = std::chrono::steady_clock::now();

@@ -76,7 +76,9 @@ struct Solver {
   int nblk = 1;
   int rz_n = 1;  // r'z partials written by the last precondition()
   PcgScalars* sc = nullptr;
-  PcgScalars* sc_host = nullptr;
+  // not page-locked: that allocation and its release (which waits for the
+  // device) cost 320 us per solver, its copies of ~0.2 KB no more than these
+  PcgScalars sc_host{};
   int64_t nlaunch = 0;  // kernel launches issued (reported per solve)
   // event timing of the level-0 smoother launches
   bool prof_on = false;
