@@ -449,9 +449,10 @@ __global__ void k_l6_fwd(Image im, const bf16* __restrict__ y5, const float* __r
 // step are independent.  Every layer computes 128 columns (the tensor cores'
 // M), the strip's 116 plus 6 on each side: layer l is exact on 128 - 2 (l - 1)
 // of them, which leaves layer 6 exact on the strip.
-//   * layer 1 (2 -> 32, CUDA cores, warps 4-7): one pixel per thread, eight
-//     output channels' FMA chains side by side, each in k_l1_fwd's order;
-//     bf16 result into ring 0.  The input window is loaded a step ahead.
+//   * layer 1 (2 -> 32, CUDA cores, warps 20-27): one pixel of two rows per
+//     thread, eight output channels' FMA chains side by side, each in
+//     k_l1_fwd's order; bf16 result into ring 0.  Two groups of four warps take
+//     the pairs of rows in turn.
 //   * layers 2-5 (tcgen05, lane 0 of warp 8 + l - 2): the MMAs are input-row
 //     stationary.  At step tau layer l takes its newest input row, rho + 1
 //     (rho = the output row it finishes), from ring l - 2 (64-byte swizzled
@@ -459,44 +460,50 @@ __global__ void k_l6_fwd(Image im, const bf16* __restrict__ y5, const float* __r
 //     copies lay them out) and multiplies it, shifted by dx = 0, 1, 2 pixels
 //     and split in two channel halves, by the weights of the three tap rows
 //     at once: N = 96 = (dy, n), contributions to output rows rho + 2 - dy.
-//     Each output row accumulates in one of four 32-column TMEM slots per
-//     layer, placed so that rows rho + 2, rho + 1, rho lie at increasing
-//     columns; runs of adjacent slots take one MMA per (dx, kh), so a layer
-//     issues 6 MMAs per step (12 when the three slots wrap), a third of the
-//     18 of the output-stationary form.  The slot of row rho receives its taps
-//     in (dy, dx, kh) order, as in k_conv32_tma, from zero.
-//   * epilogues of layers 2-4 (warps 0-3, one TMEM lane = one pixel per
-//     thread): read the finished slot of row rho and zero it for row rho + 4,
-//     bias, ReLU, bf16, 0 outside the image (the next layer's zero padding),
-//     into ring l - 1 (the swizzle applied by hand).
-//   * layers 5-6 (warps 12-15): layer 5's epilogue forms the nine tap
-//     partials of layer 6 (a float per tap and pixel, ring T) from its
+//     Each output row accumulates in one of 16 TMEM slots of 32 columns, a
+//     ring shared by the four layers (fz_col): rows rho + 2, rho + 1, rho lie
+//     at increasing columns, and a layer issues 6 MMAs per step (12 in the two
+//     steps of 16 in which its three slots wrap).  The slot of row rho receives
+//     its taps in (dy, dx, kh) order, as in k_conv32_tma, from zero.
+//   * epilogues of layers 2-4 (warps 0-7, one TMEM lane = one pixel per
+//     thread): read the finished slot of row rho and zero it, bias, ReLU,
+//     bf16, 0 outside the image (the next layer's zero padding), into ring
+//     l - 1 (the swizzle applied by hand).  Two groups of four warps take the
+//     steps in turn.
+//   * layers 5-6 (warps 12-19, in turn as well): layer 5's epilogue forms the
+//     nine tap partials of layer 6 (a float per tap and pixel, ring T) from its
 //     bf16-rounded values, nine FMA chains side by side; layer 6 adds them up:
 //     out = m (b6 + sum).
-// Activation rings hold 2 rows (row rho in slot rho & 1): a step reads row
-// rho + 1 of a ring and writes row rho + 2.  T holds 4.  Every layer's
-// arithmetic is that of the layer-by-layer path (k_l1_fwd, k_conv32_tma,
-// k_l6_fwd), so the two give identical outputs.
-// Barriers (mbarriers, two of each kind per layer, by step parity): rdy[j][b]
-// (ring j row of step k written: 4 warp arrivals -> MMA of layer j + 2 at
-// step k + 1), mdone[j][b] (commit of layer j + 2's MMAs at step k ->
-// epilogue; mdone[0] also frees ring 0's older row for layer 1), tempty[j][b]
-// (slot read and zeroed: 4 warp arrivals -> MMA at step k + 2, or k + 1 at a
-// unit's first step, after the last step of the unit before has cleared every
-// slot).  With two barriers per kind no waiter can fall two phases behind.
-// The epilogue of layer l at step k overwrites the row of ring l - 1 that
-// layer l + 1's MMAs read at step k - 1: for l = 2, 3 the epilogue warps
-// waited for those (mdone of layer l + 1, step k - 1) earlier in their own
-// program order, for l = 4 they wait for layer 5's explicitly.  Every wait is
-// bounded; one that gives up raises a shared abort flag, after which every
-// role runs its remaining steps without waiting or computing (so the named
-// barriers still match), the CTA waits (bounded) for its MMAs in flight,
-// frees TMEM and sets *err.
+// Ring 0 holds 8 rows (of step k in slot k & 7), rings 1-3 hold 2 (row rho in
+// slot rho & 1): a step reads the row that the step before wrote.  T holds 4.
+// Every layer's arithmetic is that of the layer-by-layer path (k_l1_fwd,
+// k_conv32_tma, k_l6_fwd), so the two give identical outputs.
+// Barriers (mbarriers; k counts the steps of the CTA over all its units):
+// rdy0 / rdy[j] (ring j row of step k written and, for j >= 1, the slot that
+// layer j + 2 enters next zeroed: 4 warp arrivals -> MMA of layer j + 2 at step
+// k + 1), mdone[j] (commit of layer j + 2's MMAs at step k -> epilogue; frees
+// the ring rows they read: ring 0's for layer 1 six steps on, the others' for
+// the epilogue of the next step), tempty[j] (slot read and zeroed: 4 warp
+// arrivals -> MMAs at a unit's first step, whose last step before cleared the
+// rows begun; layer 5's -> layer 2's MMAs five steps on, which enter its slot),
+// tdone (T row of step k written and read: layers 5-6 take turns).  A parity
+// wait is sound while its barrier is neither two phases ahead nor one behind:
+// eight barriers per layer for mdone, tempty and rdy0 and two for rdy and tdone
+// give that, whatever the warps' relative speeds (a random-schedule model of
+// the roles, with these waits, found four too few for mdone).  Every wait is
+// bounded; one that gives up raises a shared abort flag, after which every role
+// runs its remaining steps without waiting or computing, the CTA waits
+// (bounded) for its MMAs in flight, frees TMEM and sets *err.
+// Bound by the issue slots and the shared-memory pipe together (68 % and 79 %
+// busy; the tensor pipe 36 %).  At 2048^2: 441 us; 561 us with one group of
+// warps per role, whose epilogue (3200 cycles of work in a step of 4280) paced
+// the others, and four slots per layer (9 MMAs per step instead of 6.75); with
+// one row per thread in layer 1 and 24 warps 451 us.
 constexpr int FZ_OUT = TPX - 12;                       // 116
 constexpr int FZ_ROW = TC_PIX * NC * 2;                // 8320 bytes: one activation row, 130 pixel slots
-constexpr int FZ_RING = 2;                             // rows per activation ring
-constexpr int FZ_RINGB = FZ_RING * FZ_ROW;             // 16,640
-constexpr int FZ_W = 4 * FZ_RINGB;                     // weights of layers 2-5: 66,560
+constexpr int FZ_RINGB = 2 * FZ_ROW;                   // 16,640: rings 1-3, two rows
+constexpr int FZ_RING0 = 8 * FZ_ROW;                   // 66,560: ring 0, eight rows
+constexpr int FZ_W = 114 * 1024;                       // weights of layers 2-5: 116,736
 constexpr int FZ_WDX = 4 * 96 * 16;                    // B bytes of one horizontal tap: 6144
 constexpr int FZ_TRING = 4;                            // rows of the tap-partial ring
 constexpr int FZ_TROW = 9 * TC_PIX;                    // floats of a T row: 9 taps x 130 slots
@@ -505,9 +512,9 @@ constexpr int FZ_W1 = FZ_T + FZ_TRING * FZ_TROW * 4;   // 159,008: layer-1 weigh
 constexpr int FZ_W6 = FZ_W1 + (NC * 20 + NC) * 4;      // 161,696: W6 as [c][12 taps], then b6
 constexpr int FZ_BM = FZ_W6 + 1552;                    // 163,248: biases of layers 2-5
 constexpr int FZ_BAR = FZ_BM + NMID * NC * 4;          // 163,760
-constexpr int FZ_NBAR = 24;
+constexpr int FZ_NBAR = 80;
 constexpr int FZ_SMEM = FZ_BAR + 8 * FZ_NBAR + 16;     // 163,968
-constexpr int FZ_THREADS = 512;  // warps 0-3 epilogues 2-4, 4-7 layer 1, 8-11 MMAs, 12-15 layers 5-6
+constexpr int FZ_THREADS = 896;  // warps 0-7 epilogues 2-4, 8-11 MMAs, 12-19 layers 5-6, 20-27 layer 1
 static_assert(FZ_SMEM <= 232448, "fused forward: shared memory");
 static_assert(FZ_W % 1024 == 0 && FZ_T % 16 == 0 && FZ_BAR % 8 == 0, "fused forward: alignment");
 
@@ -525,13 +532,14 @@ struct FzArgs {
 // 64 bytes (32 bf16 = 16 words) into the pixel row at shared address row (a
 // multiple of 64) in the 64-byte swizzled layout: 16-byte chunk c of the row
 // lands at chunk c ^ (address bits 7-8)
+__device__ __forceinline__ void fz_st_chunk(uint32_t row, int c, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(row + ((c ^ ((row >> 7) & 3u)) << 4)), "r"(w0), "r"(w1),
+               "r"(w2), "r"(w3)
+               : "memory");
+}
 __device__ __forceinline__ void fz_st_row(uint32_t row, const uint32_t (&w)[NC / 2]) {
-  const uint32_t sw = (row >> 7) & 3u;
 #pragma unroll
-  for (int c = 0; c < 4; ++c)
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(row + ((c ^ sw) << 4)), "r"(w[4 * c]),
-                 "r"(w[4 * c + 1]), "r"(w[4 * c + 2]), "r"(w[4 * c + 3])
-                 : "memory");
+  for (int c = 0; c < 4; ++c) fz_st_chunk(row, c, w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
 }
 
 // Bounded wait of the fused kernel: the waiting thread asks to be suspended
@@ -566,10 +574,14 @@ __device__ __forceinline__ bool fz_wait(uint32_t bar, uint32_t parity, volatile 
   return false;
 }
 
-// tensor-memory column (within a layer's 128) of the accumulator of output row
-// r: four slots, r & 3 = 3, 2, 1, 0 at columns 0, 32, 64, 96, so that rows
-// r + 2, r + 1, r (which one input row feeds) lie at increasing columns
-__device__ __forceinline__ int fz_col(int r) { return 32 * (3 - (r & 3)); }
+// Tensor-memory column of the accumulator of layer j + 2's output row that is
+// finished at step kf.  The 16 slots of 32 columns form one ring for the four
+// layers: at step k layer j + 2 holds the rows finished at k + 2, k + 1 and k
+// (which one input row feeds) at increasing slots, and every step moves all
+// layers one slot down.  The slot a layer enters is the one that the layer below
+// it finished the step before; layer 2 enters the one that layer 5 finished five
+// steps before.
+__device__ __forceinline__ int fz_col(int j, int64_t kf) { return 32 * ((3 * j - (int)kf) & 15); }
 
 // 32 zero columns of tensor memory at taddr for this warp's 32 lanes
 __device__ __forceinline__ void fz_tmem_zero32(uint32_t taddr) {
@@ -581,13 +593,13 @@ __device__ __forceinline__ void fz_tmem_zero32(uint32_t taddr) {
       : "memory");
 }
 
-// Reads the finished accumulator of output row rho of layer j + 2 (32 columns,
-// this warp's lanes; tlane = TMEM address of lane 32 (warp % 4), column 0)
-// into v, then starts zeroing its slot for row rho + 4 (all four slots of the
-// layer at a unit's last step, which leaves no partial sums to the next unit);
-// fz_release completes it.  okw (warp-uniform) false: nothing is read, v = 0.
-__device__ __forceinline__ void fz_take(uint32_t tlane, int j, int rho, bool okw, bool last, uint32_t (&v)[NC]) {
-  const uint32_t tacc = tlane + (uint32_t)(j * 128 + fz_col(rho));
+// Reads the accumulator that layer j + 2 finished at step k (32 columns, this
+// warp's lanes; tlane = TMEM address of lane 32 (warp % 4), column 0) into v,
+// then starts zeroing its slot (at a unit's last step also the two slots of the
+// rows begun, which leaves no partial sums to the next unit); fz_release
+// completes it.  okw (warp-uniform) false: nothing is read, v = 0.
+__device__ __forceinline__ void fz_take(uint32_t tlane, int j, int64_t k, bool okw, bool last, uint32_t (&v)[NC]) {
+  const uint32_t tacc = tlane + (uint32_t)fz_col(j, k);
   if (okw) {
     asm volatile("tcgen05.fence::after_thread_sync;");
     asm volatile(
@@ -599,10 +611,10 @@ __device__ __forceinline__ void fz_take(uint32_t tlane, int j, int rho, bool okw
           "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
         : "r"(tacc));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    fz_tmem_zero32(tacc);
     if (last) {
-      for (int c = 0; c < 128; c += 32) fz_tmem_zero32(tlane + (uint32_t)(j * 128 + c));
-    } else {
-      fz_tmem_zero32(tacc);
+      fz_tmem_zero32(tlane + (uint32_t)fz_col(j, k + 1));
+      fz_tmem_zero32(tlane + (uint32_t)fz_col(j, k + 2));
     }
   } else {
 #pragma unroll
@@ -611,7 +623,7 @@ __device__ __forceinline__ void fz_take(uint32_t tlane, int j, int rho, bool okw
 }
 
 // after fz_take: the zeroing stores are complete and the slot is released to
-// the MMAs (whose next write to it comes two steps on)
+// the MMAs (layer j + 3's write it two steps on)
 __device__ __forceinline__ void fz_release(uint32_t tempty) {
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;");
@@ -640,16 +652,11 @@ __device__ __forceinline__ void fz_add2(float a0, float a1, float b0, float b1, 
   fz_upk(r, r0, r1);
 }
 
-// the 3 x 3 input window of pixel x in row tau of image img (0 outside the image)
-__device__ __forceinline__ void fz_window(const FzArgs& a, int img, int tau, int x, float2 (&v)[9]) {
-  const bool in = tau >= 0 && tau < a.im.R && x >= 0 && x < a.im.W;
-#pragma unroll
-  for (int d = 0; d < 9; ++d) {
-    const int xx = x + d % 3 - 1, rr = tau + d / 3 - 1;
-    v[d] = (in && xx >= 0 && xx < a.im.W && rr >= 0 && rr < a.im.R)
-               ? __ldg(a.in + ((int64_t)img * a.im.R + rr) * a.im.W + xx)
-               : make_float2(0.f, 0.f);
-  }
+// (max(a, 0), max(b, 0)) in bf16: rounding keeps the sign and the order, so the
+// packed maximum after it equals the two FP32 ones before it (NaN gives 0 in both)
+__device__ __forceinline__ uint32_t fz_relu2(float a, float b) {
+  const __nv_bfloat162 h = __hmax2(__floats2bfloat162_rn(a, b), __floats2bfloat162_rn(0.0f, 0.0f));
+  return *reinterpret_cast<const uint32_t*>(&h);
 }
 
 __device__ __forceinline__ void fz_unit(const FzArgs& a, int64_t u, int& img, int& r0, int& r1, int& x0) {
@@ -666,9 +673,11 @@ __global__ void __launch_bounds__(FZ_THREADS, 1) k_net_fwd(const __grid_constant
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t base = smem_addr(smem_raw);
   const uint32_t bars = base + FZ_BAR;
-  auto rdy = [&](int j, int b) { return bars + 8 * (2 * j + b); };
-  auto mdone = [&](int j, int b) { return bars + 8 * (8 + 2 * j + b); };
-  auto tempty = [&](int j, int b) { return bars + 8 * (16 + 2 * j + b); };
+  auto rdy0 = [&](int64_t k) { return bars + 8 * (int)(k & 7); };                          // ring 0
+  auto rdy = [&](int j, int64_t k) { return bars + 8 * (6 + 2 * j + (int)(k & 1)); };  // rings 1-3
+  auto mdone = [&](int j, int64_t k) { return bars + 8 * (14 + 8 * j + (int)(k & 7)); };
+  auto tempty = [&](int j, int64_t k) { return bars + 8 * (46 + 8 * j + (int)(k & 7)); };
+  auto tdone = [&](int b) { return bars + 8 * (78 + b); };
   uint32_t* tslot = reinterpret_cast<uint32_t*>(smem_raw + FZ_BAR + 8 * FZ_NBAR);
   volatile int* abort = reinterpret_cast<volatile int*>(smem_raw + FZ_BAR + 8 * FZ_NBAR + 8);
   float* sT = reinterpret_cast<float*>(smem_raw + FZ_T);
@@ -704,7 +713,7 @@ __global__ void __launch_bounds__(FZ_THREADS, 1) k_net_fwd(const __grid_constant
   for (int i = tid; i < NMID * NC; i += FZ_THREADS) sBM[i] = a.P[off_wm(i / NC) + WM_N + i % NC];
   if (tid == 0) {
     for (int b = 0; b < FZ_NBAR; ++b) {
-      const uint32_t cnt = (b >= 8 && b < 16) ? 1u : 4u;  // mdone: one commit; rdy, tempty: four warps
+      const uint32_t cnt = (b >= 14 && b < 46) ? 1u : 4u;  // mdone: one commit; rdy, tempty: four warps
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bars + 8 * b), "r"(cnt));
     }
     *abort = 0;
@@ -728,11 +737,88 @@ __global__ void __launch_bounds__(FZ_THREADS, 1) k_net_fwd(const __grid_constant
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
 
-  if (warp >= 12) {
-    // layer 5's epilogue, layer 6 and the tap partials (warps 12-15): thread t
-    // = TMEM lane t = pixel slot t + 1 (warp w reads lanes 32 (w - 12) ..)
-    const int t = tid - 384;
+  if (warp >= 20) {
+    // layer 1, two rows at a time (each weight read from shared memory serves
+    // both): warps 20-23 and 24-27 take the pairs of steps in turn; thread t of
+    // a group = pixel slot t + 1 of ring 0
+    const int t = tid & 127;
+    int grp = (warp - 20) >> 2;
+    int64_t k = 0;
+    for (int64_t u = blockIdx.x; u < a.units; u += gridDim.x) {
+      int img, r0, r1, x0;
+      fz_unit(a, u, img, r0, r1, x0);
+      const int nsteps = r1 - r0 + 15;
+      const int x = x0 - 6 + t;
+      for (int st = 0; st < nsteps; st += 2, grp ^= 1) {
+        const int np = min(2, nsteps - st), tau = r0 - 5 + st;
+        if (grp) {
+          k += np;
+          continue;
+        }
+        float2 v[12];  // rows tau - 1 .. tau + 2, columns x - 1 .. x + 1
+#pragma unroll
+        for (int d = 0; d < 12; ++d) {
+          const int xx = x + d % 3 - 1, rr = tau + d / 3 - 1;
+          v[d] = (xx >= 0 && xx < im.W && rr >= 0 && rr < im.R)
+                     ? __ldg(a.in + ((int64_t)img * im.R + rr) * im.W + xx)
+                     : make_float2(0.f, 0.f);
+        }
+        const bool in_x = x >= 0 && x < im.W;
+        const bool in0 = in_x && tau >= 0 && tau < im.R, in1 = in_x && tau + 1 >= 0 && tau + 1 < im.R;
+        // the rows overwritten here were read by layer 2's MMAs of steps k - 7 and k - 6
+        if (k >= 6) fz_wait(mdone(0, k - 6), (uint32_t)((k - 6) >> 3) & 1u, abort);
+        const uint32_t row0 = base + (uint32_t)((int)(k & 7) * FZ_ROW + (t + 1) * 64);
+        const uint32_t row1 = base + (uint32_t)((int)((k + 1) & 7) * FZ_ROW + (t + 1) * 64);
+        // eight output channels at a time, each one FMA chain in k_l1_fwd's order
+#pragma unroll
+        for (int cg = 0; cg < NC; cg += 8) {
+          uint64_t acc[2][4];  // channel pairs (cg + 2q, cg + 2q + 1) of the two rows
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            acc[0][q] = acc[1][q] = *reinterpret_cast<const uint64_t*>(sW1 + 18 * NC + cg + 2 * q);
+#pragma unroll
+          for (int e = 0; e < 18; ++e) {
+            const float4 wa = *reinterpret_cast<const float4*>(sW1 + e * NC + cg);
+            const float4 wb = *reinterpret_cast<const float4*>(sW1 + e * NC + cg + 4);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const float xv = (e & 1) ? v[(e >> 1) + 3 * h].y : v[(e >> 1) + 3 * h].x;
+              const uint64_t x2 = fz_pk(xv, xv);
+              fz_fma2(acc[h][0], fz_pk(wa.x, wa.y), x2);
+              fz_fma2(acc[h][1], fz_pk(wa.z, wa.w), x2);
+              fz_fma2(acc[h][2], fz_pk(wb.x, wb.y), x2);
+              fz_fma2(acc[h][3], fz_pk(wb.z, wb.w), x2);
+            }
+          }
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            uint32_t o[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              float a0, a1;
+              fz_upk(acc[h][q], a0, a1);
+              o[q] = (h ? in1 : in0) ? fz_relu2(a0, a1) : 0u;
+            }
+            const uint32_t row = h ? row1 : row0;
+            if (h < np) fz_st_chunk(row, cg / 8, o[0], o[1], o[2], o[3]);
+          }
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) {
+          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(rdy0(k)) : "memory");
+          if (np == 2) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(rdy0(k + 1)) : "memory");
+        }
+        k += np;
+      }
+    }
+  } else if (warp >= 12) {
+    // layer 5's epilogue, the tap partials and layer 6: warps 12-15 take the
+    // even steps, 16-19 the odd ones; thread t of a group = TMEM lane t = pixel
+    // slot t + 1
+    const int t = tid & 127, grp = (warp - 12) >> 2;
     const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    constexpr int j = NMID - 1;
     int64_t k = 0;
     for (int64_t u = blockIdx.x; u < a.units; u += gridDim.x) {
       int img, r0, r1, x0;
@@ -740,23 +826,55 @@ __global__ void __launch_bounds__(FZ_THREADS, 1) k_net_fwd(const __grid_constant
       const int nsteps = r1 - r0 + 15;
       const int x = x0 - 6 + t;
       for (int st = 0; st < nsteps; ++st, ++k) {
-        const int tau = r0 - 5 + st;
+        const int tau = r0 - 5 + st, b = (int)(k & 1);
+        if (b != grp) continue;
+        const bool last = st == nsteps - 1;
         // layer 6 writes row tau - 10 at the end of the step: its mask value now
         const int r6 = tau - 10;
         const bool out6 = r6 >= r0 && r6 < r1 && t >= 6 && t < 6 + FZ_OUT && x < im.W;
         const int64_t p6 = ((int64_t)img * im.R + r6) * im.W + x;
         const float m6 = out6 ? __ldg(a.in + p6).y : 0.0f;
         // layer 5 (row tau - 8): its values, bf16-rounded as layer 6 reads them
-        const int j = NMID - 1, b = (int)(k & 1);
-        const bool okl = fz_wait(mdone(j, b), (uint32_t)(k >> 1) & 1u, abort) && !*abort;
+        bool okl = fz_wait(mdone(j, k), (uint32_t)(k >> 3) & 1u, abort);
+        okl = okl && !*abort;
         const bool okw = __all_sync(0xffffffffu, okl);  // tcgen05.ld is warp-collective
         const int rho = tau - 2 * (j + 1);
         uint32_t v5[NC];
-        fz_take(tlane, j, rho, okw, st == nsteps - 1, v5);
+        fz_take(tlane, j, k, okw, last, v5);
         const bool in_img = okw && rho >= 0 && rho < im.R && x >= 0 && x < im.W;
-        fz_release(tempty(j, b));
+        fz_release(tempty(j, k));
+        // tap partials of row rho: nine chains over c = 0 .. 31, side by side (taps in pairs)
+        const float4* bj = reinterpret_cast<const float4*>(sBM + j * NC);
+        uint64_t tp[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) tp[q] = fz_pk(0.0f, 0.0f);
+        float t8 = 0.0f;
+#pragma unroll
+        for (int c = 0; c < NC; c += 4) {
+          const float4 bb = bj[c / 4];
+          float s0, s1, s2, s3;
+          fz_add2(__uint_as_float(v5[c]), __uint_as_float(v5[c + 1]), bb.x, bb.y, s0, s1);
+          fz_add2(__uint_as_float(v5[c + 2]), __uint_as_float(v5[c + 3]), bb.z, bb.w, s2, s3);
+          const uint32_t h0 = in_img ? fz_relu2(s0, s1) : 0u, h1 = in_img ? fz_relu2(s2, s3) : 0u;
+          const float f[4] = {__uint_as_float(h0 << 16), __uint_as_float(h0 & 0xFFFF0000u), __uint_as_float(h1 << 16),
+                              __uint_as_float(h1 & 0xFFFF0000u)};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float4 wa = *reinterpret_cast<const float4*>(sW6 + (c + e) * 12);
+            const float4 wb = *reinterpret_cast<const float4*>(sW6 + (c + e) * 12 + 4);
+            const float wc = sW6[(c + e) * 12 + 8];
+            const uint64_t f2 = fz_pk(f[e], f[e]);
+            fz_fma2(tp[0], fz_pk(wa.x, wa.y), f2);
+            fz_fma2(tp[1], fz_pk(wa.z, wa.w), f2);
+            fz_fma2(tp[2], fz_pk(wb.x, wb.y), f2);
+            fz_fma2(tp[3], fz_pk(wb.z, wb.w), f2);
+            t8 = __fmaf_rn(wc, f[e], t8);
+          }
+        }
+        // T holds the rows of the steps up to k - 1, and the slot written below
+        // was last read at step k - 1
+        if (k >= 1) fz_wait(tdone(b ^ 1), (uint32_t)((k - 1) >> 1) & 1u, abort);
         // layer 6 at row tau - 10 from the tap partials of earlier steps
-        asm volatile("bar.sync 2, 128;" ::: "memory");
         if (!*abort && out6) {
           float acc = sW6[NC * 12];
 #pragma unroll
@@ -765,34 +883,6 @@ __global__ void __launch_bounds__(FZ_THREADS, 1) k_net_fwd(const __grid_constant
             acc = __fadd_rn(acc, sT[((r6 - 1 + dy) & 3) * FZ_TROW + d * TC_PIX + t + dx]);
           }
           a.out[p6] = m6 * acc;
-        }
-        asm volatile("bar.sync 2, 128;" ::: "memory");
-        // tap partials of layer 5's row rho
-        const float* bj = sBM + j * NC;
-        float f[NC];
-#pragma unroll
-        for (int c = 0; c < NC; c += 2) {
-          float s0, s1;
-          fz_add2(__uint_as_float(v5[c]), __uint_as_float(v5[c + 1]), bj[c], bj[c + 1], s0, s1);
-          f[c] = in_img ? __bfloat162float(__float2bfloat16_rn(fmaxf(s0, 0.0f))) : 0.0f;
-          f[c + 1] = in_img ? __bfloat162float(__float2bfloat16_rn(fmaxf(s1, 0.0f))) : 0.0f;
-        }
-        // nine chains over c = 0 .. 31, side by side (taps in pairs)
-        uint64_t tp[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) tp[q] = fz_pk(0.0f, 0.0f);
-        float t8 = 0.0f;
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          const float4 wa = *reinterpret_cast<const float4*>(sW6 + c * 12);
-          const float4 wb = *reinterpret_cast<const float4*>(sW6 + c * 12 + 4);
-          const float wc = sW6[c * 12 + 8];
-          const uint64_t f2 = fz_pk(f[c], f[c]);
-          fz_fma2(tp[0], fz_pk(wa.x, wa.y), f2);
-          fz_fma2(tp[1], fz_pk(wa.z, wa.w), f2);
-          fz_fma2(tp[2], fz_pk(wb.x, wb.y), f2);
-          fz_fma2(tp[3], fz_pk(wb.z, wb.w), f2);
-          t8 = __fmaf_rn(wc, f[c], t8);
         }
         float* tr = sT + (rho & 3) * FZ_TROW + t + 1;
 #pragma unroll
@@ -803,6 +893,8 @@ __global__ void __launch_bounds__(FZ_THREADS, 1) k_net_fwd(const __grid_constant
           tr[(2 * q + 1) * TC_PIX] = tb;
         }
         tr[8 * TC_PIX] = t8;
+        __syncwarp();
+        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tdone(b)) : "memory");
       }
     }
   } else if (warp >= 8) {
@@ -819,21 +911,19 @@ __global__ void __launch_bounds__(FZ_THREADS, 1) k_net_fwd(const __grid_constant
         fz_unit(a, u, img, r0, r1, x0);
         const int nsteps = r1 - r0 + 15;
         for (int st = 0; st < nsteps && ok; ++st, ++k) {
-          const int tau = r0 - 5 + st, b = (int)(k & 1);
+          const int tau = r0 - 5 + st;
           {
-            if (k >= 1 && !fz_wait(rdy(j, (int)((k - 1) & 1)), (uint32_t)((k - 1) >> 1) & 1u, abort)) {
+            if (k >= 1 && !(j == 0 ? fz_wait(rdy0(k - 1), (uint32_t)((k - 1) >> 3) & 1u, abort)
+                                   : fz_wait(rdy(j, k - 1), (uint32_t)((k - 1) >> 1) & 1u, abort))) {
               ok = false;
               break;
             }
-            // slots are reused four rows later: the epilogue of step k - 2 has read and
-            // zeroed the slot written first here; the first step of a unit also waits
-            // for the step before, whose epilogue cleared the previous unit's slots
-            if (st == 0 && k >= 1) {
-              if (!fz_wait(tempty(j, (int)((k - 1) & 1)), (uint32_t)((k - 1) >> 1) & 1u, abort)) {
-                ok = false;
-                break;
-              }
-            } else if (k >= 2 && !fz_wait(tempty(j, b), (uint32_t)((k - 2) >> 1) & 1u, abort)) {
+            // the slot written first here has been read and zeroed: by the epilogue
+            // that wrote the input row waited for above (layer 5's of step k - 5 for
+            // layer 2); the first step of a unit also waits for the step before,
+            // whose epilogue cleared the rows that the previous unit had begun
+            if ((st == 0 && k >= 1 && !fz_wait(tempty(j, k - 1), (uint32_t)((k - 1) >> 3) & 1u, abort)) ||
+                (j == 0 && k >= 5 && !fz_wait(tempty(NMID - 1, k - 5), (uint32_t)((k - 5) >> 3) & 1u, abort))) {
               ok = false;
               break;
             }
@@ -842,12 +932,12 @@ __global__ void __launch_bounds__(FZ_THREADS, 1) k_net_fwd(const __grid_constant
             // rho (tap rows dy = 0, 1, 2): runs of those whose slots are adjacent
             // in tensor memory take one MMA per (dx, kh), N = 32 x run length
             const int rho = tau - 2 * (j + 1);
-            const uint32_t row = base + (uint32_t)(j * FZ_RINGB + ((rho + 1) & 1) * FZ_ROW);
+            const uint32_t row = base + (uint32_t)(j == 0 ? (int)((k + 7) & 7) * FZ_ROW
+                                                          : FZ_RING0 + (j - 1) * FZ_RINGB + ((rho + 1) & 1) * FZ_ROW);
             const uint32_t wl = base + (uint32_t)(FZ_W + j * TC_W);
             for (int dy = 0; dy < 3;) {
-              const int c0 = fz_col(rho + 2 - dy);
-              int n = 1;
-              while (dy + n < 3 && fz_col(rho + 2 - dy - n) == c0 + 32 * n) ++n;
+              const int c0 = fz_col(j, k + 2 - dy);
+              const int n = min(3 - dy, (512 - c0) / 32);
               const uint32_t idesc = tc_idesc(128, 32 * n);
 #pragma unroll 1
               for (int q = 0; q < 6; ++q) {
@@ -858,16 +948,16 @@ __global__ void __launch_bounds__(FZ_THREADS, 1) k_net_fwd(const __grid_constant
                 asm volatile(
                     "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
                     "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(
-                        tmem + (uint32_t)(j * 128 + c0)),
+                        tmem + (uint32_t)c0),
                     "l"(da), "l"(db), "r"(idesc), "r"(1u));
               }
               dy += n;
             }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             mdone(j, b))
+                             mdone(j, k))
                          : "memory");
-            last_bar = mdone(j, b);
-            last_par = (uint32_t)(k >> 1) & 1u;
+            last_bar = mdone(j, k);
+            last_par = (uint32_t)(k >> 3) & 1u;
           }
         }
       }
@@ -876,67 +966,11 @@ __global__ void __launch_bounds__(FZ_THREADS, 1) k_net_fwd(const __grid_constant
         fz_wait(last_bar, last_par, &never);
       }
     }
-  } else if (warp >= 4) {
-    // layer 1 (warps 4-7): thread t = pixel slot t + 1 of ring 0
-    const int t = tid - 128;
-    int64_t k = 0;
-    for (int64_t u = blockIdx.x; u < a.units; u += gridDim.x) {
-      int img, r0, r1, x0;
-      fz_unit(a, u, img, r0, r1, x0);
-      const int nsteps = r1 - r0 + 15;
-      const int x = x0 - 6 + t;
-      float2 vn[9];
-      fz_window(a, img, r0 - 5, x, vn);
-      for (int st = 0; st < nsteps; ++st, ++k) {
-        const int tau = r0 - 5 + st;
-        // the input window of this step, loaded one step ahead; the next step's now
-        const bool l1_in = tau >= 0 && tau < im.R && x >= 0 && x < im.W;
-        float2 v[9];
-#pragma unroll
-        for (int d = 0; d < 9; ++d) v[d] = vn[d];
-        if (st + 1 < nsteps) fz_window(a, img, tau + 1, x, vn);
-        bool ok = true;
-        if (k >= 1) ok = fz_wait(mdone(0, (int)((k - 1) & 1)), (uint32_t)((k - 1) >> 1) & 1u, abort);
-        uint32_t o[NC / 2];
-#pragma unroll
-        for (int c = 0; c < NC / 2; ++c) o[c] = 0u;
-        if (ok && !*abort && l1_in) {
-          // eight output channels at a time, each one FMA chain in k_l1_fwd's order
-#pragma unroll
-          for (int cg = 0; cg < NC; cg += 8) {
-            uint64_t acc[4];  // channel pairs (cg + 2q, cg + 2q + 1)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[q] = fz_pk(sW1[18 * NC + cg + 2 * q], sW1[18 * NC + cg + 2 * q + 1]);
-#pragma unroll
-            for (int e = 0; e < 18; ++e) {
-              const float4 wa = *reinterpret_cast<const float4*>(sW1 + e * NC + cg);
-              const float4 wb = *reinterpret_cast<const float4*>(sW1 + e * NC + cg + 4);
-              const float xv = (e & 1) ? v[e >> 1].y : v[e >> 1].x;
-              const uint64_t x2 = fz_pk(xv, xv);
-              fz_fma2(acc[0], fz_pk(wa.x, wa.y), x2);
-              fz_fma2(acc[1], fz_pk(wa.z, wa.w), x2);
-              fz_fma2(acc[2], fz_pk(wb.x, wb.y), x2);
-              fz_fma2(acc[3], fz_pk(wb.z, wb.w), x2);
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              float a0, a1;
-              fz_upk(acc[q], a0, a1);
-              const __nv_bfloat162 hv = __floats2bfloat162_rn(fmaxf(a0, 0.0f), fmaxf(a1, 0.0f));
-              o[cg / 2 + q] = *reinterpret_cast<const uint32_t*>(&hv);
-            }
-          }
-        }
-        fz_st_row(base + (uint32_t)((tau & 1) * FZ_ROW + (t + 1) * 64), o);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(rdy(0, (int)(k & 1))) : "memory");
-      }
-    }
   } else {
-    // epilogues of layers 2-4 (warps 0-3): thread i = TMEM lane i = pixel slot i + 1
-    const int i = tid;
-    const uint32_t tlane = tmem + ((uint32_t)(warp * 32) << 16);
+    // epilogues of layers 2-4: warps 0-3 take the even steps, 4-7 the odd ones;
+    // thread i of a group = TMEM lane i = pixel slot i + 1
+    const int i = tid & 127, grp = warp >> 2;
+    const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     int64_t k = 0;
     for (int64_t u = blockIdx.x; u < a.units; u += gridDim.x) {
       int img, r0, r1, x0;
@@ -945,32 +979,32 @@ __global__ void __launch_bounds__(FZ_THREADS, 1) k_net_fwd(const __grid_constant
       const int x = x0 - 6 + i;
       for (int st = 0; st < nsteps; ++st, ++k) {
         const int tau = r0 - 5 + st, b = (int)(k & 1);
+        if (b != grp) continue;
+        const bool last = st == nsteps - 1;
 #pragma unroll 1
         for (int j = 0; j < NMID - 1; ++j) {
-          const bool okl = fz_wait(mdone(j, b), (uint32_t)(k >> 1) & 1u, abort) && !*abort;
+          bool okl = fz_wait(mdone(j, k), (uint32_t)(k >> 3) & 1u, abort);
+          okl = okl && !*abort;
           const bool okw = __all_sync(0xffffffffu, okl);  // tcgen05.ld is warp-collective
           const int rho = tau - 2 * (j + 1);
           uint32_t v[NC];
-          fz_take(tlane, j, rho, okw, st == nsteps - 1, v);
-          fz_release(tempty(j, b));
+          fz_take(tlane, j, k, okw, last, v);
           const bool in_img = okw && rho >= 0 && rho < im.R && x >= 0 && x < im.W;
-          const float* bj = sBM + j * NC;
+          const float4* bj = reinterpret_cast<const float4*>(sBM + j * NC);
           uint32_t o[NC / 2];
 #pragma unroll
-          for (int c = 0; c < NC; c += 2) {
-            float s0, s1;
-            fz_add2(__uint_as_float(v[c]), __uint_as_float(v[c + 1]), bj[c], bj[c + 1], s0, s1);
-            const float f0 = in_img ? fmaxf(s0, 0.0f) : 0.0f;
-            const float f1 = in_img ? fmaxf(s1, 0.0f) : 0.0f;
-            const __nv_bfloat162 hv = __floats2bfloat162_rn(f0, f1);
-            o[c / 2] = *reinterpret_cast<const uint32_t*>(&hv);
+          for (int c = 0; c < NC; c += 4) {
+            const float4 bb = bj[c / 4];
+            float s0, s1, s2, s3;
+            fz_add2(__uint_as_float(v[c]), __uint_as_float(v[c + 1]), bb.x, bb.y, s0, s1);
+            fz_add2(__uint_as_float(v[c + 2]), __uint_as_float(v[c + 3]), bb.z, bb.w, s2, s3);
+            o[c / 2] = in_img ? fz_relu2(s0, s1) : 0u;
+            o[c / 2 + 1] = in_img ? fz_relu2(s2, s3) : 0u;
           }
-          // the row overwritten here was read by layer j + 3's MMAs of the step
-          // before: layers 3 and 4 were waited for above at that step, layer 5's
-          // completion (waited by warps 4-7) is waited for here
-          if (j == NMID - 2 && k >= 1)
-            fz_wait(mdone(NMID - 1, (int)((k - 1) & 1)), (uint32_t)((k - 1) >> 1) & 1u, abort);
-          fz_st_row(base + (uint32_t)((j + 1) * FZ_RINGB + (rho & 1) * FZ_ROW + (i + 1) * 64), o);
+          // the row overwritten here was read by layer j + 3's MMAs of the step before
+          if (k >= 1) fz_wait(mdone(j + 1, k - 1), (uint32_t)((k - 1) >> 3) & 1u, abort);
+          fz_release(tempty(j, k));
+          fz_st_row(base + (uint32_t)(FZ_RING0 + j * FZ_RINGB + (rho & 1) * FZ_ROW + (i + 1) * 64), o);
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           __syncwarp();
           if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(rdy(j + 1, b)) : "memory");
