@@ -61,7 +61,8 @@ N_FULL = 256
 # level-0 Chebyshev step: reads x, b, d and writes x_out, d per computational point
 CHEB_BYTES_PER_DOF = {"f32": 20, "f64": 40}
 # leapfrog step per computational point: reads u^n, u^{n-1}, the node code, writes u^{n+1}
-LEAPFROG_BYTES_PER_DOF = {"f32": 13, "f64": 25}
+# (FP32: both fields and the code read and both fields written once per 8 steps)
+LEAPFROG_BYTES_PER_DOF = {"f32": 17 / 8, "f64": 25}
 # one 32 -> 32 convolution of the learned stage per pixel: 2 x 9 x 32 x 32 FLOP
 CONV_FLOP_PER_PX = 18432
 # and its bytes per pixel: 32 BF16 channels read and 32 written
@@ -1046,7 +1047,11 @@ def stencil_subrecords(ctx, args, h3):
     dt = 0.9 * grid.h / math.sqrt(2.0)
     u0 = torch.tensor(ei.pulse(X, Y, c, w), device=ctx.dev)
     u1 = u0 - 0.5 * dt * dt * hw.apply(u0)
-    for name, dtype, bpd in (("leapfrog_4096sq_f32", torch.float32, 13), ("leapfrog_4096sq_f64", torch.float64, 25)):
+    f32_kernel = "k_leapfrog_block (8 steps per launch; bytes and time per step)"
+    f64_kernel = "k_leapfrog<double, 2> (one launch per step, 32-step CUDA-graph chunks)"
+    for name, dtype, bpd, kernel in (
+            ("leapfrog_4096sq_f32", torch.float32, LEAPFROG_BYTES_PER_DOF["f32"], f32_kernel),
+            ("leapfrog_4096sq_f64", torch.float64, LEAPFROG_BYTES_PER_DOF["f64"], f64_kernel)):
         a0, b0 = u0.to(dtype), u1.to(dtype)
         a, bb = torch.empty_like(a0), torch.empty_like(b0)
         ts = []
@@ -1059,9 +1064,7 @@ def stencil_subrecords(ctx, args, h3):
             if i >= 3:
                 ts.append(t)
         step_s = statistics.mean(ts) / 1000.0 / SUB_WAVE_STEPS
-        out[name] = {"bound": "hbm", "kernel": f"k_leapfrog<{'float' if dtype == torch.float32 else 'double'}, 2> "
-                                               "(one launch per step, 32-step CUDA-graph chunks)",
-                     "achieved": bpd * ncw / step_s / 1e9, "peak": hbm, "unit": "GB/s",
+        out[name] = {"bound": "hbm", "kernel": kernel, "achieved": bpd * ncw / step_s / 1e9, "peak": hbm, "unit": "GB/s",
                      "frac": bpd * ncw / step_s / 1e9 / hbm, "algorithmic_bytes_per_launch": bpd * ncw,
                      "avg_launch_us": step_s * 1e6, "num_cp": ncw, "tile": tile,
                      "timing": f"CUDA events around a {SUB_WAVE_STEPS}-step wave_step call (L2 flushed before it); "
@@ -1140,8 +1143,8 @@ def gpu_wave(ctx, args):
                      "dof_steps_per_s": nc * nsteps / (statistics.mean(f64) / 1000.0),
                      "max_rel_diff_f32_vs_f64_after_run": diff},
             "roofline": {"bound": "hbm",
-                         "kernel": "k_leapfrog<float, 2> (one launch per step in 32-step CUDA-graph chunks; bytes and "
-                                   "time per 10,000-step wave_step call)",
+                         "kernel": "k_leapfrog_block (8 steps per launch, in registers; bytes and time per 10,000-step "
+                                   "wave_step call; issue-bound)",
                          "achieved": achieved, "peak": pk["hbm_gbs"], "peak_kind": kind, "unit": "GB/s",
                          "frac": achieved / pk["hbm_gbs"], "traffic": None,
                          "algorithmic_bytes_per_launch": alg, "avg_launch_us": launch_s * 1e6,
