@@ -53,29 +53,50 @@ struct Image {
   __device__ int64_t npx() const { return (int64_t)W * H; }
 };
 
+// Packed FP32 pairs: fma.rn.f32x2 is two round-to-nearest FMAs in one
+// instruction, so each lane's result is the scalar __fmaf_rn's at half the FMA
+// instructions.
+__device__ __forceinline__ uint64_t fz_pk(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void fz_upk(uint64_t v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ void fz_fma2(uint64_t& acc, uint64_t w, uint64_t x) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(w), "l"(x));
+}
+// (max(a, 0), max(b, 0)) in bf16: rounding keeps the sign and the order, so the
+// packed maximum after it equals the two FP32 ones before it (NaN gives 0 in both)
+__device__ __forceinline__ uint32_t fz_relu2(float a, float b) {
+  const __nv_bfloat162 h = __hmax2(__floats2bfloat162_rn(a, b), __floats2bfloat162_rn(0.0f, 0.0f));
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+
 // ------------------------------------------------------------ forward
 // layer 1 (2 -> 32) + ReLU; in: (s_hat, m) per pixel.  A thread computes two
-// x-adjacent pixels: the 3 x 4 input window is loaded once and every weight
-// -- read from shared memory as float4s, two taps' two channels at a time --
-// is applied to both pixels, one FMA per multiply-add.
+// x-adjacent pixels of two rows: the 4 x 4 input window is loaded once and every
+// weight read from shared memory serves the four, in packed FMAs over channel
+// pairs; each output is one FMA chain b, then (tap, input channel) in order.
+// Bounded by the FMA pipe and the issue slots.  16 x 512^2: 116 us; 173 us
+// with two pixels of one row, scalar FMAs and a channel's weights at a time.
 __global__ void __launch_bounds__(128) k_l1_fwd(Image im, const float2* __restrict__ in, const float* __restrict__ P,
                                                 bf16* __restrict__ y) {
-  constexpr int WS = 20;  // a channel's 9 x 2 weights padded to five float4s
-  __shared__ __align__(16) float w[NC * WS + NC];
-  for (int i = threadIdx.x; i < NC * WS; i += blockDim.x) {
-    const int co = i / WS, j = i % WS;
-    w[i] = j < 18 ? P[OFF_W1 + co * 18 + j] : 0.0f;
-  }
-  for (int i = threadIdx.x; i < NC; i += blockDim.x) w[NC * WS + i] = P[OFF_W1 + W1_N + i];
+  __shared__ __align__(16) float w[18 * NC + NC];  // weight (tap, input) of the 32 outputs contiguous, then b
+  for (int i = threadIdx.x; i < 18 * NC; i += blockDim.x) w[i] = P[OFF_W1 + (i % NC) * 18 + i / NC];
+  for (int i = threadIdx.x; i < NC; i += blockDim.x) w[18 * NC + i] = P[OFF_W1 + W1_N + i];
   __syncthreads();
-  const int half = (im.W + 1) >> 1;
+  const int half = (im.W + 1) >> 1, rp = (im.R + 1) >> 1;
   const int64_t pp = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (pp >= (int64_t)half * im.H) return;
-  const int r = (int)(pp / half), x = 2 * (int)(pp - (int64_t)r * half);
-  const int lo = (r / im.R) * im.R, hi = lo + im.R;
-  float2 v[3][4];
+  const int64_t q = pp / half;
+  const int img = (int)(q / rp);
+  const int lo = img * im.R, hi = lo + im.R;
+  if (lo >= im.H) return;
+  const int x = 2 * (int)(pp - q * half), r = lo + 2 * (int)(q - (int64_t)img * rp);
+  float2 v[4][4];
 #pragma unroll
-  for (int dy = 0; dy < 3; ++dy) {
+  for (int dy = 0; dy < 4; ++dy) {
     const int rr = r + dy - 1;
 #pragma unroll
     for (int dx = 0; dx < 4; ++dx) {
@@ -83,44 +104,51 @@ __global__ void __launch_bounds__(128) k_l1_fwd(Image im, const float2* __restri
       v[dy][dx] = (xx >= 0 && xx < im.W && rr >= lo && rr < hi) ? in[(int64_t)rr * im.W + xx] : make_float2(0.f, 0.f);
     }
   }
-  uint32_t o0[NC / 2], o1[NC / 2];
+  bf16* const y0 = y + ((int64_t)r * im.W + x) * NC;
+  const bool okx = x + 1 < im.W, oky = r + 1 < hi;
+#pragma unroll 1
+  for (int c16 = 0; c16 < NC; c16 += 16) {
+    uint32_t o[4][8];
 #pragma unroll
-  for (int co = 0; co < NC; co += 2) {
-    float a[2][2];
+    for (int g = 0; g < 2; ++g) {
+      const int cg = c16 + 8 * g;
+      uint64_t acc[4][4];  // [pixel 2 row + column][channel pair]
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const float* wc = w + (co + k) * WS;
-      float a0 = w[NC * WS + co + k], a1 = a0;
+      for (int k = 0; k < 4; ++k)
 #pragma unroll
-      for (int q = 0; q < 5; ++q) {
-        const float4 t = *reinterpret_cast<const float4*>(wc + 4 * q);
-        const int d0 = 2 * q, d1 = 2 * q + 1;
-        a0 = fmaf(t.x, v[d0 / 3][d0 % 3].x, a0);
-        a0 = fmaf(t.y, v[d0 / 3][d0 % 3].y, a0);
-        a1 = fmaf(t.x, v[d0 / 3][d0 % 3 + 1].x, a1);
-        a1 = fmaf(t.y, v[d0 / 3][d0 % 3 + 1].y, a1);
-        if (d1 < 9) {
-          a0 = fmaf(t.z, v[d1 / 3][d1 % 3].x, a0);
-          a0 = fmaf(t.w, v[d1 / 3][d1 % 3].y, a0);
-          a1 = fmaf(t.z, v[d1 / 3][d1 % 3 + 1].x, a1);
-          a1 = fmaf(t.w, v[d1 / 3][d1 % 3 + 1].y, a1);
+        for (int c = 0; c < 4; ++c) acc[k][c] = *reinterpret_cast<const uint64_t*>(w + 18 * NC + cg + 2 * c);
+#pragma unroll
+      for (int e = 0; e < 18; ++e) {
+        const float4 wa = *reinterpret_cast<const float4*>(w + e * NC + cg);
+        const float4 wb = *reinterpret_cast<const float4*>(w + e * NC + cg + 4);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float2 t = v[(e >> 1) / 3 + (k >> 1)][(e >> 1) % 3 + (k & 1)];
+          const float xv = (e & 1) ? t.y : t.x;
+          const uint64_t x2 = fz_pk(xv, xv);
+          fz_fma2(acc[k][0], fz_pk(wa.x, wa.y), x2);
+          fz_fma2(acc[k][1], fz_pk(wa.z, wa.w), x2);
+          fz_fma2(acc[k][2], fz_pk(wb.x, wb.y), x2);
+          fz_fma2(acc[k][3], fz_pk(wb.z, wb.w), x2);
         }
       }
-      a[k][0] = fmaxf(a0, 0.0f);
-      a[k][1] = fmaxf(a1, 0.0f);
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          float a0, a1;
+          fz_upk(acc[k][c], a0, a1);
+          o[k][4 * g + c] = fz_relu2(a0, a1);
+        }
     }
-    const __nv_bfloat162 h0 = __floats2bfloat162_rn(a[0][0], a[1][0]);
-    const __nv_bfloat162 h1 = __floats2bfloat162_rn(a[0][1], a[1][1]);
-    o0[co / 2] = *reinterpret_cast<const uint32_t*>(&h0);
-    o1[co / 2] = *reinterpret_cast<const uint32_t*>(&h1);
-  }
-  const int64_t p = (int64_t)r * im.W + x;
-  int4* dst = reinterpret_cast<int4*>(y + p * NC);
 #pragma unroll
-  for (int q = 0; q < 4; ++q) dst[q] = make_int4(o0[4 * q], o0[4 * q + 1], o0[4 * q + 2], o0[4 * q + 3]);
-  if (x + 1 < im.W) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) dst[4 + q] = make_int4(o1[4 * q], o1[4 * q + 1], o1[4 * q + 2], o1[4 * q + 3]);
+    for (int k = 0; k < 4; ++k) {
+      if ((k & 1) && !okx) continue;
+      if ((k >> 1) && !oky) continue;
+      int4* dst = reinterpret_cast<int4*>(y0 + ((int64_t)(k >> 1) * im.W + (k & 1)) * NC + c16);
+      dst[0] = make_int4(o[k][0], o[k][1], o[k][2], o[k][3]);
+      dst[1] = make_int4(o[k][4], o[k][5], o[k][6], o[k][7]);
+    }
   }
 }
 
@@ -631,32 +659,11 @@ __device__ __forceinline__ void fz_release(uint32_t tempty) {
   if ((threadIdx.x & 31) == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty) : "memory");
 }
 
-// Packed FP32 pairs: fma.rn.f32x2 is two round-to-nearest FMAs in one
-// instruction, so each lane's result is the scalar __fmaf_rn's while the
-// fused kernel's CUDA-core layers issue half the FMA instructions.
-__device__ __forceinline__ uint64_t fz_pk(float a, float b) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void fz_upk(uint64_t v, float& a, float& b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ void fz_fma2(uint64_t& acc, uint64_t w, uint64_t x) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(w), "l"(x));
-}
 // (a0 + b0, a1 + b1), each rounded to nearest as a scalar addition
 __device__ __forceinline__ void fz_add2(float a0, float a1, float b0, float b1, float& r0, float& r1) {
   uint64_t r;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(fz_pk(a0, a1)), "l"(fz_pk(b0, b1)));
   fz_upk(r, r0, r1);
-}
-
-// (max(a, 0), max(b, 0)) in bf16: rounding keeps the sign and the order, so the
-// packed maximum after it equals the two FP32 ones before it (NaN gives 0 in both)
-__device__ __forceinline__ uint32_t fz_relu2(float a, float b) {
-  const __nv_bfloat162 h = __hmax2(__floats2bfloat162_rn(a, b), __floats2bfloat162_rn(0.0f, 0.0f));
-  return *reinterpret_cast<const uint32_t*>(&h);
 }
 
 __device__ __forceinline__ void fz_unit(const FzArgs& a, int64_t u, int& img, int& r0, int& r1, int& x0) {
@@ -1917,8 +1924,9 @@ static void pack(NN& N, cudaStream_t s, int64_t& nl) {
 static void forward(NN& N, const Image& im, const float2* in, float* out, cudaStream_t s, int64_t& nl,
                     Solver* prof = nullptr) {
   const int64_t npx = npx_of(im);
-  const int64_t npairs = (int64_t)((im.W + 1) / 2) * im.H;  // layer 1: two pixels per thread
-  k_l1_fwd<<<blocks_for(npairs, 128), 128, 0, s>>>(im, in, N.P, N.act[1]);
+  // layer 1: two pixels of two rows per thread
+  const int64_t nquads = (int64_t)((im.W + 1) / 2) * ((im.R + 1) / 2) * (im.H / im.R);
+  k_l1_fwd<<<blocks_for(nquads, 128), 128, 0, s>>>(im, in, N.P, N.act[1]);
   for (int l = 0; l < NMID; ++l) {
     const bool own = N.prof && !prof;  // events of the handle (not inside a solver's graph)
     if (own) {
