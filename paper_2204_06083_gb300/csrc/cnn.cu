@@ -517,13 +517,13 @@ __global__ void k_l6_fwd(Image im, const bf16* __restrict__ y5, const float* __r
 // tdone (T row of step k written and read: layers 5-6 take turns).  A parity
 // wait is sound while its barrier is neither two phases ahead nor one behind:
 // eight barriers per layer for mdone, tempty and rdy0 and two for rdy and tdone
-// give that, whatever the warps' relative speeds (a random-schedule model of
-// the roles, with these waits, found four too few for mdone).  Every wait is
+// give that, whatever the warps' relative speeds (with four for mdone a slow
+// epilogue warp can miss a phase).  Every wait is
 // bounded; one that gives up raises a shared abort flag, after which every role
 // runs its remaining steps without waiting or computing, the CTA waits
 // (bounded) for its MMAs in flight, frees TMEM and sets *err.
-// Bound by the issue slots and the shared-memory pipe together (68 % and 79 %
-// busy; the tensor pipe 36 %).  At 2048^2: 441 us; 561 us with one group of
+// Bound by the issue slots and the shared-memory pipe together (70 % and 75 %
+// busy; the tensor pipe 38 %).  At 2048^2: 440 us; 561 us with one group of
 // warps per role, whose epilogue (3200 cycles of work in a step of 4280) paced
 // the others, and four slots per layer (9 MMAs per step instead of 6.75); with
 // one row per thread in layer 1 and 24 warps 451 us.
@@ -535,13 +535,13 @@ constexpr int FZ_W = 114 * 1024;                       // weights of layers 2-5:
 constexpr int FZ_WDX = 4 * 96 * 16;                    // B bytes of one horizontal tap: 6144
 constexpr int FZ_TRING = 4;                            // rows of the tap-partial ring
 constexpr int FZ_TROW = 9 * TC_PIX;                    // floats of a T row: 9 taps x 130 slots
-constexpr int FZ_T = FZ_W + NMID * TC_W;               // 140,288
-constexpr int FZ_W1 = FZ_T + FZ_TRING * FZ_TROW * 4;   // 159,008: layer-1 weights [d][ci][co], then b1
-constexpr int FZ_W6 = FZ_W1 + (NC * 20 + NC) * 4;      // 161,696: W6 as [c][12 taps], then b6
-constexpr int FZ_BM = FZ_W6 + 1552;                    // 163,248: biases of layers 2-5
-constexpr int FZ_BAR = FZ_BM + NMID * NC * 4;          // 163,760
+constexpr int FZ_T = FZ_W + NMID * TC_W;               // 190,464
+constexpr int FZ_W1 = FZ_T + FZ_TRING * FZ_TROW * 4;   // 209,184: layer-1 weights [d][ci][co], then b1
+constexpr int FZ_W6 = FZ_W1 + (NC * 20 + NC) * 4;      // 211,872: W6 as [c][12 taps], then b6
+constexpr int FZ_BM = FZ_W6 + 1552;                    // 213,424: biases of layers 2-5
+constexpr int FZ_BAR = FZ_BM + NMID * NC * 4;          // 213,936
 constexpr int FZ_NBAR = 80;
-constexpr int FZ_SMEM = FZ_BAR + 8 * FZ_NBAR + 16;     // 163,968
+constexpr int FZ_SMEM = FZ_BAR + 8 * FZ_NBAR + 16;     // 214,592
 constexpr int FZ_THREADS = 896;  // warps 0-7 epilogues 2-4, 8-11 MMAs, 12-19 layers 5-6, 20-27 layer 1
 static_assert(FZ_SMEM <= 232448, "fused forward: shared memory");
 static_assert(FZ_W % 1024 == 0 && FZ_T % 16 == 0 && FZ_BAR % 8 == 0, "fused forward: alignment");
