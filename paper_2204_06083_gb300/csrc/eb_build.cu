@@ -56,6 +56,27 @@ __device__ double psi_star(const LSDev& L, double x, double y) {
   return __dsub_rn(rho, r);
 }
 
+// psi_star by LP adjacent lanes (lane g of the group, mask = its lanes): the
+// lanes form a harmonic each, every lane adds them up in psi_star's order
+template <int LP>
+__device__ double psi_star_lanes(const LSDev& L, double x, double y, int g, unsigned mask) {
+  if constexpr (LP == 1) return psi_star(L, x, y);
+  double dx = __dsub_rn(x, L.c[0]);
+  double dy = __dsub_rn(y, L.c[1]);
+  double rho = __dsqrt_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
+  double phi = atan2(dy, dx);
+  double r = L.r0;
+  for (int j0 = 0; j0 < L.nk; j0 += LP) {
+    const int j = min(j0 + g, L.nk - 1);
+    const double v = __dmul_rn(L.a[j], sin(__dadd_rn(__dmul_rn((double)L.k[j], phi), L.p[j])));
+    for (int t = 0; t < LP; ++t) {
+      const double w = __shfl_sync(mask, v, t, LP);
+      if (j0 + t < L.nk) r = __dadd_rn(r, w);
+    }
+  }
+  return __dsub_rn(rho, r);
+}
+
 __device__ double psi_at(const LSDev& L, const double* x) {
   return L.kind == EB_LS_QUADRIC ? psi_quadric(L, x) : psi_star(L, x[0], x[1]);
 }
@@ -92,13 +113,17 @@ __device__ double quadric_root(const LSDev& L, const double* p, int axis, double
 
 // Illinois iteration on g(t) = psi(p + sign t e_axis) over [ta, tb],
 // g(ta) < 0 <= g(tb); stops at g == 0 or when the iterate moves <= 1e-15 h.
+// LP adjacent lanes per root, all with the same arguments and result.
+template <int LP>
 __device__ double star_root(const LSDev& L, const double* p, int axis, double sign, double ta, double tb,
                             double h) {
+  const int g0 = threadIdx.x & (LP - 1);
+  const unsigned mask = LP == 1 ? 0u : ((1u << LP) - 1u) << ((threadIdx.x & 31) - g0);
   double q[2] = {p[0], p[1]};
   auto g = [&](double t) {
     double qq[2] = {q[0], q[1]};
     qq[axis] = __dadd_rn(p[axis], __dmul_rn(sign, t));
-    return psi_star(L, qq[0], qq[1]);
+    return psi_star_lanes<LP>(L, qq[0], qq[1], g0, mask);
   };
   double fa = g(ta), fb = g(tb);
   double t = tb;
@@ -245,62 +270,90 @@ __global__ void k_cp_mask(Geometry G, uint8_t* code, const int32_t* cp_off, int3
   ncut[k] = __popc((unsigned)m);
 }
 
-// pass 4: per CP, its cuts (walk + root) and the diagonal D_k = sum_s c_s
-__global__ void k_cut(Geometry G, LSDev L, const double* psi, const uint8_t* code, const int32_t* cp_node,
-                      const int32_t* cut_off, int64_t num_cp, double* diag, int32_t* cut_cp, int32_t* cut_dir,
-                      double* cut_delta, double* cut_c, double* cut_xg, int32_t* cut_far, BuildStats* st) {
+// pass 4a: the list of cuts, in the order of the CPs and their directions
+__global__ void k_cut_list(const uint8_t* code, const int32_t* cp_node, const int32_t* cut_off, int64_t num_cp,
+                           int ndir, int32_t* cut_cp, int32_t* cut_dir) {
   int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= num_cp) return;
-  int64_t node = cp_node[k];
-  uint8_t m = code[node] & 0x3F;
-  double D = 0.0, margin = 0.0;
+  const uint8_t m = code[cp_node[k]] & 0x3F;
+  if (!m) return;
   int j = cut_off[k];
+  for (int s = 0; s < ndir; ++s)
+    if (m & (1u << s)) {
+      cut_cp[j] = (int32_t)k;
+      cut_dir[j] = s;
+      ++j;
+    }
+}
+
+// pass 4b: walk and root of every cut, LP adjacent lanes each.  The root of a
+// star is a chain of some ten evaluations of FP64 functions, which takes a warp
+// the same time for one lane as for 32, so the cuts are packed into full warps
+// (one thread per CP over all directions: 259 us on a 514 x 501 star, 66 us
+// with this pass) and, while that leaves schedulers idle, eight or four lanes
+// share a root's harmonics.
+template <int LP>
+__global__ void k_cut(Geometry G, LSDev L, const double* psi, const int32_t* cp_node, int64_t num_cut,
+                      const int32_t* cut_cp, const int32_t* cut_dir, double* cut_delta, double* cut_c, double* cut_xg,
+                      int32_t* cut_far, BuildStats* st) {
+  const int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / LP;
+  if (j >= num_cut) return;
+  const int64_t node = cp_node[cut_cp[j]];
+  const int s = cut_dir[j];
   int64_t i[3];
   unflatten(G, node, i);
   const double h = G.h;
-  for (int s = 0; s < 2 * G.dim; ++s) {
+  const int axis = s >> 1;
+  const int sg = (s & 1) ? 1 : -1;
+  const int64_t st_ax = stride_of(G, axis) * sg;
+  int64_t cur = node + 2 * st_ax;  // past the BP
+  int64_t mm = 1;
+  while (psi[cur] < 0.0) {
+    ++mm;
+    cur += st_ax;
+  }
+  double p[3];
+  for (int a = 0; a < 3; ++a) {
+    int64_t ia = i[a] + (a == axis ? sg : 0);
+    p[a] = a < G.dim ? node_coord(G.lo[a], ia, h) : 0.0;
+  }
+  double delta;
+  if (L.kind == EB_LS_QUADRIC) {
+    delta = quadric_root(L, p, axis, (double)sg);
+  } else if (L.kind == EB_LS_SAMPLED) {
+    // linear ratio between the last inside node and the first outside one
+    // (Sec. 3.3): delta = (mm - 1) h + psi_in / (psi_in - psi_out) h
+    const double pin = psi[cur - st_ax], pout = psi[cur];
+    delta = __dadd_rn(__dmul_rn((double)(mm - 1), h), __dmul_rn(__ddiv_rn(pin, __dsub_rn(pin, pout)), h));
+  } else {
+    double ta = __dmul_rn((double)(mm - 1), h);
+    double tb = __dmul_rn((double)mm, h);
+    delta = star_root<LP>(L, p, axis, (double)sg, ta, tb, h);
+  }
+  if (LP > 1 && (threadIdx.x & (LP - 1))) return;
+  cut_delta[j] = delta;
+  cut_far[j] = mm > 1;  // the node past the BP is inside
+  cut_c[j] = __ddiv_rn(h, __dadd_rn(h, delta));
+  for (int a = 0; a < G.dim; ++a)
+    cut_xg[j * G.dim + a] = (a == axis) ? __dadd_rn(p[a], __dmul_rn((double)sg, delta)) : p[a];
+  if (delta > h) atomicAdd(&st->num_far, 1ull);
+  atomic_max_pos(&st->max_delta_over_h, fabs(delta / h));
+}
+
+// pass 4c: the diagonal D_k = sum_s c_s (1 towards a CP)
+__global__ void k_cut_diag(const uint8_t* code, const int32_t* cp_node, const int32_t* cut_off, const double* cut_c,
+                           int64_t num_cp, int ndir, double* diag, BuildStats* st) {
+  int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= num_cp) return;
+  const int64_t node = cp_node[k];
+  const uint8_t m = code[node] & 0x3F;
+  double D = 0.0, margin = 0.0;
+  int j = cut_off[k];
+  for (int s = 0; s < ndir; ++s) {
     double cs = 1.0;
     if (m & (1u << s)) {
-      int axis = s >> 1;
-      int sg = (s & 1) ? 1 : -1;
-      int64_t st_ax = stride_of(G, axis) * sg;
-      int64_t bp = node + st_ax;
-      int64_t cur = bp + st_ax;
-      int64_t mm = 1;
-      while (psi[cur] < 0.0) {
-        ++mm;
-        cur += st_ax;
-      }
-      double p[3];
-      for (int a = 0; a < 3; ++a) {
-        int64_t ia = i[a] + (a == axis ? sg : 0);
-        p[a] = a < G.dim ? node_coord(G.lo[a], ia, h) : 0.0;
-      }
-      double delta;
-      if (L.kind == EB_LS_QUADRIC) {
-        delta = quadric_root(L, p, axis, (double)sg);
-      } else if (L.kind == EB_LS_SAMPLED) {
-        // linear ratio between the last inside node and the first outside one
-        // (Sec. 3.3): delta = (mm - 1) h + psi_in / (psi_in - psi_out) h
-        const double pin = psi[cur - st_ax], pout = psi[cur];
-        delta = __dadd_rn(__dmul_rn((double)(mm - 1), h), __dmul_rn(__ddiv_rn(pin, __dsub_rn(pin, pout)), h));
-      } else {
-        double ta = __dmul_rn((double)(mm - 1), h);
-        double tb = __dmul_rn((double)mm, h);
-        delta = star_root(L, p, axis, (double)sg, ta, tb, h);
-      }
-      cs = __ddiv_rn(h, __dadd_rn(h, delta));
-      cut_cp[j] = (int32_t)k;
-      cut_dir[j] = s;
-      cut_delta[j] = delta;
-      cut_far[j] = mm > 1;  // the node past the BP is inside
-      cut_c[j] = cs;
-      for (int a = 0; a < G.dim; ++a)
-        cut_xg[(int64_t)j * G.dim + a] = (a == axis) ? __dadd_rn(p[a], __dmul_rn((double)sg, delta)) : p[a];
-      if (delta > h) atomicAdd(&st->num_far, 1ull);
-      atomic_max_pos(&st->max_delta_over_h, fabs(delta / h));
+      cs = cut_c[j++];
       margin = __dadd_rn(margin, cs);
-      ++j;
     }
     D = (s == 0) ? cs : __dadd_rn(D, cs);
   }
@@ -748,8 +801,20 @@ void build_handle(EBHandle& eb, const eb_grid& grid, const eb_levelset& ls, cuda
   eb.cut_c = dalloc<double>(nc, s, false);
   eb.cut_xg = dalloc<double>((int64_t)nc * G.dim, s, false);
   int32_t* cut_far = dalloc<int32_t>(nc, s, false);
-  k_cut<<<blocks_for(ncp, 128), 128, 0, s>>>(G, L, psi, eb.code, eb.cp_node, eb.cut_off, ncp, eb.diag, eb.cut_cp,
-                                             eb.cut_dir, eb.cut_delta, eb.cut_c, eb.cut_xg, cut_far, st);
+  if (nc > 0) {
+    k_cut_list<<<blocks_for(ncp, T), T, 0, s>>>(eb.code, eb.cp_node, eb.cut_off, ncp, 2 * G.dim, eb.cut_cp, eb.cut_dir);
+    auto roots = [&](auto lanes) {
+      constexpr int LP = decltype(lanes)::value;
+      k_cut<LP><<<blocks_for(LP * (int64_t)nc, 32), 32, 0, s>>>(G, L, psi, eb.cp_node, nc, eb.cut_cp, eb.cut_dir,
+                                                                eb.cut_delta, eb.cut_c, eb.cut_xg, cut_far, st);
+    };
+    // several lanes per root while that is one warp per scheduler at most
+    const bool share = L.kind == EB_LS_STAR2D && L.nk > 1;
+    if (share && nc <= (int64_t)num_sms() * 16) roots(std::integral_constant<int, 8>{});
+    else if (share && nc <= (int64_t)num_sms() * 32) roots(std::integral_constant<int, 4>{});
+    else roots(std::integral_constant<int, 1>{});
+  }
+  k_cut_diag<<<blocks_for(ncp, T), T, 0, s>>>(eb.code, eb.cp_node, eb.cut_off, eb.cut_c, ncp, 2 * G.dim, eb.diag, st);
   EB_CUDA(cudaGetLastError());
   eb.closure = closure;
   double rbf_margin = 0.0;
