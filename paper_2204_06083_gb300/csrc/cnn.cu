@@ -23,6 +23,7 @@
 #include "tma.cuh"
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <utility>
 #include <vector>
@@ -1803,7 +1804,15 @@ __global__ void k_st_correct(int64_t nn, const uint8_t* __restrict__ code, const
 }
 
 // ---------------------------------------------------------------- host
+static uint64_t next_state() {
+  static std::atomic<uint64_t> n{0};
+  return ++n;
+}
+
 struct NN {
+  // of the buffers and the route that a captured stage holds (nn_stage_state):
+  // renewed when one is reallocated or the forward path changes
+  uint64_t state = next_state();
   float* P = nullptr;  // FP32 master parameters
   float* G = nullptr;  // gradient
   float* m = nullptr;  // Adam moments
@@ -1886,6 +1895,7 @@ static void conv32(const Image& im, const bf16* x, const bf16* wk, const float* 
 
 static void ensure_act(NN& N, int64_t px, cudaStream_t s) {
   if (px <= N.cap_px) return;
+  N.state = next_state();
   for (int l = 1; l <= 5; ++l) dfree(N.act[l], s);
   dfree(N.gA, s); dfree(N.gB, s); dfree(N.out, s); dfree(N.dout, s); dfree(N.in, s); dfree(N.code, s);
   dfree(N.diag, s);
@@ -2067,12 +2077,15 @@ struct nn_handle {
 
 namespace ebk {
 
+uint64_t nn_stage_state(const nn_handle* h) { return h ? h->n.state : 0; }
+
 void nn_stage_prepare(nn_handle* h, const EBHandle& eb, cudaStream_t s) {
   NN& N = h->n;
   EB_REQUIRE(eb.g.dim == 2, EB_ERR_INVALID, "learned stage: 2D grids only");
   const int64_t nn = eb.g.num_nodes;
   ensure_act(N, nn, s);
   if (nn > N.cap_nodes) {
+    N.state = next_state();
     dfree(N.s64, s);
     dfree(N.spart, s);
     N.cap_nodes = 0;
@@ -2187,6 +2200,7 @@ int nn_set_fused(nn_handle* h, int on) {
     set_error("nn_set_fused: NULL handle");
     return EB_ERR_INVALID;
   }
+  if (h->n.fused != (on != 0)) h->n.state = next_state();
   h->n.fused = on != 0;
   return EB_OK;
 }

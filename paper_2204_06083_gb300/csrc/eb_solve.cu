@@ -1043,7 +1043,7 @@ void Solver::iteration(int kind, cudaStream_t s, const cudaGraphConditionalHandl
 // capture runs on a private stream forked from s, so s may be the legacy
 // default stream.
 void Solver::graph_prepare(int kind, int iters, int profile, cudaStream_t s) {
-  if (gexec && g_iters == iters && g_kind == kind && g_prof == profile && g_nn == nn &&
+  if (gexec && g_iters == iters && g_kind == kind && g_prof == profile && g_nn == nn_stage_state(nn) &&
       g_nn_mode == nn_mode && g_tile_gen == eb->tile_gen && g_df == (int)df_on)
     return;
   if (prof_on) {  // settle event pairs recorded so far before the capture reuses them
@@ -1073,7 +1073,7 @@ void Solver::graph_prepare(int kind, int iters, int profile, cudaStream_t s) {
   g_iters = iters;
   g_kind = kind;
   g_prof = profile;
-  g_nn = nn;
+  g_nn = nn_stage_state(nn);
   g_nn_mode = nn_mode;
   g_tile_gen = eb->tile_gen;
   g_df = (int)df_on;
@@ -1122,7 +1122,7 @@ cudaGraphExec_t build_while_graph(cudaStream_t cap,
 // Captures the device-side loop { while (!done && iters < maxit) iteration }
 // (once per argument set).
 void Solver::loop_prepare(int kind) {
-  if (lexec && l_kind == kind && l_nn == nn && l_nn_mode == nn_mode &&
+  if (lexec && l_kind == kind && l_nn == nn_stage_state(nn) && l_nn_mode == nn_mode &&
       l_tile_gen == eb->tile_gen && l_df == (int)df_on)
     return;
   loop_release();
@@ -1133,7 +1133,7 @@ void Solver::loop_prepare(int kind) {
   l_launches = nlaunch - n0;
   nlaunch = n0;
   l_kind = kind;
-  l_nn = nn;
+  l_nn = nn_stage_state(nn);
   l_nn_mode = nn_mode;
   l_tile_gen = eb->tile_gen;
   l_df = (int)df_on;

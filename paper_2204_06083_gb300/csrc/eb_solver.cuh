@@ -88,10 +88,11 @@ struct Solver {
   double prof_acc_ms = 0.0;
   int prof_acc_n = 0;
   // captured PCG iteration (CUDA graph), keyed by what it depends on: neither b
-  // nor x, whose address the iteration takes from sc
+  // nor x, whose address the iteration takes from sc, but the state of the
+  // learned stage (nn_stage_state), whose buffers and route it holds
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t gexec = nullptr;
-  const nn_handle* g_nn = nullptr;
+  uint64_t g_nn = 0;
   int g_tile_gen = -1;
   int g_nn_mode = -1;
   int g_iters = 0, g_kind = -1, g_prof = -1, g_pairs = 0;
@@ -100,7 +101,7 @@ struct Solver {
   // body is one iteration (no host round trip per iteration)
   cudaGraphExec_t lexec = nullptr;
   int l_kind = -1, l_nn_mode = -1, l_tile_gen = -1;
-  const nn_handle* l_nn = nullptr;
+  uint64_t l_nn = 0;
   int64_t l_launches = 0;  // kernel launches per loop iteration
   // the DF outer iteration (pcg_opts.outer_prec = EB_DF64) for the current
   // solve: x, r, p, q hold double-float pairs (x in xdf), z FP32; diag_df is
@@ -362,7 +363,10 @@ void amg_fill_info(const Solver& S, amg_info_t* out);
 int amg_levels(const Solver& S);  // levels of the hierarchy (0 without one)
 void amg_copy_level(const Solver& S, int level, int which, int32_t* rowptr, int32_t* col, double* val, cudaStream_t s);
 
-// learned stage (cnn.cu): buffers for grids of eb's size (before any capture),
+// learned stage (cnn.cu): a number that no other handle has or had and that
+// changes with everything a captured stage depends on (0: no stage)
+uint64_t nn_stage_state(const nn_handle* nn);
+// buffers for grids of eb's size (before any capture),
 // then z <- z + omega h^2 rms(s) N(s / rms(s), m), s = r - (shift I + A) z
 void nn_stage_prepare(nn_handle* nn, const EBHandle& eb, cudaStream_t s);
 void nn_stage_apply(nn_handle* nn, const EBHandle& eb, double shift, int mode, const double* r, double* z,
