@@ -110,10 +110,11 @@ struct LeapfrogGraph {
 };
 
 // what a handle keeps for several leapfrog steps per launch (eb_wave.cu); done
-// is created with the rest and recorded after each use
+// is recorded at the end of each use, one that fails half way included
 struct WvTask;
 struct WavePlan {
   cudaEvent_t done = nullptr;
+  bool ready = false;    // the rest is there, the task list written before done
   float* buf = nullptr;  // second pair of fields
   WvTask* task = nullptr;  // strips x chunks of rows that hold a CP
   int* ntask = nullptr;

@@ -362,7 +362,15 @@ bool launch_leapfrog_blocked(const EBHandle& eb, float* ua, float* ub, int nstep
   WavePlan& W = *eb.wave;
   const int rows = wave_rows(eb.num_cp);
   const int strips = (G.n0 + WV_CORE - 1) / WV_CORE, chunks = (G.n1 + rows - 1) / rows;
-  if (!W.done) {
+  if (!W.done) EB_CUDA(cudaEventCreateWithFlags(&W.done, cudaEventDisableTiming));
+  EB_CUDA(cudaStreamWaitEvent(s, W.done, 0));
+  // marks what has been enqueued below, also when a later launch fails
+  struct Mark {
+    cudaEvent_t e;
+    cudaStream_t s;
+    ~Mark() { cudaEventRecord(e, s); }
+  } mark{W.done, s};
+  if (!W.ready) {
     try {
       if (!W.buf) W.buf = dalloc<float>(2 * (size_t)G.num_nodes, s, false);
       if (!W.task) W.task = dalloc<WvTask>(2 * (size_t)strips * chunks, s, false);
@@ -375,9 +383,7 @@ bool launch_leapfrog_blocked(const EBHandle& eb, float* ua, float* ub, int nstep
     k_wave_tasks<<<blocks_for((int64_t)strips * chunks * 32, 256), 256, 0, s>>>(G.n0, G.n1, eb.code, rows, strips,
                                                                                 chunks, W.task, W.ntask);
     EB_CUDA(cudaGetLastError());
-    EB_CUDA(cudaEventCreateWithFlags(&W.done, cudaEventDisableTiming));
-  } else {
-    EB_CUDA(cudaStreamWaitEvent(s, W.done, 0));
+    W.ready = true;
   }
   float *b0 = W.buf, *b1 = W.buf + G.num_nodes;
   WvArgs a{};
@@ -416,7 +422,6 @@ bool launch_leapfrog_blocked(const EBHandle& eb, float* ua, float* ub, int nstep
     a.prev = op;
   }
   EB_CUDA(cudaGetLastError());
-  EB_CUDA(cudaEventRecord(W.done, s));
   return true;
 }
 
