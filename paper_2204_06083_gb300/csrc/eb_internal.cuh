@@ -109,16 +109,8 @@ struct LeapfrogGraph {
   void release();
 };
 
-// what a handle keeps for several leapfrog steps per launch (eb_wave.cu); done
-// is recorded at the end of each use, one that fails half way included
-struct WvTask;
-struct WavePlan {
-  cudaEvent_t done = nullptr;
-  bool ready = false;    // the rest is there, the task list written before done
-  float* buf = nullptr;  // second pair of fields
-  WvTask* task = nullptr;  // strips x chunks of rows that hold a CP
-  int* ntask = nullptr;
-};
+// what a handle keeps for several leapfrog steps per launch (eb_wave.cu)
+struct WavePlan;
 
 struct EBHandle {
   Geometry g;
@@ -308,7 +300,7 @@ int launch_leapfrog(const EBHandle& eb, T* ua, T* ub, int nsteps, double dt, cud
 // nsteps >= 2 FP32 leapfrog steps of a 2D grid with beta = 1 and the
 // line-by-line closure, several per launch (eb_wave.cu); the fields hold 0 off
 // the CPs of the active tiles.  false: not done (the second pair of fields could
-// not be allocated), nothing was launched
+// not be allocated or is in use), nothing was launched on the fields
 bool launch_leapfrog_blocked(const EBHandle& eb, float* ua, float* ub, int nsteps, float c2, cudaStream_t s);
 void wave_plan_free(WavePlan*& W, cudaStream_t s);
 }

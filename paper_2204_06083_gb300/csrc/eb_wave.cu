@@ -312,12 +312,25 @@ __global__ void __launch_bounds__(256) k_wave_tasks(int n0, int n1, const uint8_
   }
 }
 
-// Calls on different streams take turns with a handle's second pair of fields:
-// each waits for the event of the one before.  One mutex for all handles, held
-// while launches are enqueued.
-static std::mutex& wave_mutex() {
-  static std::mutex m;
-  return m;
+// A handle has one second pair of fields.  A call that finds it in use -- by a
+// run still in flight on another stream, or by a call that another thread is
+// enqueuing -- takes the in-place steps instead, which need none, so that calls
+// of one handle on several streams overlap.
+struct WavePlan {
+  std::mutex mu;                 // held while a call enqueues
+  cudaEvent_t done = nullptr;    // recorded at the end of each use, one that fails half way included
+  cudaStream_t stream = nullptr; // of the last use
+  bool ready = false;            // the rest is there, the task list written before done
+  float* buf = nullptr;          // second pair of fields
+  WvTask* task = nullptr;        // strips x chunks of rows that hold a CP
+  int* ntask = nullptr;
+};
+
+static WavePlan& wave_plan(const EBHandle& eb) {
+  static std::mutex m;  // of the creation of plans
+  std::lock_guard<std::mutex> lock(m);
+  if (!eb.wave) eb.wave = new WavePlan();
+  return *eb.wave;
 }
 
 void wave_plan_free(WavePlan*& W, cudaStream_t s) {
@@ -357,13 +370,25 @@ static int wave_rows(int64_t num_cp) {
 bool launch_leapfrog_blocked(const EBHandle& eb, float* ua, float* ub, int nsteps, float c2, cudaStream_t s) {
   const Geometry& G = eb.g;
   if (G.n0 >= WV_MAXX) return false;
-  std::lock_guard<std::mutex> lock(wave_mutex());
-  if (!eb.wave) eb.wave = new WavePlan();
-  WavePlan& W = *eb.wave;
+  WavePlan& W = wave_plan(eb);
+  std::unique_lock<std::mutex> lock(W.mu, std::try_to_lock);
+  if (!lock) return false;
+  if (W.done && W.stream != s) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // a query may meet another stream's capture
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const cudaError_t e = cudaEventQuery(W.done);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e == cudaErrorNotReady) {
+      cudaGetLastError();
+      return false;
+    }
+    EB_CUDA(e);
+  }
   const int rows = wave_rows(eb.num_cp);
   const int strips = (G.n0 + WV_CORE - 1) / WV_CORE, chunks = (G.n1 + rows - 1) / rows;
   if (!W.done) EB_CUDA(cudaEventCreateWithFlags(&W.done, cudaEventDisableTiming));
   EB_CUDA(cudaStreamWaitEvent(s, W.done, 0));
+  W.stream = s;
   // marks what has been enqueued below, also when a later launch fails
   struct Mark {
     cudaEvent_t e;
