@@ -383,11 +383,12 @@ __global__ void __launch_bounds__(TILE_NODES) k_g_cheb_step(TileView tv, const u
   }
 }
 
-// The batched DF iteration's x/r update (k_b_update_xr_df of the PCG: x += alpha
-// p, r -= alpha q in DF, per-tile DF partials r.r and r.zold as pairs, tiles of
-// converged geometries skipped) with the V-cycle's first level-0 step on the
-// new r's FP32 high part while it is in registers: saves a pass over r (64
-// stars: 65 + 27 us as two launches)
+// The batched DF iteration's x/r update (x += alpha p, r -= alpha q in DF,
+// per-tile DF partials r.r and r.zold as pairs) with the V-cycle's first level-0
+// step on the new r's FP32 high part while it is in registers: saves a pass
+// over r (64 stars: 65 + 27 us as two launches).  The rest of the cycle runs on
+// every tile; those of converged geometries are 0 in it, so that it neither
+// smooths their last iterate further nor carries them into the coarse levels.
 template <class V>
 __global__ void __launch_bounds__(PAIR_THREADS) k_b_update_first_df(TileView tv, BatchUpdate u,
                                                                     const uint8_t* __restrict__ code,
@@ -400,12 +401,19 @@ __global__ void __launch_bounds__(PAIR_THREADS) k_b_update_first_df(TileView tv,
   double* const x = u.sc->x;
   for (int64_t tt = blockIdx.x; tt < tv.ntiles; tt += gridDim.x) {
     const PcgScalars& S = u.sc[u.tile_geo[tt]];
-    if (S.done) continue;
+    int32_t node;
+    if (S.done) {
+      if (tile_pair<2>(tv, tt, threadIdx.x, node)) {
+        st2o(b_out + node, 0.0f, 0.0f);
+        st2o(x0 + node, 0.0f, 0.0f);
+        st2o(d + node, 0.0f, 0.0f);
+      }
+      continue;
+    }
     __syncthreads();  // s_a of the previous tile is read
     if (threadIdx.x == 0) s_a = df_from_double(S.alpha);
     __syncthreads();
     const DF a = s_a;
-    int32_t node;
     DF srr{0.0f, 0.0f}, srzo{0.0f, 0.0f};
     if (tile_pair<2>(tv, tt, threadIdx.x, node)) {
       DF r0, r1, q0, q1, p0, p1, xa, xb;
