@@ -49,18 +49,6 @@ __device__ __forceinline__ A inv_diag_t(uint32_t c, const DT* __restrict__ diag,
   return (A)1 / (o.sigma + (A)__ldg(diag + node) * o.inv_h2);
 }
 
-// division by a constant whose correctly rounded reciprocal is known: FP64 by
-// Markstein's correction of the product (IBM J. Res. Dev. 34, 1990), which
-// gives the rounded quotient in three operations; FP32 by the product
-struct DivBy {
-  double d, inv;
-};
-__device__ __forceinline__ double div_by(double a, const DivBy& c) {
-  const double q = a * c.inv;
-  return fma(fma(-q, c.d, a), c.inv, q);
-}
-__device__ __forceinline__ float div_by(float a, const DivBy& c) { return a * (float)c.inv; }
-
 // the values of GOp<double>::dinv
 __global__ void __launch_bounds__(TILE_NODES) k_cut_dinv(PairList pl, const uint8_t* __restrict__ code,
                                                          const double* __restrict__ diag, double sigma, double inv_h2,
@@ -141,7 +129,7 @@ __global__ void __launch_bounds__(TILE_NODES) k_g_cheb_first(TileView tv, const 
                                                              GOp<typename AccOf<V>::type> o,
                                                              const double* __restrict__ r, V* __restrict__ b_out,
                                                              V* __restrict__ x, V* __restrict__ d,
-                                                             DivBy theta) {
+                                                             DivBy<typename AccOf<V>::type> theta) {
   using A = typename AccOf<V>::type;
   EB_SWEEP(DIM, tv, node) {
     const GOp<A> ot = sweep_op<DIM>(tv, tt_, o);
@@ -178,7 +166,7 @@ __global__ void __launch_bounds__(TILE_NODES) k_update_first(PairList pl, PcgUpd
                                                              const typename DiagOf<V>::type* __restrict__ diag,
                                                              GOp<typename AccOf<V>::type> o, V* __restrict__ b_out,
                                                              V* __restrict__ x0, V* __restrict__ d,
-                                                             DivBy theta) {
+                                                             DivBy<typename AccOf<V>::type> theta) {
   using A = typename AccOf<V>::type;
   __shared__ double sm[TILE_NODES];
   double* const x = u.sc->x;
@@ -395,7 +383,7 @@ __global__ void __launch_bounds__(PAIR_THREADS) k_b_update_first_df(TileView tv,
                                                                     const typename DiagOf<V>::type* __restrict__ diag,
                                                                     GOp<float> o, V* __restrict__ b_out,
                                                                     V* __restrict__ x0, V* __restrict__ d,
-                                                                    float inv_theta) {
+                                                                    DivBy<float> theta) {
   __shared__ DF dsm[PAIR_THREADS / 32];
   __shared__ DF s_a;
   double* const x = u.sc->x;
@@ -435,8 +423,8 @@ __global__ void __launch_bounds__(PAIR_THREADS) k_b_update_first_df(TileView tv,
       const GOp<float> ot = tile_op(tv, tt, o);
       const float b0 = (c0 & CODE_CP) ? r0.hi : 0.0f, b1 = (c1 & CODE_CP) ? r1.hi : 0.0f;
       st2o(b_out + node, b0, b1);
-      const float v0 = (c0 & CODE_CP) ? inv_diag_t<float>(c0, diag, node, ot) * b0 * inv_theta : 0.0f;
-      const float v1 = (c1 & CODE_CP) ? inv_diag_t<float>(c1, diag, node + 1, ot) * b1 * inv_theta : 0.0f;
+      const float v0 = (c0 & CODE_CP) ? div_by(inv_diag_t<float>(c0, diag, node, ot) * b0, theta) : 0.0f;
+      const float v1 = (c1 & CODE_CP) ? div_by(inv_diag_t<float>(c1, diag, node + 1, ot) * b1, theta) : 0.0f;
       st2o(x0 + node, v0, v1);
       st2o(d + node, v0, v1);
     }
@@ -724,7 +712,7 @@ struct CoarseFirst {
   const V* dinv = nullptr;
   V* x = nullptr;
   V* d = nullptr;
-  DivBy theta{1.0, 1.0};
+  DivBy<typename AccOf<V>::type> theta{1, 1};
 };
 
 template <class V>
@@ -1187,8 +1175,7 @@ static CoarseFirst<V> coarse_first(Solver& S, size_t l) {
   f.dinv = LV::dinv(L);
   f.x = v.x;
   f.d = v.d;
-  const double theta = cheb_coef(L.rho, S.opts.cheb_degree).theta;
-  f.theta = DivBy{theta, 1.0 / theta};
+  f.theta = DivBy<typename AccOf<V>::type>::of(cheb_coef(L.rho, S.opts.cheb_degree).theta);
   return f;
 }
 
@@ -1353,9 +1340,9 @@ static int vcycle_grid(Solver& S, const double* r, double* z, cudaStream_t s, co
   if (first_done)
     S.nlaunch -= 1;  // amg_update_first did it
   else if (rdf)
-    k_g_cheb_first<DIM, V, true><<<gl, th, 0, s>>>(tv, eb.code, diag, o, r, bcopy, x, g.d, DivBy{cc.theta, 1.0 / cc.theta});
+    k_g_cheb_first<DIM, V, true><<<gl, th, 0, s>>>(tv, eb.code, diag, o, r, bcopy, x, g.d, DivBy<A>::of(cc.theta));
   else
-    k_g_cheb_first<DIM, V><<<gl, th, 0, s>>>(tv, eb.code, diag, o, r, bcopy, x, g.d, DivBy{cc.theta, 1.0 / cc.theta});
+    k_g_cheb_first<DIM, V><<<gl, th, 0, s>>>(tv, eb.code, diag, o, r, bcopy, x, g.d, DivBy<A>::of(cc.theta));
   // the tensor-copy step (batched 2D views, FP32 storage) or the sweep kernel
   auto step = [&](const V* xin, V* xout, int k) {
     if constexpr (std::is_same<V, float>::value && (DIM & (DIM_VB | DIM_LIST)) == 0 && dim_of(DIM) == 2) {
@@ -1473,7 +1460,7 @@ static void update_first(Solver& S, const PcgUpdate& u, cudaStream_t s) {
     }
   }
   k_update_first<DIM, V><<<(unsigned)u.nblk, S.iter_threads(), 0, s>>>(eb.pairs(), u, eb.code, diag_of<V>(eb), o, bcopy,
-                                                                 g.x, g.d, DivBy{cc.theta, 1.0 / cc.theta});
+                                                                 g.x, g.d, DivBy<A>::of(cc.theta));
 }
 
 template <class V>
@@ -1482,7 +1469,7 @@ static void batch_update_first(Solver& S, const BatchUpdate& u, unsigned grid, c
   const ChebCoef cc = cheb_coef(S.H->L[0].rho, S.opts.cheb_degree);
   VecSet<V>& g = LevelView<V>::grid(*S.H);
   k_b_update_first_df<V><<<grid, PAIR_THREADS, 0, s>>>(eb.tv(), u, eb.code, diag_of<V>(eb), grid_op<float>(S), g.b, g.x,
-                                                       g.d, (float)(1.0 / cc.theta));
+                                                       g.d, DivBy<float>::of(cc.theta));
 }
 
 void amg_batch_update_first(Solver& S, const BatchUpdate& u, unsigned grid, cudaStream_t s) {

@@ -36,9 +36,13 @@ constexpr int BT = PAIR_THREADS;  // one tile per CTA of 128 threads
 
 struct GeoConst {
   double h2, dt, theta;
-  double inv_dt, s, w;  // 1 / dt, h2 / theta, (1 - theta) / theta: no FP64 division per node
+  // no FP64 division per node: dt as a divisor (u / dt is 0 for dt = infinity,
+  // as 0 u / 1), h2 / theta, (1 - theta) / theta
+  DivBy<double> by_dt;
+  double s, w;
   static GeoConst make(double h2, double dt, double theta) {
-    return GeoConst{h2, dt, theta, 1.0 / dt, h2 / theta, (1.0 - theta) / theta};
+    return GeoConst{h2, dt, theta, std::isinf(dt) ? DivBy<double>{1.0, 0.0} : DivBy<double>::of(dt), h2 / theta,
+                    (1.0 - theta) / theta};
   }
 };
 
@@ -466,7 +470,7 @@ __global__ void __launch_bounds__(BT) k_b_heat_rhs(TileView tv, const int32_t* t
     stencil_pair<2, LdRO>(u, node, tv.nn, c0, c1, diag, tv.sy, tv.sz, uc, core);
     const Two<double> v1 = LdRO::ld2(b1 + node);
     const double s = c.s;
-    double r0 = s * (uc.x * c.inv_dt + c.theta * v1.x), r1 = s * (uc.y * c.inv_dt + c.theta * v1.y);
+    double r0 = s * (div_by(uc.x, c.by_dt) + c.theta * v1.x), r1 = s * (div_by(uc.y, c.by_dt) + c.theta * v1.y);
     if (c.theta < 1.0) {
       const Two<double> v0 = LdRO::ld2(b0 + node);
       const double w = c.w;

@@ -538,7 +538,8 @@ __global__ void __launch_bounds__(TILE_NODES) k_copy_tiles(TileView tv, const do
 // rhs of the theta-method: (u/dt - (1-theta) A u + theta b1 + (1-theta) b0) / theta
 template <int DIM>
 __global__ void __launch_bounds__(TILE_NODES) k_heat_rhs(TileView tv, const uint8_t* code, const double* diag,
-                                                         double inv_h2, double inv_dt, double theta, double inv_theta, const double* u,
+                                                         double inv_h2, DivBy<double> dt, double theta,
+                                                         DivBy<double> by_theta, const double* u,
                                                          const double* b1, const double* b0, double* out) {
   EB_PAIR_LOOP(DIM, tv, node) {
     uint32_t c0, c1;
@@ -546,12 +547,13 @@ __global__ void __launch_bounds__(TILE_NODES) k_heat_rhs(TileView tv, const uint
     Two<double> uc, core;
     stencil_tv<DIM, LdRO>(tv, u, node, c0, c1, diag, uc, core);
     const Two<double> b1v = LdRO::ld2(b1 + node), b0v = LdRO::ld2(b0 + node);
-    double v0 = uc.x * inv_dt + theta * b1v.x, v1 = uc.y * inv_dt + theta * b1v.y;
+    double v0 = div_by(uc.x, dt) + theta * b1v.x, v1 = div_by(uc.y, dt) + theta * b1v.y;
     if (theta < 1.0) {
       v0 += (1.0 - theta) * (b0v.x - core.x * inv_h2);
       v1 += (1.0 - theta) * (b0v.y - core.y * inv_h2);
     }
-    st2(out + node, (c0 & CODE_CP) ? v0 * inv_theta : 0.0, (c1 & CODE_CP) ? v1 * inv_theta : 0.0);
+    st2(out + node, (c0 & CODE_CP) ? div_by(v0, by_theta) : 0.0,
+        (c1 & CODE_CP) ? div_by(v1, by_theta) : 0.0);
   }
 }
 
@@ -892,8 +894,8 @@ int Solver::heat(double dt, double theta, const double* b1, const double* b0, do
   EB_REQUIRE(std::fabs(want - shift) <= 1e-12 * want, EB_ERR_INVALID,
              "heat: the hierarchy shift must equal 1/(theta dt)");
   const Geometry& G = eb->g;
-  EB_DIMV_LAUNCH(*eb, k_heat_rhs, nblk, eb->tv(), eb->code, eb->diag, 1.0 / (G.h * G.h), 1.0 / dt, theta, 1.0 / theta, u, b1,
-                b0 ? b0 : b1, tmp);
+  EB_DIMV_LAUNCH(*eb, k_heat_rhs, nblk, eb->tv(), eb->code, eb->diag, 1.0 / (G.h * G.h),
+                 DivBy<double>::of(dt), theta, DivBy<double>::of(theta), u, b1, b0 ? b0 : b1, tmp);
   EB_CUDA(cudaGetLastError());
   // the loop on the device (tmp and u keep their addresses); the solver's
   // default outer precision (amg_set_outer_prec) where it applies

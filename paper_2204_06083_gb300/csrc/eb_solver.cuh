@@ -4,6 +4,7 @@
 #include <utility>
 #include <vector>
 
+#include "divide.cuh"
 #include "eb_internal.cuh"
 
 namespace ebk {
