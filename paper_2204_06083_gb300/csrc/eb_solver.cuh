@@ -278,13 +278,22 @@ __device__ __forceinline__ bool pcg_alpha(PcgScalars* sc, const double* pq_part,
   return s_done == 0;
 }
 
+// 2^-600 <= |x| < 2^600, by the exponent bits
+__device__ __forceinline__ bool pcg_mid_range(double x) {
+  return (uint32_t)((__double2hiint(x) >> 20 & 0x7ff) - (1023 - 600)) < 1200u;
+}
+
 // The end of an iteration, thread 0's part: beta = (v - t) / rz from the summed
 // r'z (v) and, flexible, r'zold (t); with rec (one CTA of the launch) recorded
-// with the next r'z and a breakdown.  inv_rz: 1 / h.rz, formed ahead.
+// with the next r'z and a breakdown.  inv_rz: 1 / h.rz, formed ahead; the
+// quotient is that of a division (div_by), and one where the reciprocal or the
+// correction would leave FP64's normal range (r'z of a tiny right-hand side).
 __device__ __forceinline__ double pcg_beta_from(PcgScalars* sc, const PcgHead& h, double inv_rz, double v, double t,
                                                 bool rec) {
   const bool ok = v > 0.0;
-  const double beta = ok ? (v - t) * inv_rz : 0.0;
+  const double num = v - t;
+  const bool mid = pcg_mid_range(h.rz) && pcg_mid_range(num);
+  const double beta = !ok ? 0.0 : mid ? div_by(num, DivBy<double>{h.rz, inv_rz}) : num / h.rz;
   if (rec) {
     sc->beta = beta;
     sc->rz[h.k ^ 1] = v;
