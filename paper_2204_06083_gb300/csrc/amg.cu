@@ -1117,7 +1117,7 @@ void amg_build_from(Solver& S, DCsr A0, cudaStream_t s) {
       }
       DCsr AP = spgemm(A, L.P, s);
       DCsr Ac = spgemm(L.R, AP, s);
-      L.AP = AP;
+      amg_take_ap(S, lev, L, AP, s);
       A = Ac;
       continue;
     }
@@ -1190,7 +1190,7 @@ void amg_build_from(Solver& S, DCsr A0, cudaStream_t s) {
     }
     DCsr AP = spgemm(A, L.P, s);
     DCsr Ac = spgemm(L.R, AP, s);
-    L.AP = AP;
+    amg_take_ap(S, lev, L, AP, s);
     A = Ac;
   }
   // coarsest level

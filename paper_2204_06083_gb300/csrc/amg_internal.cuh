@@ -81,6 +81,8 @@ struct Hierarchy {
 DCsr level0_csr(const EBHandle& eb, double sigma, cudaStream_t s);
 void amg_build_from(Solver& S, DCsr A0, cudaStream_t s);
 DCsr transpose(const DCsr& A, cudaStream_t s);
+// keeps level lev's A P for the merged transfers, or frees it where none uses it
+void amg_take_ap(const Solver& S, int lev, Level& L, DCsr& AP, cudaStream_t s);
 void amg_alloc_vcycle(Solver& S, cudaStream_t s);
 void amg_free_vcycle(Hierarchy& H, cudaStream_t s);
 

@@ -1543,13 +1543,25 @@ static void make_pair(PairCsr& M, DCsr& A, const DCsr& B, cudaStream_t s) {
 // 25 against 11.6 + 4.6).
 constexpr int64_t PAIR_NNZ = 2000000;
 constexpr int64_t PAIR_ROW = 128;
+static bool pairs_wanted(const Solver& S, size_t l, const Level& L) {
+  if (S.opts.vcycle_prec == EB_F64) return false;
+  return l > 0 || (L.A.nnz <= PAIR_NNZ && S.eb->pair_node && S.eb->g.dim == 2);
+}
+
+// an A P that no pair is made of is the largest matrix of a set-up, so it goes
+// with its product (256^3, FP64 or FP32: level 0's)
+void amg_take_ap(const Solver& S, int lev, Level& L, DCsr& AP, cudaStream_t s) {
+  if (pairs_wanted(S, (size_t)lev, L)) L.AP = AP;
+  else csr_free(AP, s);
+}
+
 template <class V>
 static void make_pairs(Solver& S, cudaStream_t s) {
   Hierarchy& H = *S.H;
   for (size_t l = 0; l + 1 < H.L.size(); ++l) {
     Level& L = H.L[l];
+    if (!pairs_wanted(S, l, L)) continue;
     const bool small = L.A.nnz <= PAIR_NNZ;
-    if (l == 0 && !(small && S.eb->pair_node && S.eb->g.dim == 2)) continue;
     if (l > 0 && small && L.AP.nnz <= PAIR_ROW * L.AP.m) {
       DCsr T = transpose(L.AP, s);
       make_pair<V>(L.T, T, L.R, s);
@@ -1610,7 +1622,6 @@ void amg_alloc_vcycle(Solver& S, cudaStream_t s) {
     }
     for (size_t l = first; l < H.L.size(); ++l) alloc_set(H.L[l].v64, H.L[l].A.n, true, s);
   }
-  for (Level& L : H.L) csr_free(L.AP, s);
   EB_CUDA(cudaGetLastError());
 }
 
