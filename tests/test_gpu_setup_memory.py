@@ -42,7 +42,7 @@ def test_products_are_not_kept(vprec):
     import __graft_entry__ as ge
     import paper_2204_06083_gb300 as eb
     ge.build()
-    grid, ls = ei.ellipsoid_k3(100)
+    grid, ls = ei.ellipsoid_k3(160)
     h = eb.EB(grid, ls)
     get, reset = _pool()
     torch.cuda.synchronize()
