@@ -448,11 +448,12 @@ int wave_theta_step(const amg_handle* amg, double dt, double theta, double* u_pr
  * data).  On entry (u_prev, u_cur) = (u^{n-1}, u^n); on exit they hold
  * (u^{n+nsteps-1}, u^{n+nsteps}).  One kernel launch per step; whole chunks of
  * 32 steps run as one launch of a CUDA graph that the handle caches for these
- * fields, prec, dt and tile list (built on first use, which allocates).  Two or
- * more EB_F32 steps on a 2D grid with beta = 1 and the line-by-line closure run
- * eight per launch, through a second pair of fields that the handle keeps from
- * the first such call on (2 x num_nodes floats); a call that finds that pair in
- * use on another stream takes one launch per step.  The results are the same.
+ * fields, prec, dt and tile list (built on first use, which allocates).  Calls of
+ * three or more EB_F32 steps on a 2D grid with beta = 1 and the line-by-line
+ * closure run up to eight per launch, through a second pair of fields (2 x
+ * num_nodes floats) that the handle keeps once such calls have come to 32 steps;
+ * a call that finds that pair in use on another stream takes one launch per
+ * step.  The results are the same.
  * prec: EB_F64 or EB_F32 element type of both fields.  Asynchronous on
  * stream; the fields must not be touched by other work until it completes. */
 int wave_step(const eb_handle* eb, int prec, double dt, void* u_prev_dev, void* u_cur_dev, int nsteps,

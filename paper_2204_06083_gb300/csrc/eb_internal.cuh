@@ -297,10 +297,11 @@ void run_tuner(int dim, const std::function<void(const TileDims&)>& retile, cons
                int reps, eb_tune_t* out, cudaStream_t s);
 template <class T>
 int launch_leapfrog(const EBHandle& eb, T* ua, T* ub, int nsteps, double dt, cudaStream_t s, bool use_graph);
-// nsteps >= 2 FP32 leapfrog steps of a 2D grid with beta = 1 and the
+// nsteps >= 3 FP32 leapfrog steps of a 2D grid with beta = 1 and the
 // line-by-line closure, several per launch (eb_wave.cu); the fields hold 0 off
 // the CPs of the active tiles.  false: not done (the second pair of fields could
-// not be allocated or is in use), nothing was launched on the fields
+// not be allocated or is in use, or the handle has taken too few steps for one),
+// nothing was launched on the fields
 bool launch_leapfrog_blocked(const EBHandle& eb, float* ua, float* ub, int nsteps, float c2, cudaStream_t s);
 void wave_plan_free(WavePlan*& W, cudaStream_t s);
 }

@@ -288,8 +288,11 @@ int launch_leapfrog(const EBHandle& eb, T* ua, T* ub, int nsteps, double dt, cud
     // which the FP64 pipe bounds (recomputed halos cost more than the launches
     // and passes they save: 90 against 47 us per step at 4096^2), nor for RBF
     // closures (D_k > 0 tells the CPs there), nor during stream capture (the
-    // plan allocates and waits for its last use on another stream).
-    if (use_graph && G.dim == 2 && !eb.has_beta() && eb.closure == EB_CLOSURE_LINE && nsteps >= 2 && tv.pair_node &&
+    // plan allocates).  Not for two steps either, which are two passes over
+    // both fields like two launches here: 12.4 against 16.4 us at 1302^2 and 28.7
+    // against 32.8 at 4096^2, where three steps take 20.5 against 16.7 and 47.7
+    // against 34.9.
+    if (use_graph && G.dim == 2 && !eb.has_beta() && eb.closure == EB_CLOSURE_LINE && nsteps >= 3 && tv.pair_node &&
         !is_capturing(s) && launch_leapfrog_blocked(eb, ua, ub, nsteps, c2, s))
       return EB_OK;
   }

@@ -47,6 +47,11 @@ constexpr int WV_ROWF = 2 * WV_COLS;       // floats of a ring row: u^n, u^{n-1}
 constexpr int WV_WARPF = WV_RING * WV_ROWF + WV_DRING * WV_COLS;
 constexpr int WV_SMEM = WV_THREADS / 32 * WV_WARPF * 4;
 constexpr int WV_MAXROWS = 64 - 3 * WV_MAXT;  // rows of a task: a bit of its mask each, with the halo rows
+// The plan is made by the call that brings a handle's steps to this many: it
+// takes 20 us and the allocation of the second pair of fields (4096^2: 180 us),
+// which a program of a few steps does not earn back.  First call of a handle,
+// 4096^2: 8 steps 260 us with the plan and 127 without, 64 steps 465 against 649
+constexpr int WV_FIRST_STEPS = 32;
 constexpr int WV_WARPS = 8;                // warps per SM that the tasks are cut for (12 fit)
 static_assert(WV_MAXT <= WV_HALO && WV_HALO % 4 == 0 && WV_DRING >= WV_AHEAD + WV_MAXT + 1, "strip");
 
@@ -320,6 +325,7 @@ struct WavePlan {
   std::mutex mu;                 // held while a call enqueues
   cudaEvent_t done = nullptr;    // recorded at the end of each use, one that fails half way included
   cudaStream_t stream = nullptr; // of the last use
+  int64_t steps = 0;             // taken while the rest is not there
   bool ready = false;            // the rest is there, the task list written before done
   float* buf = nullptr;          // second pair of fields
   WvTask* task = nullptr;        // strips x chunks of rows that hold a CP
@@ -373,6 +379,7 @@ bool launch_leapfrog_blocked(const EBHandle& eb, float* ua, float* ub, int nstep
   WavePlan& W = wave_plan(eb);
   std::unique_lock<std::mutex> lock(W.mu, std::try_to_lock);
   if (!lock) return false;
+  if (!W.ready && (W.steps += nsteps) < WV_FIRST_STEPS) return false;
   if (W.done && W.stream != s) {
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // a query may meet another stream's capture
     cudaThreadExchangeStreamCaptureMode(&mode);
