@@ -1041,7 +1041,8 @@ def stencil_subrecords(ctx, args, h3):
     grid, ls = ei.star_wave(4096)
     hw = eb.EB(grid, ls)
     ncw = hw.info.num_cp
-    tile, _ = tune_tiles(lambda: autotune.tune_eb(hw, eb.EB_F32, reps=5, op=eb.EB_TUNE_LEAPFROG))
+    # in FP64: the FP32 steps run several per launch and do not walk the tiles
+    tile, _ = tune_tiles(lambda: autotune.tune_eb(hw, eb.EB_F64, reps=5, op=eb.EB_TUNE_LEAPFROG))
     X, Y = ei.grid_points(grid)
     c, w = ei.pulse_params(0)
     dt = 0.9 * grid.h / math.sqrt(2.0)
@@ -1084,7 +1085,8 @@ def gpu_wave(ctx, args):
     grid, ls = ei.star_wave(4096)
     h = eb.EB(grid, ls)
     nc = h.info.num_cp
-    tile, tune = tune_tiles(lambda: autotune.tune_eb(h, eb.EB_F32, reps=5, op=eb.EB_TUNE_LEAPFROG))
+    # in FP64: the FP32 steps run several per launch and do not walk the tiles
+    tile, tune = tune_tiles(lambda: autotune.tune_eb(h, eb.EB_F64, reps=5, op=eb.EB_TUNE_LEAPFROG))
     X, Y = ei.grid_points(grid)
     c, w = ei.pulse_params(0)
     dt = 0.9 * grid.h / math.sqrt(2.0)

@@ -238,8 +238,10 @@ typedef enum { EB_TUNE_APPLY = 0, EB_TUNE_LEAPFROG = 1 } eb_tune_op;
 /* Autotuner: for each candidate shape, times `reps` calls of the operation
  * (EB_TUNE_APPLY: one eb_apply launch; EB_TUNE_LEAPFROG: one wave_step of 16
  * steps) in precision prec (EB_F64, EB_F32; EB_BF16 for apply) with CUDA
- * events on stream, and keeps the fastest shape.  out (may be NULL) receives
- * the timings.  Synchronous. */
+ * events on stream, and keeps the fastest shape.  EB_F32 steps that run several
+ * per launch (wave_step) walk rows, not tiles, and hardly depend on the shape:
+ * tune in EB_F64 where both are run.  out (may be NULL) receives the timings.
+ * Synchronous. */
 int eb_autotune(eb_handle* eb, int op, int prec, int reps, eb_tune_t* out, cudaStream_t stream);
 
 /* ---------------------------------------------------------------- AMG + PCG */
