@@ -1233,8 +1233,13 @@ int batch_set_level0_tma(batch_handle* b, int on) {
     set_error("batch_set_level0_tma: NULL handle");
     return EB_ERR_INVALID;
   }
-  b->b.l0_tma = on != 0;
-  if (b->b.S) b->b.S->l0_tma = b->b.l0_tma;
+  Batch& B = b->b;
+  if (B.l0_tma == (on != 0)) return EB_OK;
+  B.l0_tma = on != 0;
+  if (B.S) B.S->l0_tma = B.l0_tma;
+  if (B.gexec) cudaGraphExecDestroy(B.gexec);  // captured iterations hold the old route
+  B.gexec = nullptr;
+  b_loop_release(B);
   return EB_OK;
 }
 
