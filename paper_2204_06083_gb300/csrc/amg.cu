@@ -1128,13 +1128,13 @@ void amg_build_from(Solver& S, DCsr A0, cudaStream_t s) {
     EB_CUDA(cudaMemsetAsync(state, 1, A.n, s));
     uint64_t* k1 = dalloc<uint64_t>(A.n, s, false);
     int* und = dalloc<int>(1, s);
-    // rounds until every node is decided (further rounds change nothing); on
-    // small levels, where a round costs less than reading the count back, four
-    // between two looks at it
-    const int batch = A.n < 300000 ? 4 : 1;
+    // rounds until every node is decided (further rounds change nothing), four
+    // between two looks at the count of undecided nodes: a set-up of 51 K rows
+    // takes 2.25 ms against 2.45 with a look at every round, of 348 K rows 4.63
+    // against 4.83, of 1.78 M rows 15.9 against 16.3
     for (int round = 0;;) {
-      for (int k = 0; k < batch; ++k, ++round) {
-        if (k + 1 == batch) EB_CUDA(cudaMemsetAsync(und, 0, sizeof(int), s));
+      for (int k = 0; k < 4; ++k, ++round) {
+        if (k == 3) EB_CUDA(cudaMemsetAsync(und, 0, sizeof(int), s));
         k_mis_max1<<<blocks_for(A.n, 256), 256, 0, s>>>(A, strong, state, k1);
         k_mis_max2<<<blocks_for(A.n, 256), 256, 0, s>>>(A, strong, k1, state, und);
       }
