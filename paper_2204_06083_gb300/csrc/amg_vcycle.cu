@@ -315,9 +315,8 @@ __global__ void __launch_bounds__(TILE_NODES) k_update_first_df(PairList pl, Pcg
 }
 
 // res = D^-1 (b - A x); d = c1 d + c2 res; xo = x + d   (xo may be FP64).
-// DOT = 1 (xo FP64, the V-cycle's output z): also the CTA's partial r.z,
-// summed over its node pairs in loop order exactly as the PCG's own dot kernel
-// does; DOT = 2 (xo FP32, r a double-float vector): the same partial summed
+// DOT = 1 (xo FP64, the V-cycle's output z): also the CTA's partial r.z, each
+// thread's node pairs in loop order, then block_sum; DOT = 2 (xo FP32, r a double-float vector): the same partial summed
 // and stored in DF.
 template <int DIM, class V, class O, int DOT = 0>
 __global__ void __launch_bounds__(TILE_NODES) k_g_cheb_step(TileView tv, const uint8_t* __restrict__ code,
@@ -1540,7 +1539,15 @@ static void make_pair(PairCsr& M, DCsr& A, const DCsr& B, cudaStream_t s) {
 // against 4.1 + 2.8 us; 256^3, whose A P has three times the entries per row:
 // 67 against 18.3 + 7.8), k_c_resid_restrict with short rows of (A P)^T, a warp
 // or less each (1022^2: 2.9 against 2.3 + 2.1 us; 256^3, 700 entries per row:
-// 25 against 11.6 + 4.6).
+// 25 against 11.6 + 4.6).  FP32 V-cycle of 2D stars with the two on no, these
+// and all levels: 76.1, 66.3, 66.9 us at 1022^2 (1.0 M entries of level 0), 85.2,
+// 77.4, 78.6 at 1330^2 (1.7 M), 90.2, 84.2, 80.3 at 1430^2 (2.0 M: just above
+// PAIR_NNZ), 97.0, 91.4, 93.1 at 1600^2 (2.5 M), 110.7, 105.0, 120.0 at 2000^2
+// (3.9 M); in 3D 56.5 each at 100^3, 77.0, 77.0, 77.9 at 160^3 (1.9 M), 120.6,
+// 120.7, 127.7 at 200^3.  BF16 cycles behave alike; their error against the FP64
+// cycle is in the median 0.74 of that with the separate launches (0.02 to 1.19
+// over 23 hierarchies and three right-hand sides; FP32: 0.93, 0.05 to 1.17), that
+// of W-cycles about a tenth.
 constexpr int64_t PAIR_NNZ = 2000000;
 constexpr int64_t PAIR_ROW = 128;
 static bool pairs_wanted(const Solver& S, size_t l, const Level& L) {
