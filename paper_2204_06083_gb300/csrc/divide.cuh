@@ -24,7 +24,9 @@ namespace ebk {
 template <class A>
 struct DivBy {
   A d, inv;
-  static DivBy of(double d) { return DivBy{(A)d, (A)1 / (A)d}; }
+  // an infinite divisor (a steady problem's time step) gives 0, as 0 a / 1: its
+  // own remainder a - 0 d is not a number
+  static DivBy of(double d) { return std::isinf((A)d) ? DivBy{1, 0} : DivBy{(A)d, (A)1 / (A)d}; }
 };
 
 // on the integer pipe: an FP64 comparison costs what an FP64 addition does

@@ -36,13 +36,11 @@ constexpr int BT = PAIR_THREADS;  // one tile per CTA of 128 threads
 
 struct GeoConst {
   double h2, dt, theta;
-  // no FP64 division per node: dt as a divisor (u / dt is 0 for dt = infinity,
-  // as 0 u / 1), h2 / theta, (1 - theta) / theta
+  // no FP64 division per node: dt as a divisor, h2 / theta, (1 - theta) / theta
   DivBy<double> by_dt;
   double s, w;
   static GeoConst make(double h2, double dt, double theta) {
-    return GeoConst{h2, dt, theta, std::isinf(dt) ? DivBy<double>{1.0, 0.0} : DivBy<double>::of(dt), h2 / theta,
-                    (1.0 - theta) / theta};
+    return GeoConst{h2, dt, theta, DivBy<double>::of(dt), h2 / theta, (1.0 - theta) / theta};
   }
 };
 
