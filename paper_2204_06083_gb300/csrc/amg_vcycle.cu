@@ -316,8 +316,8 @@ __global__ void __launch_bounds__(TILE_NODES) k_update_first_df(PairList pl, Pcg
 
 // res = D^-1 (b - A x); d = c1 d + c2 res; xo = x + d   (xo may be FP64).
 // DOT = 1 (xo FP64, the V-cycle's output z): also the CTA's partial r.z, each
-// thread's node pairs in loop order, then block_sum; DOT = 2 (xo FP32, r a double-float vector): the same partial summed
-// and stored in DF.
+// thread's node pairs in loop order, then block_sum; DOT = 2 (xo FP32, r a
+// double-float vector): the same partial summed and stored in DF.
 template <int DIM, class V, class O, int DOT = 0>
 __global__ void __launch_bounds__(TILE_NODES) k_g_cheb_step(TileView tv, const uint8_t* __restrict__ code,
                                                             const typename DiagOf<V>::type* __restrict__ diag,
