@@ -1322,7 +1322,8 @@ static int vcycle_grid(Solver& S, const double* r, double* z, cudaStream_t s, co
   const unsigned gl = LIST ? blocks_for(eb.num_pairs, th) : gb;
   // the launch that forms the r'z partials: DF sums are cheap to repeat, and
   // that step runs faster on eight CTAs per SM (256^3: 10.3 against 12.5 us)
-  const unsigned gd = LIST ? (unsigned)list_blocks(eb, dot && dot->df ? 8 : 4) : gb;
+  const int td = LIST && dot && dot->df ? list_threads_df(eb.num_pairs) : th;
+  const unsigned gd = LIST ? (unsigned)list_blocks(eb.num_pairs, td, dot && dot->df ? 8 : 4) : gb;
   const ChebCoef cc = cheb_coef(L0.rho, S.opts.cheb_degree);
   const TileView tv = eb.tv();
   using A = typename AccOf<V>::type;
@@ -1394,7 +1395,7 @@ static int vcycle_grid(Solver& S, const double* r, double* z, cudaStream_t s, co
     const bool mark = !(k == cc.deg - 1 && dot);
     if (mark) S.prof_mark(s, true);
     if (k == cc.deg - 1 && rdf && dot->part)  // z in FP32 for the DF outer iteration, with the r'z partials
-      k_g_cheb_step<DIM, V, float, 2><<<gd, th, 0, s>>>(tv, eb.code, diag, o, b, x,
+      k_g_cheb_step<DIM, V, float, 2><<<gd, td, 0, s>>>(tv, eb.code, diag, o, b, x,
                                                                 reinterpret_cast<float*>(z), g.d, (A)cc.c1[k],
                                                                 (A)cc.c2[k], dot->r, dot->part);
     else if (k == cc.deg - 1 && rdf && dot->tile_part) {  // batched: with the per-tile r'z partials
@@ -1624,7 +1625,7 @@ void amg_alloc_vcycle(Solver& S, cudaStream_t s) {
     const EBHandle& eb = *S.eb;
     if (eb.pair_node && H.L.size() > 1) {
       H.cut_dinv = dalloc<double>(nn, s, false);
-      k_cut_dinv<<<list_blocks(eb), list_threads(eb.num_pairs), 0, s>>>(eb.pairs(), eb.code, eb.diag, S.shift,
+      k_cut_dinv<<<list_blocks(eb.num_pairs, list_threads(eb.num_pairs)), list_threads(eb.num_pairs), 0, s>>>(eb.pairs(), eb.code, eb.diag, S.shift,
                                                                         1.0 / (eb.g.h * eb.g.h), H.cut_dinv);
     }
     for (size_t l = first; l < H.L.size(); ++l) alloc_set(H.L[l].v64, H.L[l].A.n, true, s);

@@ -263,11 +263,17 @@ inline unsigned blocks_for(int64_t n, int threads);
 // work spreads over every SM's schedulers (128^2: 1,500 pairs are 24 CTAs of 64
 // threads, not 6 of 256; one FP64 Chebyshev step 4.4 -> 2.4 us)
 inline int list_threads(int64_t pairs) { return pairs < (int64_t)num_sms() * 256 ? 64 : 256; }
-// CTAs of the list kernels that form reduction partials: at most four per SM
-// (every CTA of the next launch sums the partials again)
-inline int list_blocks(const EBHandle& eb, int per_sm = 4) {
-  const int t = list_threads(eb.num_pairs);
-  return (int)std::max<int64_t>(1, std::min<int64_t>((eb.num_pairs + t - 1) / t, (int64_t)num_sms() * per_sm));
+// The same for the kernels of the double-float iteration, whose work is FP32 but
+// whose CTAs each sum all partials in a chain of some twenty operations per
+// partial: small CTAs, with as many partials as CTAs, only up to 64 pairs per SM.
+// FP32 V-cycle, double-float solves with 64 and 256 threads: 801 and 853 us at
+// 48^3 (19 pairs per SM), 1045 and 1075 at 64^3 (51), 1120 and 1092 at 72^3 (74),
+// 1338 and 1150 at 100^3 (210), 1407 and 1201 on a 580^2 star (215)
+inline int list_threads_df(int64_t pairs) { return pairs < (int64_t)num_sms() * 64 ? 64 : 256; }
+// CTAs of t threads of the list kernels that form reduction partials: at most
+// four per SM (every CTA of the next launch sums the partials again)
+inline int list_blocks(int64_t pairs, int t, int per_sm = 4) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>((pairs + t - 1) / t, (int64_t)num_sms() * per_sm));
 }
 
 inline unsigned blocks_for(int64_t n, int threads) {

@@ -61,7 +61,7 @@ struct Solver {
   // reduction partials: [p'q | r'r] regions of 2 npart each, then the r'z region
   // (nblk partials from the PCG's own dot kernel, one per CTA of the V-cycle's
   // last smoothing launch), then the r'zold region of npart
-  int npart = 1;  // max(nblk, nblk_iter())
+  int npart = 1;  // max(nblk, nblk_iter() of the FP64 iteration, which has no fewer CTAs than the DF one)
   double* part = nullptr;
   double* part_pq() const { return part; }
   double* part_rr() const { return part + 2 * (int64_t)npart; }
@@ -71,8 +71,8 @@ struct Solver {
   // CTAs (= partials) of the iteration's x/r update and p update + apply
   // (a full grid leaves room for the CTA of the loop test, so that all are
   // resident at once)
-  int nblk_iter() const { return std::min(list_blocks(*eb), 4 * num_sms() - 1); }
-  int iter_threads() const { return list_threads(eb->num_pairs); }
+  int nblk_iter() const { return std::min(list_blocks(eb->num_pairs, iter_threads()), 4 * num_sms() - 1); }
+  int iter_threads() const { return df_on ? list_threads_df(eb->num_pairs) : list_threads(eb->num_pairs); }
   int64_t rz_cap = 0;
   int nblk = 1;
   int rz_n = 1;  // r'z partials written by the last precondition()
