@@ -1625,8 +1625,9 @@ void amg_alloc_vcycle(Solver& S, cudaStream_t s) {
     const EBHandle& eb = *S.eb;
     if (eb.pair_node && H.L.size() > 1) {
       H.cut_dinv = dalloc<double>(nn, s, false);
-      k_cut_dinv<<<list_blocks(eb.num_pairs, list_threads(eb.num_pairs)), list_threads(eb.num_pairs), 0, s>>>(eb.pairs(), eb.code, eb.diag, S.shift,
-                                                                        1.0 / (eb.g.h * eb.g.h), H.cut_dinv);
+      const int th = list_threads(eb.num_pairs);
+      k_cut_dinv<<<list_blocks(eb.num_pairs, th), th, 0, s>>>(eb.pairs(), eb.code, eb.diag, S.shift,
+                                                              1.0 / (eb.g.h * eb.g.h), H.cut_dinv);
     }
     for (size_t l = first; l < H.L.size(); ++l) alloc_set(H.L[l].v64, H.L[l].A.n, true, s);
   }
